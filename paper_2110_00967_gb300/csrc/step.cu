@@ -475,13 +475,10 @@ __device__ void tail(const StepArgs &p, const ForceRegion &reg) {
 // node update
 // ---------------------------------------------------------------------------
 
-// Coefficients 3 w_a of the odd (momentum-carrying) part of the equilibrium
-// and of the forcing term, for the axis directions (k1 = 3 w_1 = 1/3) and the
-// diagonals (k2 = 3 w_5 = 1/12).  In the compute type they are chosen with
-// 2 k1 + 4 k2 = 1 exactly, so that the odd equilibrium carries exactly the
-// node's momentum: with the rounded weights 1/9 and 1/36 of FP32 (both
-// 7.45e-9 too large) every collision would add 7.45e-9 s- of the momentum
-// offset, a bias that compounds step after step.
+// Coefficients 3 w_a of the odd part of the forcing term, for the axis
+// directions (k1 = 3 w_1 = 1/3) and the diagonals (k2 = 3 w_5 = 1/12), in the
+// compute type with 2 k1 + 4 k2 = 1 exactly, so that the forcing adds exactly
+// its momentum.
 template <typename T>
 struct OddW;
 template <>
@@ -499,62 +496,13 @@ __device__ __forceinline__ constexpr T odd_w(int a) {
   return a <= 4 ? OddW<T>::k1 : OddW<T>::k2;
 }
 
-// BGK/TRT collision with the forcing term (Eq. TRT) of one node, into o.
-// The equilibrium enters through its offset heq = feq(rho, u) - E, written
-// with the small quantities drho = rho - 1 and du = u - u_ref only:
-// heq_a = w_a [drho (1 + Q_a(u)) + Q_a(u) - Q_a(u_ref)],
-// Q_a(u) = 3 c.u + 4.5 (c.u)^2 - 1.5 |u|^2, split into its even and odd parts
-// for TRT.  kForce = false drops the forcing term (G = 0: a fluid node
-// without body force).  The rest population takes what the moving
-// populations' even parts give up, o_0 = h_0 - sum_{a>0} (even change of a):
-// equal to the relaxation of h_0 towards heq_0 (plus F_0) in exact
-// arithmetic, and conserving mass exactly up to the rounding of that sum,
-// where rounded weights would make the collision a mass source proportional
-// to rho - 1.
-template <typename T, bool kForce>
-__device__ __forceinline__ void collide(const T (&h)[9], T drho, T dux, T duy, T gx, T gy,
-                                        const Consts<T> &c, T (&o)[9]) {
-  const T ux = c.urx + dux, uy = c.ury + duy;
-  const T uu = ux * ux + uy * uy;
-  const T dsu = dux * (ux + c.urx) + duy * (uy + c.ury);  // |u|^2 - |u_ref|^2
-  const T ug = kForce ? ux * gx + uy * gy : (T)0;
-  T even = 0;  // sum over the pairs of the even change of one population
-#pragma unroll
-  for (int a = 1; a <= 6; ++a) {
-    if (a == 3 || a == 4) continue;
-    const int b = opp_of(a);
-    const T w = (T)w_of(a);
-    const T k = odd_w<T>(a);
-    const T cu = (T)cx_of(a) * ux + (T)cy_of(a) * uy;
-    const T cdu = (T)cx_of(a) * dux + (T)cy_of(a) * duy;
-    const T csu = cu + ((T)cx_of(a) * c.urx + (T)cy_of(a) * c.ury);
-    const T heqp = w * (drho * ((T)1 + (T)4.5 * cu * cu - (T)1.5 * uu) + (T)4.5 * cdu * csu -
-                        (T)1.5 * dsu);
-    const T heqm = k * (drho * cu + cdu);
-    const T hp = (T)0.5 * (h[a] + h[b]);
-    const T hm = (T)0.5 * (h[a] - h[b]);
-    T dp = -c.s_plus * (hp - heqp);
-    T dm = -c.s_minus * (hm - heqm);
-    if (kForce) {
-      const T cg = (T)cx_of(a) * gx + (T)cy_of(a) * gy;
-      dp += c.a_plus * (w * ((T)9 * cu * cg - (T)3 * ug));
-      dm += c.a_minus * (k * cg);
-    }
-    even += dp;
-    o[a] = h[a] + dp + dm;
-    o[b] = h[b] + dp - dm;
-  }
-  o[0] = h[0] - (T)2 * even;
-}
-
-// ---------------------------------------------------------------------------
-// FP32 arithmetic of the 16-bit forms' fluid-node update in the packed f32x2
-// instructions of sm_100 and later (one instruction for two nodes).  The
-// special kernel updates its 16-bit fluid nodes with the same instructions,
-// the node in both lanes: the compiler fuses some packed multiplies with a
-// following add (even when the PTX names a rounding mode), so only the same
-// instruction sequence gives a node the same bits in either kernel.
-// ---------------------------------------------------------------------------
+// The update is written over a value type V: double for FP64 lattices, and for
+// FP32 compute the packed f32x2 instructions of sm_100 and later (one
+// instruction for two nodes).  The special kernels update a single node with
+// the same packed instructions, the node in both lanes: the compiler fuses
+// some packed multiplies with a following add (even when the PTX names a
+// rounding mode), so only the same instruction sequence gives a node the same
+// bits in every kernel.
 struct F2 {
   float2 v;
 };
@@ -568,10 +516,6 @@ __device__ __forceinline__ F2 bits_f2(unsigned long long r) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(a.v.x), "=f"(a.v.y) : "l"(r));
   return a;
 }
-template <typename V>
-__device__ __forceinline__ V vsplat(float c);
-template <>
-__device__ __forceinline__ F2 vsplat<F2>(float c) { return F2{make_float2(c, c)}; }
 __device__ __forceinline__ F2 vpair(float x, float y) { return F2{make_float2(x, y)}; }
 __device__ __forceinline__ F2 vsame(float x) { return F2{make_float2(x, x)}; }
 __device__ __forceinline__ F2 vadd(F2 a, F2 b) { return F2{__fadd2_rn(a.v, b.v)}; }
@@ -582,41 +526,187 @@ __device__ __forceinline__ F2 vsub(F2 a, F2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_bits(a)), "l"(f2_bits(b)));
   return bits_f2(r);
 }
-__device__ __forceinline__ F2 vrcp(F2 a) { return vpair(__frcp_rn(a.v.x), __frcp_rn(a.v.y)); }
 __device__ __forceinline__ float vlo(F2 a) { return a.v.x; }
 __device__ __forceinline__ float vhi(F2 a) { return a.v.y; }
+__device__ __forceinline__ double vadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double vmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double vsub(double a, double b) { return __dsub_rn(a, b); }
+template <typename V>
+struct Val;
+template <>
+struct Val<F2> {
+  using T = float;
+  static __device__ __forceinline__ F2 splat(float c) { return vsame(c); }
+};
+template <>
+struct Val<double> {
+  using T = double;
+  static __device__ __forceinline__ double splat(double c) { return c; }
+};
 __device__ __forceinline__ bool rho_bad(float r) { return !(r > 0.f) || !isfinite(r); }
+__device__ __forceinline__ bool rho_bad(double r) { return !(r > 0.0) || !isfinite(r); }
 
-// The collision of collide() in the packed FP32 arithmetic above, with the
-// relaxation rate and weights folded into the even part's coefficients: for
-// each pair
+// 1 / a by Newton's iteration y <- y + y (1 - a y) from the hardware's
+// approximation (relative error below 2^-22 in FP32, about 2^-20 in FP64; the
+// error squares at each iteration): one iteration in FP32, two in FP64, each
+// two FMAs, where the correctly rounded division's range checks and fix-ups
+// cost several times that.  Densities are near 1.
+__device__ __forceinline__ F2 vrcp(F2 a) {
+  float x, y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(a.v.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a.v.y));
+  const F2 r = vpair(x, y);
+  return vfma(r, vfma(vmul(a, vsame(-1.0f)), r, vsame(1.0f)), r);
+}
+__device__ __forceinline__ double vrcp(double a) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+#pragma unroll
+  for (int k = 0; k < 2; ++k) r = vfma(r, vfma(-a, r, 1.0), r);
+  return r;
+}
+
+// Sums and differences of the opposite pairs (a, opp(a)), a = 1, 2, 5, 6, and
+// the moments of the offsets: drho = rho - 1 and (djx, djy) = j - u_ref.
+template <typename V>
+struct Moments {
+  V s[4], d[4], drho, djx, djy;
+  __device__ __forceinline__ explicit Moments(const V (&h)[9]) {
+    s[0] = vadd(h[1], h[3]);
+    d[0] = vsub(h[1], h[3]);
+    s[1] = vadd(h[2], h[4]);
+    d[1] = vsub(h[2], h[4]);
+    s[2] = vadd(h[5], h[7]);
+    d[2] = vsub(h[5], h[7]);
+    s[3] = vadd(h[6], h[8]);
+    d[3] = vsub(h[6], h[8]);
+    drho = vadd(vadd(h[0], vadd(s[0], s[1])), vadd(s[2], s[3]));
+    djx = vadd(d[0], vsub(d[2], d[3]));
+    djy = vadd(d[1], vadd(d[2], d[3]));
+  }
+};
+
+// BGK/TRT collision with the forcing term (Eq. TRT), into o.  The equilibrium
+// enters through its offset heq = feq(rho, u) - E, written with the small
+// quantities drho, du = u - u_ref and dj = rho u - u_ref only.  Its second
+// moments are three products,
+//   X = rho u_x^2 - u_ref,x^2 = dj_x u_x + u_ref,x du_x, Y alike, and
+//   P = rho u_x u_y - u_ref,x u_ref,y = dj_x u_y + u_ref,x du_y,
+// from which the even parts follow, heq+ = w [drho - 1.5 (X + Y) + 4.5 X_a]
+// with X_1 = X, X_2 = Y, X_5,6 = X + Y +- 2 P; the odd parts are
+// heq- = 3 w c.dj.  (FP64 runs at about 1/58 of the FP32 rate on this part and
+// FP32 is bound by its FMA pipe in the kernels that fuse two steps, so the
+// operation count is what both pay for: 76 operations per node, where the form
+// with (c.u)^2 and c.u per direction took 115 and a division.)
+//
+// The odd rates sm_k1 = 3 w_1 s- and sm_k2 = 3 w_5 s- satisfy
+// sm_k1 + 2 sm_k2 = s-/2 exactly (api.cu), so that the odd equilibrium carries
+// exactly the node's momentum: rounded independently they would make every
+// collision add about 1e-8 of the momentum offset, a bias that compounds step
+// after step.  The
+// rest population takes what the moving populations' even parts give up,
+// o_0 = h_0 - 2 sum (even change of a pair's population): equal to the
+// relaxation of h_0 towards heq_0 (plus F_0) in exact arithmetic, and
+// conserving mass exactly up to the rounding of that sum.  kForce = false
+// drops the forcing term (G = 0: a fluid node without body force).
+template <typename V, bool kForce>
+__device__ __forceinline__ void collide(const V (&h)[9], const Moments<V> &m, V djx, V djy, V ux,
+                                        V uy, V dux, V duy, V gx, V gy,
+                                        const Consts<typename Val<V>::T> &c, V (&o)[9]) {
+  using T = typename Val<V>::T;
+  auto k = [](T v) { return Val<V>::splat(v); };
+  const V X = vfma(djx, ux, vmul(k(c.urx), dux));
+  const V Y = vfma(djy, uy, vmul(k(c.ury), duy));
+  const V P = vfma(djx, uy, vmul(k(c.urx), duy));
+  const V t = vadd(X, Y);
+  const V axis = vmul(k(c.sp_w1), vfma(k((T)-1.5), t, m.drho));
+  const V diag = vmul(k(c.sp_w5), vfma(k((T)3), t, m.drho));
+  V even{};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int a = q < 2 ? q + 1 : q + 3, b = opp_of(a);
+    // s+ heq+ of the pair and c.dj
+    const V ep = q == 0   ? vfma(k(c.sp_45w1), X, axis)
+                 : q == 1 ? vfma(k(c.sp_45w1), Y, axis)
+                 : q == 2 ? vfma(k(c.sp_9w5), P, diag)
+                          : vfma(k(-c.sp_9w5), P, diag);
+    const V cdj = q == 0 ? djx : q == 1 ? djy : q == 2 ? vadd(djx, djy) : vsub(djy, djx);
+    V dp = vfma(k(c.nsp_half), m.s[q], ep);
+    V dm = vfma(k(c.nsm_half), m.d[q], vmul(k(q < 2 ? c.sm_k1 : c.sm_k2), cdj));
+    if (kForce) {
+      // F_a = w [3 c.G + 9 (c.u)(c.G) - 3 u.G], even and odd parts
+      const V cu = q == 0 ? ux : q == 1 ? uy : q == 2 ? vadd(ux, uy) : vsub(uy, ux);
+      const V cg = q == 0 ? gx : q == 1 ? gy : q == 2 ? vadd(gx, gy) : vsub(gy, gx);
+      const V ug = vfma(ux, gx, vmul(uy, gy));
+      const T w = (T)w_of(a);
+      dp = vfma(k(c.a_plus * w * (T)9), vmul(cu, cg), vfma(k(c.a_plus * w * (T)-3), ug, dp));
+      dm = vfma(k(c.a_minus), vmul(k(odd_w<T>(a)), cg), dm);
+    }
+    even = q == 0 ? dp : vadd(even, dp);
+    o[a] = vadd(vadd(h[a], dp), dm);
+    o[b] = vsub(vadd(h[b], dp), dm);
+  }
+  o[0] = vfma(k((T)-2), even, h[0]);
+}
+
+// The update of fluid nodes (no penalization): moments, velocity and the
+// collision, from the pre-collision offsets h of a node (FP64), a node pair or
+// one node in both lanes (FP32); kForce adds the uniform body force.  Returns
+// rho.
+template <typename V, bool kForce>
+__device__ __forceinline__ V fluid_update(const Lattice &L, const Consts<typename Val<V>::T> &cst,
+                                          const V (&h)[9], V (&o)[9]) {
+  using T = typename Val<V>::T;
+  const Moments<V> m(h);
+  const V rho = vadd(Val<V>::splat((T)1), m.drho);
+  const V inv = vrcp(rho);
+  V djx = m.djx, djy = m.djy, gx{}, gy{};
+  if (kForce) {
+    gx = Val<V>::splat(lat_bf<T>(L, 0));
+    gy = Val<V>::splat(lat_bf<T>(L, 1));
+    djx = vfma(Val<V>::splat((T)0.5), gx, djx);
+    djy = vfma(Val<V>::splat((T)0.5), gy, djy);
+  }
+  const V dux = vmul(vfma(m.drho, Val<V>::splat(-cst.urx), djx), inv);
+  const V duy = vmul(vfma(m.drho, Val<V>::splat(-cst.ury), djy), inv);
+  collide<V, kForce>(h, m, djx, djy, vadd(Val<V>::splat(cst.urx), dux),
+                     vadd(Val<V>::splat(cst.ury), duy), dux, duy, gx, gy, cst, o);
+  return rho;
+}
+
+// ---------------------------------------------------------------------------
+// 16-bit storage keeps the arithmetic it began with, bit for bit: every stored
+// value is rounded to 16 bits, so any change of FP32 rounding flips some of
+// them and the run follows another rounding history (instantaneous forces move
+// by 1e-3, where the form above moves FP32 lattices by 1e-6).  Per pair
 // (a, opp(a))
 //   s+ heq+ = s+ w K + 4.5 s+ w X,  X = drho (c.u)^2 + (c.du)(c.u + c.u_ref),
 //   K = drho (1 - 1.5 |u|^2) - 1.5 (|u|^2 - |u_ref|^2),
-// the same terms as heq_a = w_a [drho (1 + Q_a(u)) + Q_a(u) - Q_a(u_ref)].  The
-// odd part keeps collide()'s form -s- (h- - k (drho c.u + c.du)) with the
-// coefficients k of odd_w (its momentum is then exact: a folded s- k would
-// round differently from s-), and the rest population takes the even
-// changes' remainder as in collide().
-template <typename V, typename T, bool kForce>
-__device__ __forceinline__ void collide2(const V (&h)[9], V drho, V dux, V duy, V gx, V gy,
-                                         const Consts<T> &c, V (&o)[9]) {
-  const V urx = vsplat<V>(c.urx), ury = vsplat<V>(c.ury);
+// the odd part is -s- (h- - k (drho c.u + c.du)), and the rest population
+// takes the even changes' remainder.
+// ---------------------------------------------------------------------------
+template <bool kForce>
+__device__ __forceinline__ void collide16(const F2 (&h)[9], F2 drho, F2 dux, F2 duy, F2 gx, F2 gy,
+                                          const Consts<float> &c, F2 (&o)[9]) {
+  using V = F2;
+  using T = float;
+  const V urx = vsame(c.urx), ury = vsame(c.ury);
   const V ux = vadd(urx, dux), uy = vadd(ury, duy);
   const V uu = vfma(ux, ux, vmul(uy, uy));
   const V dsu = vfma(dux, vadd(ux, urx), vmul(duy, vadd(uy, ury)));
-  const V m15 = vsplat<V>((T)-1.5);
-  const V K = vfma(m15, dsu, vmul(drho, vfma(m15, uu, vsplat<V>((T)1))));
+  const V m15 = vsame((T)-1.5);
+  const V K = vfma(m15, dsu, vmul(drho, vfma(m15, uu, vsame((T)1))));
   V ug{};
   if (kForce) ug = vfma(ux, gx, vmul(uy, gy));
-  const V nsph = vsplat<V>((T)-0.5 * c.s_plus), nsm = vsplat<V>(-c.s_minus), half = vsplat<V>((T)0.5);
-  V even = vsplat<V>((T)0);
+  const V nsph = vsame((T)-0.5 * c.s_plus), nsm = vsame(-c.s_minus), half = vsame((T)0.5);
+  V even = vsame((T)0);
 #pragma unroll
   for (int a = 1; a <= 6; ++a) {
     if (a == 3 || a == 4) continue;
     const int b = opp_of(a);
     const T w = (T)w_of(a);
-    const V k = vsplat<V>(odd_w<T>(a));
+    const V k = vsame(odd_w<T>(a));
     // c.u, c.du for the four directions 1 (1,0), 2 (0,1), 5 (1,1), 6 (-1,1)
     V cu, cdu;
     if (a == 1) {
@@ -632,10 +722,10 @@ __device__ __forceinline__ void collide2(const V (&h)[9], V drho, V dux, V duy, 
       cu = vsub(uy, ux);
       cdu = vsub(duy, dux);
     }
-    const V csu = vadd(cu, vsplat<V>((T)cx_of(a) * c.urx + (T)cy_of(a) * c.ury));
+    const V csu = vadd(cu, vsame((T)cx_of(a) * c.urx + (T)cy_of(a) * c.ury));
     const V dc = vmul(drho, cu);
     const V X = vfma(dc, cu, vmul(cdu, csu));
-    const V P = vfma(vsplat<V>((T)4.5 * c.s_plus * w), X, vmul(vsplat<V>(c.s_plus * w), K));
+    const V P = vfma(vsame((T)4.5 * c.s_plus * w), X, vmul(vsame(c.s_plus * w), K));
     V dp = vfma(nsph, vadd(h[a], h[b]), P);
     // -s- (h- - heq-), h- = (h_a - h_b) / 2, heq- = k (drho c.u + c.du)
     V dm = vmul(nsm, vsub(vmul(half, vsub(h[a], h[b])), vmul(k, vadd(dc, cdu))));
@@ -649,132 +739,124 @@ __device__ __forceinline__ void collide2(const V (&h)[9], V drho, V dux, V duy, 
         cg = vadd(gx, gy);
       else
         cg = vsub(gy, gx);
-      dp = vfma(vsplat<V>(c.a_plus * w * (T)9), vmul(cu, cg), vfma(vsplat<V>(c.a_plus * w * (T)-3), ug, dp));
-      dm = vfma(vsplat<V>(c.a_minus), vmul(k, cg), dm);
+      dp = vfma(vsame(c.a_plus * w * (T)9), vmul(cu, cg), vfma(vsame(c.a_plus * w * (T)-3), ug, dp));
+      dm = vfma(vsame(c.a_minus), vmul(k, cg), dm);
     }
     even = vadd(even, dp);
     o[a] = vadd(vadd(h[a], dp), dm);
     o[b] = vsub(vadd(h[b], dp), dm);
   }
-  o[0] = vfma(vsplat<V>((T)-2), even, h[0]);
+  o[0] = vfma(vsame((T)-2), even, h[0]);
 }
 
-// The update of fluid nodes (no penalization) in FP32: moments, velocity and
-// the collision, from the pre-collision offsets h of a node pair (or of one
-// node in both lanes); kForce adds the uniform body force.  Returns rho.
-template <typename V, bool kForce>
-__device__ __forceinline__ V fluid_update(const Lattice &L, const Consts<float> &cst,
-                                          const V (&h)[9], V (&o)[9]) {
-  const V drho = vadd(vadd(vadd(h[0], h[1]), vadd(h[2], h[3])),
-                      vadd(vadd(vadd(h[4], h[5]), vadd(h[6], h[7])), h[8]));
-  V djx = vadd(vadd(vsub(h[1], h[3]), vsub(h[5], h[6])), vsub(h[8], h[7]));
-  V djy = vadd(vadd(vsub(h[2], h[4]), vsub(h[5], h[7])), vsub(h[6], h[8]));
-  const V rho = vadd(vsplat<V>(1.0f), drho);
-  const V inv = vrcp(rho);
+// moments of nine offsets in the order of the 16-bit forms
+__device__ __forceinline__ void moments16(const F2 (&h)[9], F2 &drho, F2 &djx, F2 &djy) {
+  drho = vadd(vadd(vadd(h[0], h[1]), vadd(h[2], h[3])),
+              vadd(vadd(vadd(h[4], h[5]), vadd(h[6], h[7])), h[8]));
+  djx = vadd(vadd(vsub(h[1], h[3]), vsub(h[5], h[6])), vsub(h[8], h[7]));
+  djy = vadd(vadd(vsub(h[2], h[4]), vsub(h[5], h[7])), vsub(h[6], h[8]));
+}
+
+template <bool kForce>
+__device__ __forceinline__ F2 fluid_update16(const Lattice &L, const Consts<float> &cst,
+                                             const F2 (&h)[9], F2 (&o)[9]) {
+  F2 drho, djx, djy;
+  moments16(h, drho, djx, djy);
+  const F2 rho = vadd(vsame(1.0f), drho);
+  const F2 inv = vpair(__frcp_rn(rho.v.x), __frcp_rn(rho.v.y));
+  F2 gx{}, gy{};
   if (kForce) {
-    const V gx = vsplat<V>(lat_bf<float>(L, 0)), gy = vsplat<V>(lat_bf<float>(L, 1));
-    djx = vfma(vsplat<V>(0.5f), gx, djx);
-    djy = vfma(vsplat<V>(0.5f), gy, djy);
-    collide2<V, float, true>(h, drho, vmul(vfma(drho, vsplat<V>(-cst.urx), djx), inv),
-                             vmul(vfma(drho, vsplat<V>(-cst.ury), djy), inv), gx, gy, cst, o);
-  } else {
-    collide2<V, float, false>(h, drho, vmul(vfma(drho, vsplat<V>(-cst.urx), djx), inv),
-                              vmul(vfma(drho, vsplat<V>(-cst.ury), djy), inv), V{}, V{}, cst, o);
+    gx = vsame(lat_bf<float>(L, 0));
+    gy = vsame(lat_bf<float>(L, 1));
+    djx = vfma(vsame(0.5f), gx, djx);
+    djy = vfma(vsame(0.5f), gy, djy);
   }
+  collide16<kForce>(h, drho, vmul(vfma(drho, vsame(-cst.urx), djx), inv),
+                    vmul(vfma(drho, vsame(-cst.ury), djy), inv), gx, gy, cst, o);
   return rho;
 }
+
+// the fluid update of storage form S
+template <typename S, bool kForce, typename V>
+__device__ __forceinline__ V update_fluid(const Lattice &L,
+                                          const Consts<typename Val<V>::T> &cst,
+                                          const V (&h)[9], V (&o)[9]) {
+  if constexpr (sizeof(S) == 2)
+    return fluid_update16<kForce>(L, cst, h, o);
+  else
+    return fluid_update<V, kForce>(L, cst, h, o);
+}
+
+// a single node's value as V (in both lanes) and back
+template <typename T>
+struct NodeVal;
+template <>
+struct NodeVal<float> {
+  using V = F2;
+  static __device__ __forceinline__ float get(F2 v) { return vlo(v); }
+};
+template <>
+struct NodeVal<double> {
+  using V = double;
+  static __device__ __forceinline__ double get(double v) { return v; }
+};
 
 // Moments, penalized velocity and force density of one node (Eqs. updatestep
 // .. updatestepm: G = -rho (chi/eta)(u - u_s) in the rearranged form
 // -(chi/eta)(j - rho u_s)/(1 + chi dt/(2 eta)), plus the body force), then
-// the collision.  Returns true for a non-finite or non-positive density.
-template <typename T, bool kPacked>
-__device__ __forceinline__ bool update_node(const T (&h)[9], uint8_t m, int i, int j,
+// the collision; a fluid node gets the same bits as from the bulk kernels.
+// (pen_x, pen_y): the penalization part of G (solid nodes only).  Returns true
+// for a non-finite or non-positive density.
+template <typename S, typename T>
+__device__ __forceinline__ bool update_node(const T (&h)[9], uint8_t mask, int i, int j,
                                             const Lattice &L, const BodyState *body,
                                             const Consts<T> &cst, T (&o)[9], T &pen_x,
                                             T &pen_y) {
-  pen_x = pen_y = (T)0;  // the penalization part of G (solid nodes only)
-  if constexpr (kPacked) {
-    // FP32 compute (FP32 and 16-bit storage): the packed arithmetic of
-    // fluid_update, which the bulk kernels of these forms use, with the node
-    // in both lanes, so that a fluid node gets the same bits in either kernel
-    F2 hv[9], ov[9];
+  using N = NodeVal<T>;
+  using V = typename N::V;
+  pen_x = pen_y = (T)0;
+  V hv[9], ov[9], rho;
 #pragma unroll
-    for (int a = 0; a < 9; ++a) hv[a] = vsame(h[a]);
-    F2 rho;
-    if (!(m & kSolid)) {
-      rho = L.has_bf ? fluid_update<F2, true>(L, cst, hv, ov) : fluid_update<F2, false>(L, cst, hv, ov);
-    } else {
-      const F2 drho = vadd(vadd(vadd(hv[0], hv[1]), vadd(hv[2], hv[3])),
-                           vadd(vadd(vadd(hv[4], hv[5]), vadd(hv[6], hv[7])), hv[8]));
-      F2 djx = vadd(vadd(vsub(hv[1], hv[3]), vsub(hv[5], hv[6])), vsub(hv[8], hv[7]));
-      F2 djy = vadd(vadd(vsub(hv[2], hv[4]), vsub(hv[5], hv[7])), vsub(hv[6], hv[8]));
-      rho = vadd(vsame(1.0f), drho);
-      const float bfx = lat_bf<float>(L, 0), bfy = lat_bf<float>(L, 1);
-      djx = vfma(vsame(0.5f), vsame(bfx), djx);
-      djy = vfma(vsame(0.5f), vsame(bfy), djy);
-      float usx, usy;
-      solid_velocity<float>(*body, i, j, usx, usy);
-      const float k = cst.half_pen, r = vlo(rho), dr = vlo(drho);
-      const float den = r + k * r;
-      // the momentum defect j - rho u_s, and u - u_ref written as
-      // (u_s - u_ref) + (j - rho u_s)/(rho (1 + k)) (see below)
-      const float defx = vlo(djx) - dr * usx + (cst.urx - usx);
-      const float defy = vlo(djy) - dr * usy + (cst.ury - usy);
-      const float dux = (usx - cst.urx) + defx / den, duy = (usy - cst.ury) + defy / den;
-      const float pen = 2.0f * k;
-      pen_x = -pen * defx / (1.0f + k);
-      pen_y = -pen * defy / (1.0f + k);
-      collide2<F2, float, true>(hv, drho, vsame(dux), vsame(duy), vsame(bfx + pen_x),
-                                vsame(bfy + pen_y), cst, ov);
-    }
-#pragma unroll
-    for (int a = 0; a < 9; ++a) o[a] = vlo(ov[a]);
-    return rho_bad(vlo(rho));
+  for (int a = 0; a < 9; ++a) hv[a] = Val<V>::splat(h[a]);
+  if (!(mask & kSolid)) {
+    rho = L.has_bf ? update_fluid<S, true>(L, cst, hv, ov) : update_fluid<S, false>(L, cst, hv, ov);
   } else {
-  const T drho = ((h[0] + h[1]) + (h[2] + h[3])) + ((h[4] + h[5]) + (h[6] + h[7])) + h[8];
-  const T rho = (T)1 + drho;
-  // j - u_ref (the offsets' first moment; sum_a c_a E_a = u_ref)
-  T djx = (h[1] - h[3]) + (h[5] - h[6]) + (h[8] - h[7]);
-  T djy = (h[2] - h[4]) + (h[5] - h[7]) + (h[6] - h[8]);
-  if ((m & kSolid) || L.has_bf) {
+    const Moments<V> m(hv);
+    V drho = m.drho, jx = m.djx, jy = m.djy;
+    if constexpr (sizeof(S) == 2) moments16(hv, drho, jx, jy);
+    rho = vadd(Val<V>::splat((T)1), drho);
     const T bfx = lat_bf<T>(L, 0), bfy = lat_bf<T>(L, 1);
-    djx += (T)0.5 * bfx;
-    djy += (T)0.5 * bfy;
-    T dux, duy, gx = bfx, gy = bfy;
-    if (m & kSolid) {
-      T usx, usy;
-      solid_velocity<T>(*body, i, j, usx, usy);
-      const T k = cst.half_pen;
-      const T den = rho + k * rho;
-      // the momentum defect j - rho u_s, from the offsets' first moment
-      const T defx = djx - drho * usx + (cst.urx - usx);
-      const T defy = djy - drho * usy + (cst.ury - usy);
-      // u - u_ref = (j + k rho u_s)/(rho (1 + k)) - u_ref, written as
-      // (u_s - u_ref) + (j - rho u_s)/(rho (1 + k)): the large part is exact
-      // and the small one keeps its relative precision (k rho u_s alone
-      // would carry an FP32 rounding of 1e-3 into the division by k rho)
-      dux = (usx - cst.urx) + defx / den;
-      duy = (usy - cst.ury) + defy / den;
-      // G = -(chi/eta)(j - rho u_s)/(1 + k)
-      const T pen = (T)2 * k;
-      pen_x = -pen * defx / ((T)1 + k);
-      pen_y = -pen * defy / ((T)1 + k);
-      gx += pen_x;
-      gy += pen_y;
+    const T djx = N::get(vfma(Val<V>::splat((T)0.5), Val<V>::splat(bfx), jx));
+    const T djy = N::get(vfma(Val<V>::splat((T)0.5), Val<V>::splat(bfy), jy));
+    T usx, usy;
+    solid_velocity<T>(*body, i, j, usx, usy);
+    const T k = cst.half_pen, r = N::get(rho), dr = N::get(drho);
+    const T den = r + k * r;
+    // the momentum defect j - rho u_s, from the offsets' first moment
+    const T defx = djx - dr * usx + (cst.urx - usx);
+    const T defy = djy - dr * usy + (cst.ury - usy);
+    // u - u_ref = (j + k rho u_s)/(rho (1 + k)) - u_ref, written as
+    // (u_s - u_ref) + (j - rho u_s)/(rho (1 + k)): the large part is exact
+    // and the small one keeps its relative precision (k rho u_s alone
+    // would carry an FP32 rounding of 1e-3 into the division by k rho)
+    const T dux = (usx - cst.urx) + defx / den, duy = (usy - cst.ury) + defy / den;
+    // G = -(chi/eta)(j - rho u_s)/(1 + k)
+    const T pen = (T)2 * k;
+    pen_x = -pen * defx / ((T)1 + k);
+    pen_y = -pen * defy / ((T)1 + k);
+    const V vx = Val<V>::splat(dux), vy = Val<V>::splat(duy);
+    const V gx = Val<V>::splat(bfx + pen_x), gy = Val<V>::splat(bfy + pen_y);
+    if constexpr (sizeof(S) == 2) {
+      collide16<true>(hv, drho, vx, vy, gx, gy, cst, ov);
     } else {
-      const T inv = (T)1 / rho;
-      dux = (djx - drho * cst.urx) * inv;
-      duy = (djy - drho * cst.ury) * inv;
+      // rho u - u_ref with the penalized velocity
+      const V ux = Val<V>::splat(usx + defx / den), uy = Val<V>::splat(usy + defy / den);
+      collide<V, true>(hv, m, vfma(drho, ux, vx), vfma(drho, uy, vy), ux, uy, vx, vy, gx, gy, cst, ov);
     }
-    collide<T, true>(h, drho, dux, duy, gx, gy, cst, o);
-  } else {
-    const T inv = (T)1 / rho;
-    collide<T, false>(h, drho, (djx - drho * cst.urx) * inv, (djy - drho * cst.ury) * inv, (T)0,
-                      (T)0, cst, o);
   }
-  return !(rho > (T)0) || !isfinite(rho);
-  }
+#pragma unroll
+  for (int a = 0; a < 9; ++a) o[a] = N::get(ov[a]);
+  return rho_bad(N::get(rho));
 }
 
 // ---------------------------------------------------------------------------
@@ -877,8 +959,7 @@ __device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bo
     m = p.chi[node];
   }
   T o[9], pen_x, pen_y;
-  const bool bad = update_node<T, sizeof(T) == 4>(h, m, i, j, L, p.body_src, Consts<T>(p), o, pen_x,
-                                                  pen_y);
+  const bool bad = update_node<S>(h, m, i, j, L, p.body_src, Consts<T>(p), o, pen_x, pen_y);
   if (sizeof(S) == 2 && p.sr) {
     const SrBits r(sr_level(p), (uint32_t)node >> 1);
 #pragma unroll
@@ -1034,26 +1115,11 @@ __global__ void __launch_bounds__(kThreads * kTiles) bulk_kernel(const StepArgs 
     const ForceRegion reg = *p.reg_src;
     if (ti >= reg.ti0 && ti <= reg.ti1 && tj >= reg.tj0 && tj <= reg.tj1) return;  // special kernel
   }
-  const Consts<T> cst(p);
-  const T drho = ((h[0] + h[1]) + (h[2] + h[3])) + ((h[4] + h[5]) + (h[6] + h[7])) + h[8];
-  const T rho = (T)1 + drho;
-  T djx = (h[1] - h[3]) + (h[5] - h[6]) + (h[8] - h[7]);
-  T djy = (h[2] - h[4]) + (h[5] - h[7]) + (h[6] - h[8]);
   T o[9];
-  const T inv = (T)1 / rho;
-  if (kForce) {
-    const T bfx = lat_bf<T>(L, 0), bfy = lat_bf<T>(L, 1);
-    djx += (T)0.5 * bfx;
-    djy += (T)0.5 * bfy;
-    collide<T, true>(h, drho, (djx - drho * cst.urx) * inv, (djy - drho * cst.ury) * inv, bfx,
-                     bfy, cst, o);
-  } else {
-    collide<T, false>(h, drho, (djx - drho * cst.urx) * inv, (djy - drho * cst.ury) * inv, (T)0,
-                      (T)0, cst, o);
-  }
+  const T rho = update_fluid<S, kForce>(L, Consts<T>(p), h, o);
 #pragma unroll
   for (int a = 0; a < 9; ++a) Store<S>::st(dst + (int64_t)a * L.plane + node, o[a]);
-  if (!(rho > (T)0) || !isfinite(rho)) atomicOr(p.status, kStatusUnstable);
+  if (rho_bad(rho)) atomicOr(p.status, kStatusUnstable);
 }
 
 // ---------------------------------------------------------------------------
@@ -1104,7 +1170,7 @@ __global__ void __launch_bounds__(kThreads / 2 * kTiles) bulk32x2_kernel(const S
   const bool ok0 = i >= 1 && i <= L.nx - 2, ok1 = i + 1 <= L.nx - 2;
   if (!ok0 && !ok1) return;
   F2 o[9];
-  const F2 rho = fluid_update<F2, kForce>(L, Consts<float>(p), h, o);
+  const F2 rho = update_fluid<float, kForce>(L, Consts<float>(p), h, o);
   float *dst = static_cast<float *>(p.dst) + (int64_t)j * L.pitch + i;
   if (ok0 && ok1) {
 #pragma unroll
@@ -1177,7 +1243,7 @@ __device__ __forceinline__ F2 collide_pair16(const StepArgs &p, const uint32_t (
 #pragma unroll
   for (int a = 0; a < 9; ++a) h[a] = vpair(P::lo(w[a]), P::hi(w[a]));
   F2 o[9];
-  const F2 rho = fluid_update<F2, kForce>(p.L, Consts<float>(p), h, o);
+  const F2 rho = update_fluid<S, kForce>(p.L, Consts<float>(p), h, o);
   if constexpr (kSR) {
     const SrBits r(level, node >> 1);
 #pragma unroll

@@ -410,6 +410,15 @@ struct ForceRegion {
 // less than one node per step, so its mask update stays inside the region
 constexpr int kRegionMargin = 4;
 
+// relaxation rates folded with the lattice weights (w1 axis, w5 diagonal),
+// and with k = 3 w for the odd parts: sm_k1 + 2 sm_k2 = s-/2 exactly
+template <typename T>
+struct CollideC {
+  T nsp_half, nsm_half;                 // -s+/2, -s-/2
+  T sp_w1, sp_w5, sp_45w1, sp_9w5;      // s+ w1, s+ w5, 4.5 s+ w1, 9 s+ w5
+  T sm_k1, sm_k2;
+};
+
 // ---------------------------------------------------------------------------
 // parameters of the fused step kernel
 // ---------------------------------------------------------------------------
@@ -446,12 +455,14 @@ struct StepArgs {
   int32_t *status;
   // collision constants, FP64 and FP32 copies (FP32 paths must not convert
   // from FP64 per node: GB300 runs FP64 at a small fraction of FP32)
-  double s_plus, s_minus;  // 1/tau+, 1/tau-
   double a_plus, a_minus;  // forcing prefactors
   double half_pen;         // dt/(2 eta)
   double tau_plus;
   double sim_const[3];     // -(1/3) sum S n and its moment: the SIM constant part
   float f_s_plus, f_s_minus, f_a_plus, f_a_minus, f_half_pen, f_sim_s;
+  // the collision's folded coefficients (CollideC), in either precision
+  CollideC<double> coll;
+  CollideC<float> f_coll;
   int32_t ntiles_x, ntiles_y;
   int32_t region_capacity;  // most force-region tiles a step may hold
   int32_t tile_w;           // nodes along x of one tile
@@ -546,17 +557,17 @@ __host__ __device__ inline void edge_node(int e, int nx, int ny, int &i, int &j)
 template <typename T>
 struct Consts;
 template <>
-struct Consts<double> {
-  double s_plus, s_minus, a_plus, a_minus, half_pen, sim_s, urx, ury;
+struct Consts<double> : CollideC<double> {
+  double a_plus, a_minus, half_pen, sim_s, urx, ury;
   __device__ __forceinline__ explicit Consts(const StepArgs &p)
-      : s_plus(p.s_plus), s_minus(p.s_minus), a_plus(p.a_plus), a_minus(p.a_minus),
-        half_pen(p.half_pen), sim_s(1.0 - 0.5 / p.tau_plus), urx(p.L.ur[0]), ury(p.L.ur[1]) {}
+      : CollideC<double>(p.coll), a_plus(p.a_plus), a_minus(p.a_minus), half_pen(p.half_pen),
+        sim_s(1.0 - 0.5 / p.tau_plus), urx(p.L.ur[0]), ury(p.L.ur[1]) {}
 };
 template <>
-struct Consts<float> {
+struct Consts<float> : CollideC<float> {
   float s_plus, s_minus, a_plus, a_minus, half_pen, sim_s, urx, ury;
   __device__ __forceinline__ explicit Consts(const StepArgs &p)
-      : s_plus(p.f_s_plus), s_minus(p.f_s_minus), a_plus(p.f_a_plus), a_minus(p.f_a_minus),
+      : CollideC<float>(p.f_coll), s_plus(p.f_s_plus), s_minus(p.f_s_minus), a_plus(p.f_a_plus), a_minus(p.f_a_minus),
         half_pen(p.f_half_pen), sim_s(p.f_sim_s), urx(p.L.ur_f[0]), ury(p.L.ur_f[1]) {}
 };
 
