@@ -53,6 +53,7 @@ BULK_NAME = {"f32": "bulk32x2_kernel", "f16": "bulk16_kernel<__half>",
              "bf16sr": "bulk16_kernel<__nv_bfloat16, sr>"}
 PROFILE = os.path.join(ROOT, "profiles", "step_kernel_naca2048_f32.md")
 KERNEL_SOURCES = ("paper_2110_00967_gb300/csrc/step.cu",
+                  "paper_2110_00967_gb300/csrc/pair.cuh",
                   "paper_2110_00967_gb300/csrc/vplbm_internal.cuh",
                   "paper_2110_00967_gb300/csrc/api.cu")
 METRIC = "VP-LBM MLUPS"

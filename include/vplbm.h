@@ -183,8 +183,10 @@ vplbm_status vplbm_set_body(vplbm_ctx *ctx, const vplbm_body *body);
  * Runs of steps are replayed from CUDA graphs of 1, 2, 4, ..., 32 steps,
  * captured (all of them, from either population buffer) at the first run
  * that can use one: when the lattice is past its first step and SIM runs
- * every step or never.  The call returns with the last step's forces in the
- * history. */
+ * every step or never.  In these graphs a lattice with a fixed body or none,
+ * FP32 or 16-bit storage and at least 100000 nodes takes two steps per launch
+ * where that is faster; the results are those of single steps bit for bit.  The
+ * call returns with the last step's forces in the history. */
 vplbm_status vplbm_step(vplbm_ctx *ctx, int32_t nsteps);
 
 /* Captures and uploads, now, the step graphs that runs of nsteps steps use
@@ -329,7 +331,8 @@ vplbm_status vplbm_launch_count(vplbm_ctx *ctx, int64_t *n);
  * from the edges and the body comes in three launch forms which compute the
  * same values bit for bit: FP32/FP64 storage, blocks of one, two or four
  * 128 x 2 tiles; 16-bit storage, eight nodes per thread at 96 or 126
- * registers, or four nodes per thread.
+ * registers, or four nodes per thread; lattices stepped two steps per launch
+ * (see vplbm_step), runs of rows by a rule on the size, or of 12 or 24 rows.
  * Form 0 is the default.
  *
  * vplbm_autotune times the forms on this lattice's own steps: three passes

@@ -50,7 +50,7 @@ size_t elem_bytes(int dtype) {
 
 struct Layout {
   size_t buf[2], prev[2], chi, sim_pts, sim_nodes, hist, body[2], region[2], sums, counts,
-      dev_step, ticket, status, acc, rng, total;
+      dev_step, ticket, status, acc, rng, snap_end, acc2, total;
 };
 
 int effective_max_sim(const vplbm_config &c) { return c.max_sim_points > 0 ? c.max_sim_points : 4096; }
@@ -96,6 +96,8 @@ Layout make_layout(const vplbm_config &c) {
   l.status = take(sizeof(int32_t));
   l.acc = take(2 * kAccWords * sizeof(unsigned long long));  // by step parity
   l.rng = take(2 * sizeof(unsigned long long));                // rounding counter, by parity
+  l.snap_end = off;  // a snapshot ends here: what follows is zero between calls
+  l.acc2 = take(2 * kAccWords * sizeof(unsigned long long));  // second steps of pairs, by parity
   l.total = off;
   return l;
 }
@@ -210,6 +212,21 @@ bool build_polygon(const vplbm_body &b, int n, std::vector<SimPoint> &pts) {
   return true;
 }
 
+// the body's polygon box (each edge's midpoint widened by half its length)
+struct Extent {
+  double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
+};
+Extent extent_of(const vplbm_body &b, const std::vector<SimPoint> &pts) {
+  Extent e;
+  for (const SimPoint &p : pts) {
+    e.x0 = std::min(e.x0, b.x_c + p.dx - 0.5 * p.s);
+    e.x1 = std::max(e.x1, b.x_c + p.dx + 0.5 * p.s);
+    e.y0 = std::min(e.y0, b.y_c + p.dy - 0.5 * p.s);
+    e.y1 = std::max(e.y1, b.y_c + p.dy + 0.5 * p.s);
+  }
+  return e;
+}
+
 int default_sim_points(const vplbm_body &b) {
   if (b.n_sim_points > 0) return b.n_sim_points;
   if (b.kind == VPLBM_BODY_DISK) return (int)ceil(2.0 * M_PI * (0.5 * b.length) / 0.5);
@@ -217,6 +234,11 @@ int default_sim_points(const vplbm_body &b) {
 }
 
 }  // namespace
+
+// How a call's step graphs step: one step per launch pair, or two steps per
+// launch (pair.cuh) with the run lengths of a lattice alone or of one among
+// many.  The results are the same bit for bit.
+enum StepMode { kSingle = 0, kPairAlone = 1, kPairBatch = 2, kStepModes = 3 };
 
 struct vplbm_ctx {
   vplbm_config cfg;
@@ -231,6 +253,7 @@ struct vplbm_ctx {
   uint8_t *chi;
   SimPoint *sim_pts;
   unsigned long long *acc;
+  unsigned long long *acc2;
   unsigned long long *rng;
   int32_t *sim_nodes;
   double *hist;
@@ -245,6 +268,10 @@ struct vplbm_ctx {
   bool pre = true;    // the state is a pre-collision field (first step reads in place)
   bool pending = false;      // the last queued step's force sums still await finalizing
   bool pending_sim = false;  // ... and that step evaluated SIM
+  int pending_rows = 1;      // ... of one step, or of the two of a pair
+  bool pair_ok = false;      // two steps per launch are possible (pair_plan)
+  int mode = 0;              // how the current call steps (StepMode)
+  int box[4] = {0, -1, 0, -1};  // nodes around the body (StepArgs::box)
   bool mask_stale = false;   // a moving body's chi lags its body by a step
   bool has_body = false;
   vplbm_body body_cfg{};
@@ -255,11 +282,12 @@ struct vplbm_ctx {
   long long steps = 0;
   int64_t launches = 0;
   uint64_t generation = 0;  // bumped whenever captured step graphs go stale
-  // graphs[p][n]: n steps starting from buffer p, ending with finalized forces
-  cudaGraphExec_t graphs[2][kGraphMax + 1] = {};
-  cudaGraph_t graph_defs[2][kGraphMax + 1] = {};  // their definitions (batch graphs clone them)
+  // graphs[mode][p][n]: n steps starting from buffer p, ending with finalized
+  // forces; captured for the modes that calls use
+  cudaGraphExec_t graphs[kStepModes][2][kGraphMax + 1] = {};
+  cudaGraph_t graph_defs[kStepModes][2][kGraphMax + 1] = {};  // their definitions (batch graphs clone them)
   bool graph_wanted[kGraphMax + 1] = {};  // lengths beyond the powers of two
-  bool graphs_ready = false;
+  bool graphs_ready[kStepModes] = {};
   cudaStream_t side = nullptr;      // the special kernel's stream
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int region_slots = 1;             // blocks reserved for force-region tiles
@@ -331,6 +359,10 @@ StepArgs step_args(vplbm_ctx *c, int src, bool do_sim) {
   a.reg_dst = c->region[1 - src];
   a.acc = c->acc + kAccWords * src;
   a.acc_prev = c->acc + kAccWords * (1 - src);
+  a.acc2 = c->acc2 + kAccWords * src;
+  a.acc2_prev = c->acc2 + kAccWords * (1 - src);
+  a.prev_rows = c->pending_rows;
+  for (int k = 0; k < 4; ++k) a.box[k] = c->box[k];
   a.sim_pts = c->sim_pts;
   for (int k = 0; k < 3; ++k) a.sim_const[k] = c->sim_const[k];
   a.sim_nodes = c->sim_nodes;
@@ -430,8 +462,46 @@ cudaError_t queue_step(vplbm_ctx *c, cudaStream_t s, int src, bool pre, bool do_
   c->launches += 2;
   c->pending = a.defer != 0;
   c->pending_sim = do_sim;
+  c->pending_rows = 1;
   return e;
 }
+
+constexpr int64_t kPairSmall = 700000;
+// Rows per warp of the bulk blocks.  Long runs recompute fewer rim rows
+// ((rows + 2) / rows of the first step's work); short ones are more and shorter
+// blocks, which a lattice alone needs to fill 152 SMs and to keep its last wave
+// of blocks short.  us per step, FP32 (8 / 16 / 24 rows): 3614 x 1946 alone
+// 45.1 / 46.8 / 48.4, 2048 x 1024 alone 15.2 / 15.4 / 19.2, five of them 13.4 /
+// 13.05 / 12.8; 512 x 256 (6 / 12 / 16 rows) 3.9 / 4.4 / 5.0.
+int pair_rows(const vplbm_ctx *c) {
+  if (c->bulk_variant > 0) return c->bulk_variant == 1 ? 12 : 24;
+  if (c->mode == kPairBatch) return 20;
+  return (int64_t)c->L.nx * c->L.ny < kPairSmall || elem_bytes(c->cfg.dtype) == 2 ? 6 : 8;
+}
+
+// Two time steps in one launch on stream s (pair.cuh).
+cudaError_t queue_pair(vplbm_ctx *c, cudaStream_t s, int src, bool do_sim) {
+  StepArgs a = step_args(c, src, do_sim);
+  a.defer = 1;
+  a.finalize_prev = c->pending ? 1 : 0;
+  a.prev_sim = c->pending_sim ? 1 : 0;
+  a.pair_rows = pair_rows(c);
+  ++c->launches;
+  c->pending = true;
+  c->pending_sim = do_sim;
+  c->pending_rows = 2;
+  return launch_pair(storage_dtype(c->cfg.dtype), a, s);
+}
+
+// a graph of n steps: its moves of the state to the other buffer (one per
+// pair of steps, or per step), and its launches (one per pair, two per single
+// step, and those that end the run)
+int graph_moves(const vplbm_ctx *c, int n) { return c->mode != kSingle ? n / 2 + (n & 1) : n; }
+int graph_launches(const vplbm_ctx *c, int n) {
+  return (c->mode != kSingle ? n / 2 + 2 * (n & 1) : 2 * n) + 1 + (c->body_host.moving ? 1 : 0);
+}
+// the buffer holding the state after a graph of n steps from buffer cur
+int buffer_after(const vplbm_ctx *c, int cur, int n) { return cur ^ (graph_moves(c, n) & 1); }
 
 vplbm_status one_step(vplbm_ctx *c, cudaStream_t s) {
   VPLBM_CUDA(c, queue_step(c, s, c->cur, c->pre, sim_due(c, c->steps)));
@@ -442,28 +512,89 @@ vplbm_status one_step(vplbm_ctx *c, cudaStream_t s) {
 }
 
 void drop_graphs(vplbm_ctx *c) {
-  for (auto &row : c->graphs)
-    for (cudaGraphExec_t &g : row)
-      if (g) {
-        cudaGraphExecDestroy(g);
-        g = nullptr;
-      }
-  for (auto &row : c->graph_defs)
-    for (cudaGraph_t &g : row)
-      if (g) {
-        cudaGraphDestroy(g);
-        g = nullptr;
-      }
-  c->graphs_ready = false;
+  for (auto &mode : c->graphs)
+    for (auto &row : mode)
+      for (cudaGraphExec_t &g : row)
+        if (g) {
+          cudaGraphExecDestroy(g);
+          g = nullptr;
+        }
+  for (auto &mode : c->graph_defs)
+    for (auto &row : mode)
+      for (cudaGraph_t &g : row)
+        if (g) {
+          cudaGraphDestroy(g);
+          g = nullptr;
+        }
+  for (bool &ready : c->graphs_ready) ready = false;
   ++c->generation;  // batch graphs made of these go stale
 }
+
+// Decides whether the step graphs of the placed body take two steps per
+// launch, and sets the box of nodes around it that their special blocks update:
+// a fixed body (or none) with FP32 compute, SIM walks cached, clear of the
+// lattice edges (so that neither the box nor a sampled node's neighbours carry a
+// side condition), on a lattice of at least kPairMinNodes (a smaller one is a
+// few launches' latency either way) whose planes are addressed in 32-bit byte
+// offsets.
+constexpr int64_t kPairMinNodes = 100000;
+constexpr double kPairClearance = 12.0;
+// the box's margin around the polygon: the surface bulges beyond its edges by
+// far less than a node, an interface node lies one node off a solid one, and
+// the bulk blocks recompute one more
+constexpr double kBoxMargin = 3.0;
+struct PairPlan {
+  bool ok = false;
+  int box[4] = {0, -1, 0, -1};
+};
+PairPlan pair_plan(const vplbm_ctx *c, const vplbm_body &b, const std::vector<SimPoint> &pts) {
+  PairPlan q;
+  const Lattice &L = c->L;
+  if (c->cfg.dtype == VPLBM_F64 || b.moving || (int64_t)L.nx * L.ny < kPairMinNodes || L.nx < 64 ||
+      L.ny < 32 || L.nx > 0xffff || L.ny > 0xffff || L.plane >= (int64_t)1 << 30)
+    return q;
+  if (b.kind != VPLBM_BODY_NONE) {
+    const Extent e = extent_of(b, pts);
+    if (!(e.x0 >= kPairClearance && e.y0 >= kPairClearance && e.x1 <= L.nx - 1 - kPairClearance &&
+          e.y1 <= L.ny - 1 - kPairClearance))
+      return q;
+    q.box[0] = (int)floor(e.x0 - kBoxMargin) & ~1;
+    q.box[1] = (int)ceil(e.x1 + kBoxMargin) | 1;
+    q.box[2] = (int)floor(e.y0 - kBoxMargin);
+    q.box[3] = (int)ceil(e.y1 + kBoxMargin);
+  }
+  q.ok = true;
+  return q;
+}
+
+// Chooses how the lattices of a call step, from the nodes that the call steps
+// side by side.  FP32 steps in pairs wherever it can: it is bound by HBM, and a
+// pair halves the traffic (five 2048 x 1024 lattices 22.9 -> 13.0 us per step
+// each, one 512 x 256 lattice 7.3 -> 3.9).  16-bit storage already reads half
+// as much and is bound by its arithmetic once the GPU is full, where the rim
+// that a pair recomputes costs what the traffic saves (the serving mix of
+// five sizes, FP16 stochastic: 6.5 us per lattice step singly, 6.6 in pairs with
+// long runs, 7.6 with short ones); alone and up to about 1.5 M nodes the GPU is
+// not full, and half as many launches win (512 x 256: 9.7 -> 4.4 us, 1024 x 512:
+// 10.2 -> 7.0, 1536 x 768: 12.2 -> 10.7, 2048 x 1024: 16.5 -> 16.6).
+constexpr int64_t kPair16Nodes = 1500000;
+constexpr int64_t kPairBatchNodes = 4000000;  // a full GPU: longer runs
+void choose_mode(vplbm_ctx *c, int64_t call_nodes) {
+  const int64_t own = (int64_t)c->L.nx * c->L.ny;
+  if (!c->pair_ok || (elem_bytes(c->cfg.dtype) == 2 && call_nodes > kPair16Nodes))
+    c->mode = kSingle;
+  else
+    c->mode = call_nodes >= 2 * own && call_nodes > kPairBatchNodes ? kPairBatch : kPairAlone;
+}
+// ... for a lattice stepped by itself
+void choose_mode(vplbm_ctx *c) { choose_mode(c, (int64_t)c->L.nx * c->L.ny); }
 
 bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
 // the longest captured graph from buffer cur that fits in `left` steps
 int graph_length_from(const vplbm_ctx *c, int cur, int left) {
   for (int n = std::min(left, kGraphMax); n > 1; --n)
-    if (c->graphs[cur][n]) return n;
+    if (c->graphs[c->mode][cur][n]) return n;
   return 1;
 }
 
@@ -480,7 +611,7 @@ int graph_length(const vplbm_ctx *c, int left) {
 // one, so that later runs of any length find theirs; each is uploaded on the
 // stream s that will launch it.
 vplbm_status ensure_graphs(vplbm_ctx *c, cudaStream_t s) {
-  if (c->graphs_ready) return VPLBM_OK;
+  if (c->graphs_ready[c->mode]) return VPLBM_OK;
   VPLBM_CUDA(c, flush_forces(c, s));  // the graphs start with nothing pending
   if (!c->capture_stream)
     VPLBM_CUDA(c, cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking));
@@ -490,14 +621,20 @@ vplbm_status ensure_graphs(vplbm_ctx *c, cudaStream_t s) {
   for (int n = 1; n <= kGraphMax; ++n) {
     if (!is_pow2(n) && !c->graph_wanted[n]) continue;
     for (int p = 0; p < 2; ++p) {
-      if (c->graphs[p][n]) continue;
+      if (c->graphs[c->mode][p][n]) continue;
       cudaGraph_t g = nullptr;
       VPLBM_CUDA(c, cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeThreadLocal));
       cudaError_t e = cudaSuccess;
       const int cur = c->cur;
-      c->cur = (p + n) & 1;  // the level the graph ends at, for the end-of-run work
-      for (int q = 0; q < n && e == cudaSuccess; ++q)
-        e = queue_step(c, c->capture_stream, (p + q) & 1, false, do_sim);
+      c->cur = buffer_after(c, p, n);  // where the graph ends, for the end-of-run work
+      for (int q = 0, u = p; q < n && e == cudaSuccess; u ^= 1)
+        if (c->mode != kSingle && n - q >= 2) {
+          e = queue_pair(c, c->capture_stream, u, do_sim);
+          q += 2;
+        } else {
+          e = queue_step(c, c->capture_stream, u, false, do_sim);
+          ++q;
+        }
       if (e == cudaSuccess) e = flush_forces(c, c->capture_stream);
       if (e == cudaSuccess) e = refresh_mask(c, c->capture_stream);
       c->cur = cur;
@@ -513,21 +650,21 @@ vplbm_status ensure_graphs(vplbm_ctx *c, cudaStream_t s) {
         drop_graphs(c);
         return cuda_fail(c, e2, "cudaStreamEndCapture");
       }
-      e = cudaGraphInstantiate(&c->graphs[p][n], g, 0);
-      c->graph_defs[p][n] = g;
+      e = cudaGraphInstantiate(&c->graphs[c->mode][p][n], g, 0);
+      c->graph_defs[c->mode][p][n] = g;
       if (e != cudaSuccess) {
-        c->graphs[p][n] = nullptr;
+        c->graphs[c->mode][p][n] = nullptr;
         drop_graphs(c);
         return cuda_fail(c, e, "cudaGraphInstantiate");
       }
-      e = cudaGraphUpload(c->graphs[p][n], s);  // so that its first launch does not pay for it
+      e = cudaGraphUpload(c->graphs[c->mode][p][n], s);  // so that its first launch does not pay for it
       if (e != cudaSuccess) {
         drop_graphs(c);
         return cuda_fail(c, e, "cudaGraphUpload");
       }
     }
   }
-  c->graphs_ready = true;
+  c->graphs_ready[c->mode] = true;
   return VPLBM_OK;
 }
 
@@ -543,10 +680,10 @@ vplbm_status run_steps(vplbm_ctx *c, cudaStream_t s, int nsteps) {
       VPLBM_CUDA(c, flush_forces(c, s));  // a graph starts with nothing pending
       if (vplbm_status st = ensure_graphs(c, s)) return st;
       const int n = graph_length(c, left);
-      VPLBM_CUDA(c, cudaGraphLaunch(c->graphs[c->cur][n], s));
-      c->launches += 2 * n + 1 + (c->body_host.moving ? 1 : 0);
+      VPLBM_CUDA(c, cudaGraphLaunch(c->graphs[c->mode][c->cur][n], s));
+      c->launches += graph_launches(c, n);
       c->steps += n;
-      c->cur ^= n & 1;
+      c->cur = buffer_after(c, c->cur, n);
       c->pending = false;
       c->mask_stale = false;  // the graph ends with the mask refreshed
       left -= n;
@@ -638,6 +775,7 @@ vplbm_status vplbm_create(const vplbm_config *cfg, void *dev_workspace, size_t b
   c->chi = (uint8_t *)(c->ws + lay.chi);
   c->sim_pts = (SimPoint *)(c->ws + lay.sim_pts);
   c->acc = (unsigned long long *)(c->ws + lay.acc);
+  c->acc2 = (unsigned long long *)(c->ws + lay.acc2);
   c->rng = (unsigned long long *)(c->ws + lay.rng);
   c->sim_nodes = (int32_t *)(c->ws + lay.sim_nodes);
   c->hist = (double *)(c->ws + lay.hist);
@@ -830,14 +968,18 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   const int new_slots = std::max(1, slots);
   const int new_every = (b->moving && b->estimator == VPLBM_SIM) ? 1 : c->cfg.sim_every;
   const double new_const[3] = {cfx, cfy, ctq};
+  const PairPlan plan = pair_plan(c, *b, pts);
   const bool keep_graphs = c->has_body && c->n_sim == n_sim && c->region_slots == new_slots &&
                            c->body_host.moving == bs.moving && c->sim_every == new_every &&
+                           c->pair_ok == plan.ok && std::memcmp(c->box, plan.box, sizeof(plan.box)) == 0 &&
                            std::memcmp(c->sim_const, new_const, sizeof(new_const)) == 0;
   c->sim_const[0] = cfx;
   c->sim_const[1] = cfy;
   c->sim_const[2] = ctq;
   c->body_cfg = *b;
   c->body_host = bs;
+  c->pair_ok = plan.ok;
+  std::memcpy(c->box, plan.box, sizeof(plan.box));
   c->region_slots = new_slots;
   c->n_sim = n_sim;
   c->sim_every = new_every;
@@ -892,6 +1034,7 @@ vplbm_status vplbm_step(vplbm_ctx *c, int32_t nsteps) {
   if (!c) return fail(nullptr, VPLBM_EINVAL, "ctx is NULL");
   if (nsteps < 0) return fail(c, VPLBM_EINVAL, "nsteps must be >= 0");
   if (!c->has_body) return fail(c, VPLBM_ESTATE, "no body placed (vplbm_set_body)");
+  choose_mode(c);
   return run_steps(c, c->stream, nsteps);
 }
 
@@ -905,7 +1048,7 @@ bool want_length(vplbm_ctx *c, int nsteps) {
   const int r = nsteps > kGraphMax ? nsteps % kGraphMax : nsteps;
   if (r <= 1 || is_pow2(r) || c->graph_wanted[r]) return false;
   c->graph_wanted[r] = true;
-  c->graphs_ready = false;  // ensure_graphs captures the missing lengths only
+  for (bool &ready : c->graphs_ready) ready = false;  // ensure_graphs captures the missing lengths only
   return true;
 }
 
@@ -920,6 +1063,7 @@ vplbm_status vplbm_prepare(vplbm_ctx *c, int32_t nsteps) {
   if (!c->has_body) return fail(c, VPLBM_ESTATE, "no body placed (vplbm_set_body)");
   want_length(c, nsteps);
   if (c->sim_every > 1) return VPLBM_OK;  // steps are queued one by one
+  choose_mode(c);
   if (vplbm_status st = ensure_graphs(c, c->stream)) return st;
   return sync(c);
 }
@@ -1225,7 +1369,7 @@ constexpr char kSnapMagic[8] = {'V', 'P', 'L', 'B', 'M', 'S', 'N', 'P'};
 constexpr int32_t kSnapVersion = 3;  // 3: SIM points carry their cached walk
 
 size_t snap_header_bytes() { return align_up(sizeof(SnapHeader), 64); }
-size_t snap_tail_bytes(const vplbm_ctx *c) { return c->lay.total - c->lay.prev[0]; }
+size_t snap_tail_bytes(const vplbm_ctx *c) { return c->lay.snap_end - c->lay.prev[0]; }
 size_t snap_pop_bytes(const vplbm_ctx *c) { return 9 * (size_t)c->L.plane * elem_bytes(c->cfg.dtype); }
 
 bool same_config(const vplbm_config &a, const vplbm_config &b) {
@@ -1313,6 +1457,14 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
   c->n_sim = h.n_sim;
   c->sim_every = h.sim_every;
   c->region_slots = h.region_slots;
+  {
+    std::vector<SimPoint> pts;
+    if (h.body_cfg.kind != VPLBM_BODY_NONE && !build_polygon(h.body_cfg, h.n_sim, pts))
+      return fail(c, VPLBM_EINVAL, "corrupt snapshot body");
+    const PairPlan plan = pair_plan(c, h.body_cfg, pts);
+    c->pair_ok = plan.ok;
+    std::memcpy(c->box, plan.box, sizeof(plan.box));
+  }
   c->pending = false;
   c->pending_sim = false;
   c->mask_stale = false;
@@ -1478,10 +1630,17 @@ cudaError_t batch_join(vplbm_batch *b, cudaStream_t s) {
   return e;
 }
 
+// Chooses how each lattice steps in this batch's calls.
+void batch_modes(vplbm_batch *b) {
+  int64_t nodes = 0;
+  for (const vplbm_ctx *c : b->ctxs) nodes += (int64_t)c->L.nx * c->L.ny;
+  for (vplbm_ctx *c : b->ctxs) choose_mode(c, nodes);
+}
+
 // Every lattice replays step graphs (no per-step launches) from where it is.
 bool batch_graphable(const vplbm_batch *b) {
   for (const vplbm_ctx *c : b->ctxs)
-    if (c->sim_every > 1 || c->pre || !c->graphs_ready) return false;
+    if (c->sim_every > 1 || c->pre || !c->graphs_ready[c->mode]) return false;
   return true;
 }
 
@@ -1493,9 +1652,15 @@ void for_pieces(const vplbm_ctx *c, int cur, int n, F piece) {
     for (int r = std::min(left, kGraphMax); r > 0;) {
       const int len = graph_length_from(c, cur, r);
       piece(cur, len);
-      cur ^= len & 1;
+      cur = buffer_after(c, cur, len);
       r -= len;
     }
+}
+
+// the buffer that lattice c's state is in after a batch call of n steps
+int buffer_after_call(const vplbm_ctx *c, int cur, int n) {
+  for_pieces(c, cur, n, [&](int p, int len) { cur = buffer_after(c, p, len); });
+  return cur;
 }
 
 const BatchGraph *find_batch_graph(const vplbm_batch *b, int n) {
@@ -1520,13 +1685,13 @@ vplbm_status build_batch_graph(vplbm_batch *b, int n, const std::vector<int> &cu
     cudaGraphNode_t prev = nullptr;
     for_pieces(c, cur[k], n, [&](int p, int len) {
       if (e != cudaSuccess) return;
-      if (!c->graph_defs[p][len]) {
+      if (!c->graph_defs[c->mode][p][len]) {
         e = cudaErrorInvalidValue;
         return;
       }
       cudaGraphNode_t node = nullptr;
       e = cudaGraphAddChildGraphNode(&node, g, prev ? &prev : nullptr, prev ? 1 : 0,
-                                     c->graph_defs[p][len]);
+                                     c->graph_defs[c->mode][p][len]);
       prev = node;
     });
   }
@@ -1646,6 +1811,7 @@ vplbm_status vplbm_batch_prepare(vplbm_batch *b, int32_t nsteps) {
   Range range_("vplbm_batch_prepare");
   if (!b) return batch_fail(VPLBM_EINVAL, "vplbm_batch_prepare: batch is NULL");
   if (nsteps < 0) return batch_fail(VPLBM_EINVAL, "vplbm_batch_prepare: nsteps must be >= 0");
+  batch_modes(b);
   for (size_t k = 0; k < b->ctxs.size(); ++k) {
     vplbm_ctx *c = b->ctxs[k];
     if (!c->has_body)
@@ -1661,11 +1827,12 @@ vplbm_status vplbm_batch_prepare(vplbm_batch *b, int32_t nsteps) {
   // a call of nsteps steps as one graph launch, from the current buffers and
   // from the other ones (where the lattices stand after an odd step count)
   if (nsteps > 0 && batch_graphable(b)) {
-    std::vector<int> cur;
-    for (const vplbm_ctx *c : b->ctxs) cur.push_back(c->cur);
-    for (int flip = 0; flip < 2; ++flip) {
-      std::vector<int> from(cur);
-      for (int &p : from) p ^= flip;
+    // (a lattice stepped in pairs moves between its buffers at another rate
+    // than one stepped singly: both are also built where a call leaves them)
+    for (int k = 0; k < 4; ++k) {
+      std::vector<int> from;
+      for (const vplbm_ctx *c : b->ctxs)
+        from.push_back((k & 1) ^ (k & 2 ? buffer_after_call(c, c->cur, nsteps) : c->cur));
       bool have = false;
       for (const BatchGraph &bg : b->graphs)
         if (bg.n == nsteps && bg.cur == from) {
@@ -1690,6 +1857,7 @@ vplbm_status vplbm_batch_step(vplbm_batch *b, int32_t nsteps) {
     if (!b->ctxs[k]->has_body)
       return batch_fail(VPLBM_ESTATE, fmt("vplbm_batch_step: lattice %d has no body placed", k));
   if (nsteps == 0) return VPLBM_OK;
+  batch_modes(b);
   cudaStream_t s = b->stream;
   // the batch's work follows what each lattice's own stream holds
   for (int k = 0; k < n; ++k) {
@@ -1710,10 +1878,10 @@ vplbm_status vplbm_batch_step(vplbm_batch *b, int32_t nsteps) {
       for (int k = 0; k < n; ++k) {
         vplbm_ctx *c = b->ctxs[k];
         for_pieces(c, c->cur, nsteps, [&](int, int len) {
-          c->launches += 2 * len + 1 + (c->body_host.moving ? 1 : 0);
+          c->launches += graph_launches(c, len);
         });
         c->steps += nsteps;
-        c->cur ^= nsteps & 1;
+        c->cur = buffer_after_call(c, c->cur, nsteps);
         c->pending = false;
         c->mask_stale = false;
       }

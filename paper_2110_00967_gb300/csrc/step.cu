@@ -48,81 +48,101 @@ struct FixAcc {
   }
 };
 
+// the sum of a 64-bit integer over the warp, by three 32-bit warp reductions
+// of its 24-, 24- and 16-bit pieces (a butterfly takes ten shuffles)
+__device__ __forceinline__ long long warp_sum(long long v) {
+  const unsigned lo = __reduce_add_sync(kFull, (unsigned)v & 0xffffffu);
+  const unsigned mid = __reduce_add_sync(kFull, (unsigned)(v >> 24) & 0xffffffu);
+  const int hi = __reduce_add_sync(kFull, (int)(v >> 48));
+  return (long long)((unsigned long long)lo + ((unsigned long long)mid << 24) +
+                     ((unsigned long long)(long long)hi << 48));
+}
+
 // adds the warp's fixed-point words into acc[slot][word] for the three
 // quantities starting at slot base
 template <typename T>
 __device__ __forceinline__ void warp_add(const FixAcc<T> &a, unsigned long long *acc, int base) {
   constexpr int W = Fix<T>::kWords;
-  long long v[3][W];
   long long any = 0;
 #pragma unroll
   for (int q = 0; q < 3; ++q)
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-      v[q][k] = a.f[q][k];
-      any |= v[q][k];
-    }
+    for (int k = 0; k < W; ++k) any |= a.f[q][k];
   if (!__any_sync(kFull, any != 0)) return;
 #pragma unroll
   for (int q = 0; q < 3; ++q)
 #pragma unroll
-    for (int k = 0; k < W; ++k)
-      for (int o = 16; o > 0; o >>= 1) v[q][k] += __shfl_xor_sync(kFull, v[q][k], o);
-  if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-#pragma unroll
-      for (int k = 0; k < W; ++k)
-        if (v[q][k]) atomicAdd(acc + 2 * (base + q) + k, (unsigned long long)v[q][k]);
-  }
+    for (int k = 0; k < W; ++k) {
+      const long long v = warp_sum(a.f[q][k]);
+      if ((threadIdx.x & 31) == 0 && v) atomicAdd(acc + 2 * (base + q) + k, (unsigned long long)v);
+    }
 }
+
+// the nine populations of a node, passed by value
+template <typename T>
+struct Offsets {
+  T h[9];
+};
 
 // ---------------------------------------------------------------------------
 // SIM (Sec. 2.3.2)
 // ---------------------------------------------------------------------------
 
+// The SIM terms are written with named roundings, so that a state gives the
+// same bits in a single step and in either step of a pair, whatever the
+// compiler would fuse around them.
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float rrcp(float a) { return __frcp_rn(a); }
+__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double rrcp(double a) { return __drcp_rn(a); }
+
 // The part of the stress beyond -(1/3) I at a fluid node,
 // sigma + (1/3) I = -(rho - 1)/3 I - (1 - 1/(2 tau+)) sum c c (f - feq),
-// from its pre-collision offsets, in the compute type (all terms are small;
-// f - feq = h - heq, with heq the equilibrium's offset as in collide()).
-template <typename S, bool kGather>
-__device__ __forceinline__ void node_stress(const S *buf, const typename Store<S>::T *prev,
-                                            const Lattice &L, const Consts<typename Store<S>::T> &c,
-                                            int i, int j, typename Store<S>::T sig[3]) {
-  using T = typename Store<S>::T;
-  T h[9];
-#pragma unroll
-  for (int a = 0; a < 9; ++a) h[a] = pre_pop<S, kGather>(buf, prev, L, a, i, j);
-  T drho = 0, jx = 0, jy = 0;
-#pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    drho += h[a];
-    jx += (T)cx_of(a) * h[a];
-    jy += (T)cy_of(a) * h[a];
-  }
-  const T rho = (T)1 + drho;
-  const T inv = (T)1 / rho;
-  const T dux = (jx + (T)0.5 * lat_bf<T>(L, 0) - drho * c.urx) * inv;
-  const T duy = (jy + (T)0.5 * lat_bf<T>(L, 1) - drho * c.ury) * inv;
-  const T ux = c.urx + dux, uy = c.ury + duy, uu = ux * ux + uy * uy;
-  const T dsu = dux * (ux + c.urx) + duy * (uy + c.ury);
-  T pxx = 0, pxy = 0, pyy = 0;
-#pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    const T cu = (T)cx_of(a) * ux + (T)cy_of(a) * uy;
-    const T cdu = (T)cx_of(a) * dux + (T)cy_of(a) * duy;
-    const T csu = cu + ((T)cx_of(a) * c.urx + (T)cy_of(a) * c.ury);
-    const T heq = (T)w_of(a) * (drho * ((T)1 + (T)3 * cu + (T)4.5 * cu * cu - (T)1.5 * uu) +
-                                (T)3 * cdu + (T)4.5 * cdu * csu - (T)1.5 * dsu);
-    const T d = h[a] - heq;
-    pxx += (T)(cx_of(a) * cx_of(a)) * d;
-    pxy += (T)(cx_of(a) * cy_of(a)) * d;
-    pyy += (T)(cy_of(a) * cy_of(a)) * d;
-  }
-  sig[0] = -drho / (T)3 - c.sim_s * pxx;
-  sig[1] = -c.sim_s * pxy;
-  sig[2] = -drho / (T)3 - c.sim_s * pyy;
+// from its pre-collision offsets h, in the compute type (all terms are small).
+// The second moment of the equilibrium's offset is (rho - 1)/3 I plus
+// rho u u - u_ref u_ref, three products as in collide(), so the sum over the
+// populations needs only the offsets' own second moment (about 40 operations
+// where summing c c (h_a - heq_a) took 200: FP64's SIM blocks were bound by it).
+template <typename T>
+struct Stress {
+  T xx, xy, yy;
+};
+template <typename T>
+__device__ __forceinline__ Stress<T> stress_of(const Offsets<T> &f, const StepArgs &p) {
+  const Lattice &L = p.L;
+  const Consts<T> c(p);
+  const T(&h)[9] = f.h;
+  const T s1 = radd(h[1], h[3]), s2 = radd(h[2], h[4]), s5 = radd(h[5], h[7]), s6 = radd(h[6], h[8]);
+  const T d5 = radd(h[5], -h[7]), d6 = radd(h[6], -h[8]), diag = radd(s5, s6);
+  const T drho = radd(radd(h[0], radd(s1, s2)), diag);
+  const T djx = rfma((T)0.5, lat_bf<T>(L, 0), radd(radd(h[1], -h[3]), radd(d5, -d6)));
+  const T djy = rfma((T)0.5, lat_bf<T>(L, 1), radd(radd(h[2], -h[4]), radd(d5, d6)));
+  const T inv = rrcp(radd((T)1, drho));
+  const T dux = rmul(rfma(drho, -c.urx, djx), inv), duy = rmul(rfma(drho, -c.ury, djy), inv);
+  const T ux = radd(c.urx, dux), uy = radd(c.ury, duy);
+  const T third = rmul(drho, (T)(1.0 / 3.0));
+  const T pxx = radd(radd(radd(s1, diag), -third), -rfma(djx, ux, rmul(c.urx, dux)));
+  const T pyy = radd(radd(radd(s2, diag), -third), -rfma(djy, uy, rmul(c.ury, duy)));
+  const T pxy = radd(radd(s5, -s6), -rfma(djx, uy, rmul(c.urx, duy)));
+  return Stress<T>{rfma(-c.sim_s, pxx, -third), rmul(-c.sim_s, pxy), rfma(-c.sim_s, pyy, -third)};
 }
+
+// the pre-collision offsets of node (i, j) of the level that buf holds
+template <typename S, bool kGather>
+struct FieldNode {
+  const S *buf;
+  const typename Store<S>::T *prev;
+  const Lattice &L;
+  __device__ __forceinline__ void operator()(int i, int j,
+                                             Offsets<typename Store<S>::T> &f) const {
+#pragma unroll
+    for (int a = 0; a < 9; ++a) f.h[a] = pre_pop<S, kGather>(buf, prev, L, a, i, j);
+  }
+};
 
 // mask byte of node (i, j) (inside the lattice) as SIM and MEM see it: chi,
 // or for a moving body the predicate of Eq. fcar on the current body, since
@@ -204,60 +224,80 @@ __global__ void sim_cache_kernel(const StepArgs p) {
   sp->n_cand = n;
 }
 
-// One SIM integration point: its sampled nodes (walked now, or for a fixed
-// body found when it was placed), the stress averaged over them, then
-// S (sigma + I/3) n and its moment; the -(1/3) S n part sums to a constant of
-// the polygon added in the tail.
-template <typename S, bool kGather>
-__device__ __noinline__ FixAcc<typename Store<S>::T> sim_point(const StepArgs &p, const S *buf, double bxg, double byg,
-                                         int q, bool &missing) {
-  using T = typename Store<S>::T;
-  const SimPoint sp = p.sim_pts[q];
-  uint32_t cand[4] = {sp.cand[0], sp.cand[1], sp.cand[2], sp.cand[3]};
-  const int n = sp.n_cand >= 0 ? sp.n_cand : sim_candidates(p, sp, bxg, byg, cand);
-  const T *prev = static_cast<const T *>(p.prev_src);
+// S (sigma + I/3) n and its moment of SIM point sp, from the stress summed over
+// its n sampled nodes
+template <typename T>
+__device__ __forceinline__ FixAcc<T> sim_sum(const SimPoint &sp, const Stress<T> sig, int n) {
+  FixAcc<T> r;
+  // mean over 1, 2 or 4 candidates: an exact power-of-two scaling
+  const T inv = (n == 1) ? (T)1 : ((n == 2) ? (T)0.5 : (T)0.25);
+  T dx, dy, nx, ny, sl;
+  sim_geom<T>(sp, dx, dy, nx, ny, sl);
+  const T sxx = rmul(sig.xx, inv), sxy = rmul(sig.xy, inv), syy = rmul(sig.yy, inv);
+  const T tx = rmul(sl, rfma(sxx, nx, rmul(sxy, ny)));
+  const T ty = rmul(sl, rfma(sxy, nx, rmul(syy, ny)));
+  r.add(0, tx);
+  r.add(1, ty);
+  r.add(2, rfma(dx, ty, -rmul(dy, tx)));
+  return r;
+}
+
+// The stress at SIM point sp extrapolated linearly along its sampling direction
+// from the sampled node (qi, qj) and the next one (sim_order 1)
+template <typename T>
+__device__ __forceinline__ Stress<T> extrapolate(const SimPoint &sp, double bxg, double byg, int qi,
+                                              int qj, Stress<T> s3, const Stress<T> next) {
+  const double x = bxg + sp.dx, y = byg + sp.dy;
+  const int c2 = cx_of(sp.dir) * cx_of(sp.dir) + cy_of(sp.dir) * cy_of(sp.dir);
+  const T t = (T)(((x - qi) * cx_of(sp.dir) + (y - qj) * cy_of(sp.dir)) / (double)c2);
+  s3.xx = rfma(t, radd(next.xx, -s3.xx), s3.xx);
+  s3.xy = rfma(t, radd(next.xy, -s3.xy), s3.xy);
+  s3.yy = rfma(t, radd(next.yy, -s3.yy), s3.yy);
+  return s3;
+}
+
+// The force terms of SIM point sp from its n sampled nodes cand; node(i, j, f) gives the pre-collision offsets
+// of a node at the step's level.  The -(1/3) S n part sums to a constant of
+// the polygon added when the sums are finalized.
+template <typename T, typename Node>
+__device__ __forceinline__ FixAcc<T> sim_terms(const StepArgs &p, const SimPoint &sp, double bxg,
+                                               double byg, const uint32_t (&cand)[4], int n,
+                                               const Node &node) {
   T sig[3] = {0, 0, 0};
-  int first = -1;
-  const bool ok = n > 0;
   for (int k = 0; k < n; ++k) {
     const int qi = (int)(cand[k] & 0xffffu), qj = (int)(cand[k] >> 16);
-    if (first < 0) first = qj * p.L.nx + qi;
-    T s3[3];
-    node_stress<S, kGather>(buf, prev, p.L, Consts<T>(p), qi, qj, s3);
+    Offsets<T> f;
+    node(qi, qj, f);
+    Stress<T> s3 = stress_of<T>(f, p);
     if (p.sim_order == 1) {
       // first order: extrapolated to the point along the direction from
       // the next node, where that node is fluid and inside the lattice
       const int ni = qi + cx_of(sp.dir), nj = qj + cy_of(sp.dir);
       if (ni >= 0 && ni < p.L.nx && nj >= 0 && nj < p.L.ny && !(solid_at(p, ni, nj) & kSolid)) {
-        T s3n[3];
-        node_stress<S, kGather>(buf, prev, p.L, Consts<T>(p), ni, nj, s3n);
-        const double x = bxg + sp.dx, y = byg + sp.dy;
-        const int c2 = cx_of(sp.dir) * cx_of(sp.dir) + cy_of(sp.dir) * cy_of(sp.dir);
-        const T t = (T)(((x - qi) * cx_of(sp.dir) + (y - qj) * cy_of(sp.dir)) / (double)c2);
-        s3[0] += t * (s3n[0] - s3[0]);
-        s3[1] += t * (s3n[1] - s3[1]);
-        s3[2] += t * (s3n[2] - s3[2]);
+        node(ni, nj, f);
+        s3 = extrapolate<T>(sp, bxg, byg, qi, qj, s3, stress_of<T>(f, p));
       }
     }
-    sig[0] += s3[0];
-    sig[1] += s3[1];
-    sig[2] += s3[2];
+    sig[0] = radd(sig[0], s3.xx);
+    sig[1] = radd(sig[1], s3.xy);
+    sig[2] = radd(sig[2], s3.yy);
   }
-  p.sim_nodes[q] = ok ? first : -1;
-  missing = !ok;
-  FixAcc<T> r;
-  if (!ok) return r;
-  // mean over 1, 2 or 4 candidates: an exact power-of-two scaling
-  const T inv = (n == 1) ? (T)1 : ((n == 2) ? (T)0.5 : (T)0.25);
-  T dx, dy, nx, ny, sl;
-  sim_geom<T>(sp, dx, dy, nx, ny, sl);
-  const T sxx = sig[0] * inv, sxy = sig[1] * inv, syy = sig[2] * inv;
-  const T tx = sl * (sxx * nx + sxy * ny);
-  const T ty = sl * (sxy * nx + syy * ny);
-  r.add(0, tx);
-  r.add(1, ty);
-  r.add(2, dx * ty - dy * tx);
-  return r;
+  return n > 0 ? sim_sum<T>(sp, Stress<T>{sig[0], sig[1], sig[2]}, n) : FixAcc<T>();
+}
+
+// One SIM integration point: its sampled nodes (walked now, or for a fixed
+// body found when it was placed) and its force terms.
+template <typename S, bool kGather>
+__device__ __noinline__ FixAcc<typename Store<S>::T> sim_point(const StepArgs &p, const S *buf, double bxg, double byg,
+                                         int q, bool &missing) {
+  using T = typename Store<S>::T;
+  const SimPoint &sp = p.sim_pts[q];
+  uint32_t cand[4] = {sp.cand[0], sp.cand[1], sp.cand[2], sp.cand[3]};
+  const int n = sp.n_cand >= 0 ? sp.n_cand : sim_candidates(p, sp, bxg, byg, cand);
+  missing = n <= 0;
+  p.sim_nodes[q] = n > 0 ? (int)(cand[0] >> 16) * p.L.nx + (int)(cand[0] & 0xffffu) : -1;
+  return sim_terms<T>(p, sp, bxg, byg, cand, n,
+                      FieldNode<S, kGather>{buf, static_cast<const T *>(p.prev_src), p.L});
 }
 
 // ---------------------------------------------------------------------------
@@ -303,27 +343,51 @@ __device__ __forceinline__ uint8_t tile_mask_byte(const Lattice &L, const TileMa
 // MEM (Sec. 2.3.1)
 // ---------------------------------------------------------------------------
 
+// The links of node (i, j) (bit a: the neighbour along a lies in the lattice and
+// in the other phase), from chi or from the tile's mask when it rasterises its
+// own.  Off the edges the eight bytes are loaded together with the node's own
+// populations: the links' latency is then not added to theirs.
+__device__ __forceinline__ uint32_t node_links(const StepArgs &p, int i, int j, bool solid,
+                                               const TileMask *tm) {
+  const Lattice &L = p.L;
+  const uint8_t self = solid ? kSolid : (uint8_t)0;
+  uint32_t links = 0;
+  if (i > 0 && i < L.nx - 1 && j > 0 && j < L.ny - 1 && !tm) {
+    uint8_t m[9];
+#pragma unroll
+    for (int a = 1; a < 9; ++a) m[a] = p.chi[(int64_t)(j + cy_of(a)) * L.pitch + i + cx_of(a)];
+#pragma unroll
+    for (int a = 1; a < 9; ++a) links |= (uint32_t)((m[a] ^ self) & kSolid) << a;
+    return links;
+  }
+#pragma unroll
+  for (int a = 1; a < 9; ++a) {
+    int ni, nj;
+    if (!neighbour(L, a, i, j, ni, nj)) continue;
+    const uint8_t m = tm ? tm->s[threadIdx.y + 1 + cy_of(a)][threadIdx.x + 1 + cx_of(a)]
+                         : p.chi[(int64_t)nj * L.pitch + ni];
+    links |= (uint32_t)((m ^ self) & kSolid) << a;
+  }
+  return links;
+}
+
 // The link terms of one interface node (Eq. MMEL): for each lattice
 // neighbour of the other phase, the fluid end adds (c_a - u_Gamma) f~_a and
 // the solid end subtracts its own (c_a - u_Gamma) f~_a, with x_Gamma the link
 // midpoint and u_Gamma the rigid velocity there; torques about the reference
 // point (Eq. fluidtorque).  f~ = h~ + E is split so that the E parts, which
-// cancel in pairs around a fixed body, are rounded exactly.  The neighbours'
-// phases come from chi, or from the tile's mask when it rasterises its own.
+// cancel in pairs around a fixed body, are rounded exactly.
 template <typename T>
-__device__ __forceinline__ void mem_terms(const StepArgs &p, const T (&o)[9], int i, int j,
-                                          uint8_t m, const TileMask *tm, FixAcc<T> &acc) {
+__device__ __forceinline__ FixAcc<T> mem_terms(const StepArgs &p, const Offsets<T> post, int i, int j,
+                                            bool solid, uint32_t links) {
+  const T(&o)[9] = post.h;
+  FixAcc<T> acc;
   const Lattice &L = p.L;
   const BodyRef<T> b(*p.body_src);
-  const bool solid = m & kSolid;
   const T sg = solid ? (T)-1 : (T)1;
 #pragma unroll
   for (int a = 1; a < 9; ++a) {
-    int ni, nj;
-    if (!neighbour(L, a, i, j, ni, nj)) continue;
-    const bool nsolid = tm ? (tm->s[threadIdx.y + 1 + cy_of(a)][threadIdx.x + 1 + cx_of(a)] & kSolid)
-                           : (p.chi[(int64_t)nj * L.pitch + ni] & kSolid);
-    if (nsolid == solid) continue;
+    if (!(links >> a & 1u)) continue;
     const T rx = ((T)i - b.xg) + (T)(0.5 * cx_of(a));
     const T ry = ((T)j - b.yg) + (T)(0.5 * cy_of(a));
     const T vx = (T)cx_of(a) - (b.ux - b.om * ry);
@@ -337,6 +401,20 @@ __device__ __forceinline__ void mem_terms(const StepArgs &p, const T (&o)[9], in
     acc.add(2, rx * lyh - ry * lxh);
     acc.add(2, rx * lyw - ry * lxw);
   }
+  return acc;
+}
+
+// The volume-integral terms of one solid node (Eq. Angotforce, reading R19):
+// the penalization force (pen_x, pen_y) on the fluid, reversed, and its moment
+// about the reference point.
+template <typename T>
+__device__ __forceinline__ FixAcc<T> vol_terms(const BodyRef<T> b, int i, int j, T pen_x, T pen_y) {
+  FixAcc<T> vol;
+  const T fx = -pen_x, fy = -pen_y;
+  vol.add(0, fx);
+  vol.add(1, fy);
+  vol.add(2, ((T)i - b.xg) * fy - ((T)j - b.yg) * fx);
+  return vol;
 }
 
 // ---------------------------------------------------------------------------
@@ -362,41 +440,53 @@ __device__ void rigid_update(BodyState &b, const double F[3]) {
   body_sync_f32(b);
 }
 
-// Force bookkeeping of a step whose tail was deferred (a fixed body): its
-// fixed-point sums (acc) become the step's history row and are added to the
-// running sums; the step counter advances and acc is cleared for reuse two
-// steps later.  Runs in one block beside the next step's work, or alone at
-// the end of a call.  Loads are spread over threads and issued together.
+// Force bookkeeping of a launch whose tail was deferred (a fixed body): the
+// fixed-point sums of its step, or of the two steps of a pair, become the
+// steps' history rows and are added to the running sums in step order; the
+// step counter advances and the sums are cleared for reuse two launches later.
+// Runs in one block beside the next launch's work, or alone at the end of a
+// call.  Loads are spread over threads and issued together.
 template <typename T>
-__device__ void finalize(const StepArgs &p, unsigned long long *acc) {
+__device__ void finalize(const StepArgs &p) {
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  __shared__ double tot[kAccSlots];
+  const int rows = p.prev_rows;
+  __shared__ double tot[2][kAccSlots];
   __shared__ long long step_s;
   const bool do_sim = p.prev_sim != 0;
-  if (tid < kAccSlots) {
-    const long long w0 = (long long)__ldcg(acc + 2 * tid);
-    const long long w1 = (long long)__ldcg(acc + 2 * tid + 1);
+  const int row = tid >> 5, col = tid & 31;  // warps 0 and 1: the rows
+  if (row < rows && col < kAccSlots) {
+    const unsigned long long *acc = row ? p.acc2_prev : p.acc_prev;
+    const long long w0 = (long long)__ldcg(acc + 2 * col);
+    const long long w1 = (long long)__ldcg(acc + 2 * col + 1);
     double v = Fix<T>::value(w0, w1);
-    if (tid >= 3 && tid < 6) v += p.sim_const[tid - 3];
-    tot[tid] = v;
+    if (col >= 3 && col < 6) v += p.sim_const[col - 3];
+    tot[row][col] = v;
   } else if (tid == 64) {
     step_s = __ldcg(p.dev_step);
   }
   __syncthreads();
-  if (tid < kHistCols) {
+  if (row < rows && col < kHistCols) {
     // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
-    const bool have = tid < 3 || tid >= 6 || do_sim;
-    p.hist[kHistCols * (step_s % p.hist_len) + tid] =
-        have ? tot[tid] : __longlong_as_double(0x7ff8000000000000LL);
-    if (have && tid < 6) p.sums[tid] += tot[tid];
-  } else if (tid == 16) {
-    p.counts[0] += 1;
-  } else if (tid == 17 && do_sim) {
-    p.counts[1] += 1;
-  } else if (tid == 32) {
-    *p.dev_step = step_s + 1;
+    const bool have = col < 3 || col >= 6 || do_sim;
+    p.hist[kHistCols * ((step_s + row) % p.hist_len) + col] =
+        have ? tot[row][col] : __longlong_as_double(0x7ff8000000000000LL);
   }
-  if (tid < kAccWords) acc[tid] = 0ull;  // every read of acc above precedes the barrier
+  if (tid >= 64 && tid < 64 + 6) {
+    const int q = tid - 64;
+    if (q < 3 || do_sim) {
+      double v = p.sums[q] + tot[0][q];
+      if (rows > 1) v += tot[1][q];
+      p.sums[q] = v;
+    }
+  } else if (tid == 80) {
+    p.counts[0] += rows;
+  } else if (tid == 81 && do_sim) {
+    p.counts[1] += rows;
+  } else if (tid == 96) {
+    *p.dev_step = step_s + rows;
+  }
+  // every read of the sums above precedes the barrier
+  if (row < rows && col < kAccWords) (row ? p.acc2_prev : p.acc_prev)[col] = 0ull;
 }
 
 // The last participating block: the step's forces from the fixed-point sums
@@ -809,7 +899,7 @@ struct NodeVal<double> {
 // the collision; a fluid node gets the same bits as from the bulk kernels.
 // (pen_x, pen_y): the penalization part of G (solid nodes only).  Returns true
 // for a non-finite or non-positive density.
-template <typename S, typename T>
+template <typename S, bool kForce, typename T>
 __device__ __forceinline__ bool update_node(const T (&h)[9], uint8_t mask, int i, int j,
                                             const Lattice &L, const BodyState *body,
                                             const Consts<T> &cst, T (&o)[9], T &pen_x,
@@ -821,7 +911,7 @@ __device__ __forceinline__ bool update_node(const T (&h)[9], uint8_t mask, int i
 #pragma unroll
   for (int a = 0; a < 9; ++a) hv[a] = Val<V>::splat(h[a]);
   if (!(mask & kSolid)) {
-    rho = L.has_bf ? update_fluid<S, true>(L, cst, hv, ov) : update_fluid<S, false>(L, cst, hv, ov);
+    rho = update_fluid<S, kForce>(L, cst, hv, ov);
   } else {
     const Moments<V> m(hv);
     V drho = m.drho, jx = m.djx, jy = m.djy;
@@ -866,8 +956,8 @@ __device__ __forceinline__ bool update_node(const T (&h)[9], uint8_t mask, int i
 // ---------------------------------------------------------------------------
 // hash of the level being written: the rounding counter, which the special
 // kernel advances by one per step
-__device__ __forceinline__ uint32_t sr_level(const StepArgs &p) {
-  const unsigned long long n = __ldg(p.rng_src);
+__device__ __forceinline__ uint32_t sr_level(const StepArgs &p, int step = 0) {
+  const unsigned long long n = __ldg(p.rng_src) + (unsigned long long)step;
   return pcg_hash((uint32_t)n ^ (uint32_t)(n >> 32));
 }
 
@@ -960,8 +1050,14 @@ __device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bo
   } else {
     m = p.chi[node];
   }
+  // FP64's long update hides the links' loads; elsewhere only interface nodes
+  // look for theirs
+  const uint32_t links = in_reg && ((sizeof(S) == 8 && !tm) || (m & kInterface))
+                             ? node_links(p, i, j, m & kSolid, tm)
+                             : 0u;
   T o[9], pen_x, pen_y;
-  const bool bad = update_node<S>(h, m, i, j, L, p.body_src, Consts<T>(p), o, pen_x, pen_y);
+  const bool bad = L.has_bf ? update_node<S, true>(h, m, i, j, L, p.body_src, Consts<T>(p), o, pen_x, pen_y)
+                            : update_node<S, false>(h, m, i, j, L, p.body_src, Consts<T>(p), o, pen_x, pen_y);
   if (sizeof(S) == 2 && p.sr) {
     const SrBits r(sr_level(p), (uint32_t)node >> 1);
 #pragma unroll
@@ -972,16 +1068,13 @@ __device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bo
     for (int a = 0; a < 9; ++a)
       store_pop<S, false>(dst + (int64_t)a * L.plane + node, o[a], nullptr, a, (uint32_t)node);
   }
-  if (in_reg && (m & kInterface)) mem_terms<T>(p, o, i, j, m, tm, acc);
-  if (in_reg && (m & kSolid)) {
-    // volume integral (Eq. Angotforce, reading R19): the penalization force
-    // on the fluid, reversed, and its moment about the reference point
-    const BodyRef<T> b(*p.body_src);
-    const T fx = -pen_x, fy = -pen_y;
-    vol.add(0, fx);
-    vol.add(1, fy);
-    vol.add(2, ((T)i - b.xg) * fy - ((T)j - b.yg) * fx);
+  if (links) {
+    Offsets<T> post;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) post.h[a] = o[a];
+    acc = mem_terms<T>(p, post, i, j, m & kSolid, links);
   }
+  if (in_reg && (m & kSolid)) vol = vol_terms<T>(BodyRef<T>(*p.body_src), i, j, pen_x, pen_y);
   return bad;
 }
 
@@ -1010,7 +1103,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) special_kernel(const Ste
   if (p.sr && b == 0 && tid == 0) *p.rng_dst = *p.rng_src + 1ull;  // the next level's counter
   if (p.finalize_prev && b == (int)gridDim.x - 1) {
     // the previous step's force sums, beside this step's work
-    finalize<T>(p, p.acc_prev);
+    finalize<T>(p);
     return;
   }
 
@@ -1414,6 +1507,8 @@ __global__ void __launch_bounds__(32 * kTileY, 12) bulk16x4_kernel(const StepArg
   if (bad) atomicOr(p.status, kStatusUnstable);
 }
 
+#include "pair.cuh"
+
 template <typename S, bool kGather>
 cudaError_t special_t(const StepArgs &a, cudaStream_t s) {
   const int tiles = a.all_tiles ? a.ntiles_x * a.ntiles_y : a.edge_blocks + a.region_slots;
@@ -1427,7 +1522,7 @@ cudaError_t special_t(const StepArgs &a, cudaStream_t s) {
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads) finalize_kernel(const StepArgs p) {
-  finalize<T>(p, p.acc_prev);
+  finalize<T>(p);
 }
 
 // chi of a moving body on the force-region tiles, tile by tile as the special
@@ -1495,6 +1590,15 @@ cudaError_t launch_special(int dtype, bool gather, const StepArgs &a, cudaStream
     case VPLBM_F16_OFS: return gather ? special_t<__half, true>(a, s) : special_t<__half, false>(a, s);
     case VPLBM_BF16_OFS:
       return gather ? special_t<__nv_bfloat16, true>(a, s) : special_t<__nv_bfloat16, false>(a, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_pair(int dtype, const StepArgs &a, cudaStream_t s) {
+  switch (dtype) {
+    case VPLBM_F32: return pair_t<float>(a, s);
+    case VPLBM_F16_OFS: return pair_t<__half>(a, s);
+    case VPLBM_BF16_OFS: return pair_t<__nv_bfloat16>(a, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -11,6 +11,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <string>
+#include <type_traits>
 
 #include "vplbm.h"
 
@@ -293,26 +294,42 @@ __device__ __forceinline__ typename Store<S>::T pop_at(const S *post, const Latt
   return Store<S>::ld(post + (int64_t)a * L.plane + (int64_t)j * L.pitch + i);
 }
 
+// The source of population a at node (i, j), side conditions included, read
+// through src(a, i, j), whose coordinates may lie beyond a periodic side (the
+// accessor wraps them: a global field, or a tile in shared memory).
+template <typename T, typename Src>
+__device__ __forceinline__ T gather_from(const Src &src, const Lattice &L, int a, int i, int j) {
+  const int si = i - cx_of(a), sj = j - cy_of(a);
+  const bool xin = (si >= 0 || L.bc[0] == VPLBM_PERIODIC) && (si < L.nx || L.bc[1] == VPLBM_PERIODIC);
+  const bool yin = (sj >= 0 || L.bc[2] == VPLBM_PERIODIC) && (sj < L.ny || L.bc[3] == VPLBM_PERIODIC);
+  if (xin && yin) return src(a, si, sj);
+  if (!xin) {
+    const int kind = L.bc[si < 0 ? 0 : 1];
+    if (kind == VPLBM_INLET_BB) return src(opp_of(a), i, j) + LatC<T>::kin(L, a);
+    return src(opp_of(a), i, j) + LatC<T>::knos(L, a);  // no-slip bounce-back
+  }
+  const int kind = L.bc[sj < 0 ? 2 : 3];
+  if (kind == VPLBM_SYMMETRY) return src(flipy_of(a), si, j) + LatC<T>::ksym(L, a);
+  return src(opp_of(a), i, j) + LatC<T>::knos(L, a);  // no-slip bounce-back
+}
+
+// wraps a coordinate at most one period outside [0, n)
+__device__ __forceinline__ int wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+
+// a stored field in global memory
+template <typename S>
+struct FieldSrc {
+  const S *post;
+  const Lattice &L;
+  __device__ __forceinline__ typename Store<S>::T operator()(int a, int i, int j) const {
+    return pop_at(post, L, a, wrap(i, L.nx), wrap(j, L.ny));
+  }
+};
+
 template <typename S>
 __device__ __forceinline__ typename Store<S>::T gather_core(const S *post, const Lattice &L, int a,
                                                              int i, int j) {
-  using T = typename Store<S>::T;
-  int si = i - cx_of(a), sj = j - cy_of(a);
-  if (si < 0 && L.bc[0] == VPLBM_PERIODIC) si += L.nx;
-  if (si >= L.nx && L.bc[1] == VPLBM_PERIODIC) si -= L.nx;
-  if (sj < 0 && L.bc[2] == VPLBM_PERIODIC) sj += L.ny;
-  if (sj >= L.ny && L.bc[3] == VPLBM_PERIODIC) sj -= L.ny;
-  const bool xin = si >= 0 && si < L.nx;
-  const bool yin = sj >= 0 && sj < L.ny;
-  if (xin && yin) return pop_at(post, L, a, si, sj);
-  if (!xin) {
-    const int kind = L.bc[si < 0 ? 0 : 1];
-    if (kind == VPLBM_INLET_BB) return pop_at(post, L, opp_of(a), i, j) + LatC<T>::kin(L, a);
-    return pop_at(post, L, opp_of(a), i, j) + LatC<T>::knos(L, a);  // no-slip bounce-back
-  }
-  const int kind = L.bc[sj < 0 ? 2 : 3];
-  if (kind == VPLBM_SYMMETRY) return pop_at(post, L, flipy_of(a), si, j) + LatC<T>::ksym(L, a);
-  return pop_at(post, L, opp_of(a), i, j) + LatC<T>::knos(L, a);  // no-slip bounce-back
+  return gather_from<typename Store<S>::T>(FieldSrc<S>{post, L}, L, a, i, j);
 }
 
 __device__ __forceinline__ int outlet_slot(int a) { return a == 3 ? 0 : (a == 6 ? 1 : 2); }
@@ -474,6 +491,14 @@ struct StepArgs {
                             // from body_src themselves, and SIM tests nodes with the
                             // predicate instead of reading chi
   int32_t sr;               // 1: 16-bit stores round stochastically
+  // ---- a pair of steps in one launch (fixed or no body; api.cu: pair_ok) ----
+  unsigned long long *acc2;       // sums of the pair's second step
+  unsigned long long *acc2_prev;  // ... of the previous pair
+  int32_t prev_rows;     // steps that finalize_prev finalizes: 1, or 2 after a pair
+  int32_t box[4];        // i0, i1, j0, j1 (inclusive): nodes around the body that the pair's
+                         // special blocks update; i0 even, i1 odd; i1 < i0: none
+  int32_t pair_rows;     // rows per warp of the bulk blocks
+  int32_t pair_bx;       // bulk blocks side by side (set at the launch)
   const unsigned long long *rng_src;  // the rounding counter of this step's level
   unsigned long long *rng_dst;        // ... and of the next (written by the special kernel)
 };
@@ -628,6 +653,8 @@ cudaError_t launch_sim_cache(const StepArgs &a, cudaStream_t s);
 // eight nodes per thread at 96 or 126 registers, or four nodes per thread
 constexpr int kBulkVariants = 3;
 cudaError_t launch_bulk(int dtype, int variant, const StepArgs &a, cudaStream_t s);
+// two steps of a lattice in one launch (pair.cuh; FP32 compute only)
+cudaError_t launch_pair(int dtype, const StepArgs &a, cudaStream_t s);
 
 // auxiliary kernels (aux.cu)
 cudaError_t launch_raster(const Lattice &L, const BodyState *body, uint8_t *chi, int i0, int j0,
