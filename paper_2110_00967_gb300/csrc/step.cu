@@ -144,18 +144,18 @@ struct FieldNode {
   }
 };
 
-// mask byte of node (i, j) (inside the lattice) as SIM and MEM see it: chi,
-// or for a moving body the predicate of Eq. fcar on the current body, since
+// mask byte of node (i, j) (inside the lattice) as SIM sees it: chi, or for a
+// moving body (a disk; t given) the predicate of Eq. fcar on the current body, since
 // the force-region tiles rewrite chi during the step
-__device__ __forceinline__ uint8_t solid_at(const StepArgs &p, int i, int j) {
-  if (p.raster) return body_contains(*p.body_src, i, j) ? kSolid : (uint8_t)0;
+__device__ __forceinline__ uint8_t solid_at(const StepArgs &p, const NearTest *t, int i, int j) {
+  if (t) return disk_contains(*p.body_src, *t, i, j) ? kSolid : (uint8_t)0;
   return p.chi[(int64_t)j * p.L.pitch + i];
 }
 
 // first fluid node of q_k = (qi, qj) + k c_a, k = 0..3, inside the lattice
 // (the four mask bytes are loaded together)
-__device__ __forceinline__ bool sim_walk(const StepArgs &p, int a, int qi, int qj, int &oi,
-                                         int &oj) {
+__device__ __forceinline__ bool sim_walk(const StepArgs &p, const NearTest *t, int a, int qi,
+                                         int qj, int &oi, int &oj) {
   const Lattice &L = p.L;
   uint8_t m[4];
   bool in[4];
@@ -163,7 +163,7 @@ __device__ __forceinline__ bool sim_walk(const StepArgs &p, int a, int qi, int q
   for (int k = 0; k < 4; ++k) {
     const int ii = qi + k * cx_of(a), jj = qj + k * cy_of(a);
     in[k] = ii >= 0 && ii < L.nx && jj >= 0 && jj < L.ny;
-    m[k] = in[k] ? solid_at(p, ii, jj) : (uint8_t)kSolid;
+    m[k] = in[k] ? solid_at(p, t, ii, jj) : (uint8_t)kSolid;
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -196,8 +196,9 @@ __device__ __forceinline__ void sim_geom<float>(const SimPoint &sp, float &dx, f
 // to the normal to the first fluid node.  Returns their count (1, 2 or 4; 0
 // when a walk finds no fluid node), the nodes packed i | j << 16 in the order
 // the stress sum takes them.
-__device__ __forceinline__ int sim_candidates(const StepArgs &p, const SimPoint &sp, double bxg,
-                                              double byg, uint32_t (&cand)[4]) {
+__device__ __forceinline__ int sim_candidates(const StepArgs &p, const NearTest *t,
+                                              const SimPoint &sp, double bxg, double byg,
+                                              uint32_t (&cand)[4]) {
   const double x = bxg + sp.dx, y = byg + sp.dy;
   const double rx = floor(x + 0.5), ry = floor(y + 0.5);
   const int ncx = (rx == x + 0.5) ? 2 : 1, ncy = (ry == y + 0.5) ? 2 : 1;
@@ -205,7 +206,7 @@ __device__ __forceinline__ int sim_candidates(const StepArgs &p, const SimPoint 
   for (int u = 0; u < ncy; ++u)
     for (int v = 0; v < ncx; ++v) {
       int qi, qj;
-      if (!sim_walk(p, sp.dir, (int)rx - v, (int)ry - u, qi, qj)) return 0;
+      if (!sim_walk(p, t, sp.dir, (int)rx - v, (int)ry - u, qi, qj)) return 0;
       cand[n++] = (uint32_t)qi | ((uint32_t)qj << 16);
     }
   return n;
@@ -218,7 +219,7 @@ __global__ void sim_cache_kernel(const StepArgs p) {
   if (q >= p.n_sim) return;
   SimPoint *sp = const_cast<SimPoint *>(p.sim_pts) + q;
   uint32_t cand[4] = {0u, 0u, 0u, 0u};
-  const int n = sim_candidates(p, *sp, p.body_src->xg, p.body_src->yg, cand);
+  const int n = sim_candidates(p, nullptr, *sp, p.body_src->xg, p.body_src->yg, cand);
 #pragma unroll
   for (int k = 0; k < 4; ++k) sp->cand[k] = cand[k];
   sp->n_cand = n;
@@ -260,8 +261,9 @@ __device__ __forceinline__ Stress<T> extrapolate(const SimPoint &sp, double bxg,
 // of a node at the step's level.  The -(1/3) S n part sums to a constant of
 // the polygon added when the sums are finalized.
 template <typename T, typename Node>
-__device__ __forceinline__ FixAcc<T> sim_terms(const StepArgs &p, const SimPoint &sp, double bxg,
-                                               double byg, const uint32_t (&cand)[4], int n,
+__device__ __forceinline__ FixAcc<T> sim_terms(const StepArgs &p, const NearTest *t,
+                                               const SimPoint &sp, double bxg, double byg,
+                                               const uint32_t (&cand)[4], int n,
                                                const Node &node) {
   T sig[3] = {0, 0, 0};
   for (int k = 0; k < n; ++k) {
@@ -273,7 +275,7 @@ __device__ __forceinline__ FixAcc<T> sim_terms(const StepArgs &p, const SimPoint
       // first order: extrapolated to the point along the direction from
       // the next node, where that node is fluid and inside the lattice
       const int ni = qi + cx_of(sp.dir), nj = qj + cy_of(sp.dir);
-      if (ni >= 0 && ni < p.L.nx && nj >= 0 && nj < p.L.ny && !(solid_at(p, ni, nj) & kSolid)) {
+      if (ni >= 0 && ni < p.L.nx && nj >= 0 && nj < p.L.ny && !(solid_at(p, t, ni, nj) & kSolid)) {
         node(ni, nj, f);
         s3 = extrapolate<T>(sp, bxg, byg, qi, qj, s3, stress_of<T>(f, p));
       }
@@ -293,10 +295,12 @@ __device__ __noinline__ FixAcc<typename Store<S>::T> sim_point(const StepArgs &p
   using T = typename Store<S>::T;
   const SimPoint &sp = p.sim_pts[q];
   uint32_t cand[4] = {sp.cand[0], sp.cand[1], sp.cand[2], sp.cand[3]};
-  const int n = sp.n_cand >= 0 ? sp.n_cand : sim_candidates(p, sp, bxg, byg, cand);
+  const NearTest near(*p.body_src);
+  const NearTest *t = p.raster ? &near : nullptr;  // a moving body: its predicate, not chi
+  const int n = sp.n_cand >= 0 ? sp.n_cand : sim_candidates(p, t, sp, bxg, byg, cand);
   missing = n <= 0;
   p.sim_nodes[q] = n > 0 ? (int)(cand[0] >> 16) * p.L.nx + (int)(cand[0] & 0xffffu) : -1;
-  return sim_terms<T>(p, sp, bxg, byg, cand, n,
+  return sim_terms<T>(p, t, sp, bxg, byg, cand, n,
                       FieldNode<S, kGather>{buf, static_cast<const T *>(p.prev_src), p.L});
 }
 
@@ -313,6 +317,7 @@ struct TileMask {
 __device__ __forceinline__ void tile_solid(const StepArgs &p, int ti, int tj, TileMask &tm) {
   const Lattice &L = p.L;
   const int tid = threadIdx.y * kTileX + threadIdx.x;
+  const NearTest near(*p.body_src);
   for (int q = tid; q < (kTileY + 2) * (kTileX + 2); q += kThreads) {
     const int hx = q % (kTileX + 2), hy = q / (kTileX + 2);
     int gi = ti * kTileX + hx - 1, gj = tj * kTileY + hy - 1;
@@ -321,7 +326,7 @@ __device__ __forceinline__ void tile_solid(const StepArgs &p, int ti, int tj, Ti
     if (L.bc[0] == VPLBM_PERIODIC) gi = gi < 0 ? gi + L.nx : (gi >= L.nx ? gi - L.nx : gi);
     if (L.bc[2] == VPLBM_PERIODIC) gj = gj < 0 ? gj + L.ny : (gj >= L.ny ? gj - L.ny : gj);
     const bool in = gi >= 0 && gi < L.nx && gj >= 0 && gj < L.ny;
-    tm.s[hy][hx] = (in && body_contains(*p.body_src, gi, gj)) ? kSolid : (uint8_t)0;
+    tm.s[hy][hx] = (in && disk_contains(*p.body_src, near, gi, gj)) ? kSolid : (uint8_t)0;
   }
 }
 
@@ -421,23 +426,20 @@ __device__ __forceinline__ FixAcc<T> vol_terms(const BodyRef<T> b, int i, int j,
 // rigid body and the tail
 // ---------------------------------------------------------------------------
 
-// Rigid-body update (Eqs. dep1 and theta2, explicit trapezoid in time) for a
-// disk of density ratio rho_s/rho in a fluid of density 1.
-__device__ void rigid_update(BodyState &b, const double F[3]) {
+// What the rigid-body update of a disk of density ratio rho_s/rho in a fluid of
+// density 1 needs of its constants: 1/m, 1/m, 1/I and the buoyant acceleration
+// (1 - 1/rho_r) g of the three coordinates.  Computed by three lanes of every
+// block that may turn out the last, while its other warps work: the tail's
+// chain of FP64 operations (some 60 cycles each) is then four operations long,
+// where it held the mass, the inertia and four divisions.
+struct RigidConst {
+  double inv[3], acc[3];
+};
+__device__ __forceinline__ void rigid_const(const BodyState &b, RigidConst &c, int k) {
   const double r = 0.5 * b.length;
   const double m = b.density_ratio * 3.14159265358979323846 * r * r;
-  const double inertia = 0.5 * m * r * r;
-  const double buoy = 1.0 - 1.0 / b.density_ratio;
-  const double ax = F[0] / m + buoy * b.gx;
-  const double ay = F[1] / m + buoy * b.gy;
-  const double u0x = b.ux, u0y = b.uy, w0 = b.omega;
-  b.ux = u0x + ax;
-  b.uy = u0y + ay;
-  b.omega = w0 + F[2] / inertia;
-  b.xg += 0.5 * (u0x + b.ux);
-  b.yg += 0.5 * (u0y + b.uy);
-  b.theta += 0.5 * (w0 + b.omega);
-  body_sync_f32(b);
+  c.inv[k] = 1.0 / (k == 2 ? 0.5 * m * r * r : m);
+  c.acc[k] = k == 2 ? 0.0 : (1.0 - 1.0 / b.density_ratio) * (k == 0 ? b.gx : b.gy);
 }
 
 // Force bookkeeping of a launch whose tail was deferred (a fixed body): the
@@ -490,12 +492,12 @@ __device__ void finalize(const StepArgs &p) {
 }
 
 // The last participating block: the step's forces from the fixed-point sums
-// (plus the polygon's constant SIM part), histories, running sums, body.
-// Its loads are spread over threads and issued together, and each thread then
-// stores its own words: the tail costs a few memory round trips, not one per
-// word.
+// (plus the polygon's constant SIM part), histories, running sums, body
+// (Eqs. dep1 and theta2, explicit trapezoid in time).  Its loads are spread over
+// threads and issued together, and the three coordinates of the body are updated
+// by three lanes side by side.
 template <typename T>
-__device__ void tail(const StepArgs &p, const ForceRegion &reg) {
+__device__ void tail(const StepArgs &p, const ForceRegion &reg, const RigidConst &rc) {
   constexpr int kBodyWords = (int)(sizeof(BodyState) / sizeof(unsigned long long));
   static_assert(sizeof(BodyState) % sizeof(unsigned long long) == 0, "BodyState in 8-byte words");
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -511,13 +513,61 @@ __device__ void tail(const StepArgs &p, const ForceRegion &reg) {
     if (tid >= 3 && tid < 6) v += p.sim_const[tid - 3];
     tot[tid] = v;
   } else if (tid >= 32 && tid < 32 + kBodyWords) {
-    reinterpret_cast<unsigned long long *>(&old_b)[tid - 32] =
+    const unsigned long long w =
         __ldcg(reinterpret_cast<const unsigned long long *>(p.body_src) + (tid - 32));
+    reinterpret_cast<unsigned long long *>(&old_b)[tid - 32] = w;
+    reinterpret_cast<unsigned long long *>(&new_b)[tid - 32] = w;
   } else if (tid == 64) {
     step_s = __ldcg(p.dev_step);
   }
   __syncthreads();
-  if (tid < kHistCols) {
+  if (tid >= 32 && tid < 64) {
+    // the warp of the body: lanes 0, 1, 2 update x, y and the rotation
+    const int k = min(tid - 32, 2);
+    const bool sim = old_b.estimator == VPLBM_SIM;
+    const double v0 = k == 0 ? old_b.ux : k == 1 ? old_b.uy : old_b.omega;
+    const double x0 = k == 0 ? old_b.xg : k == 1 ? old_b.yg : old_b.theta;
+    const double v1 = v0 + fma(tot[sim ? 3 + k : k], rc.inv[k], rc.acc[k]);
+    const double x1 = x0 + 0.5 * (v0 + v1);
+    const double x = __shfl_sync(kFull, x1, 0), y = __shfl_sync(kFull, x1, 1);
+    ForceRegion nreg = reg;
+    bool ok = true;
+    if (old_b.moving) {
+      nreg = make_region(p.L, x, y, 0.5 * old_b.length, p.ntiles_x, p.ntiles_y, p.tile_w);
+      // the body left the lattice or moved a node in one step: keep it where
+      // it was and flag the run as unstable
+      ok = !(nreg.error || nreg.count > p.region_slots || nreg.count > p.region_capacity ||
+             fabs(x - old_b.xg) >= 1.0 || fabs(y - old_b.yg) >= 1.0);
+    }
+    if (old_b.moving && ok) {
+      if (tid == 32) {
+        new_b.ux = v1;
+        new_b.xg = x1;
+        new_b.f_ux = (float)v1;
+        new_b.f_xg = (float)x1;
+      } else if (tid == 33) {
+        new_b.uy = v1;
+        new_b.yg = x1;
+        new_b.f_uy = (float)v1;
+        new_b.f_yg = (float)x1;
+      } else if (tid == 34) {
+        new_b.omega = v1;
+        new_b.theta = x1;
+        new_b.f_omega = (float)v1;
+      }
+    }
+    if (tid == 32) {
+      if (!ok) {
+        atomicOr(p.status, kStatusUnstable);
+        nreg = reg;
+      }
+      *p.reg_dst = nreg;
+    }
+    __syncwarp();
+    if (tid < 32 + kBodyWords)
+      reinterpret_cast<unsigned long long *>(p.body_dst)[tid - 32] =
+          reinterpret_cast<const unsigned long long *>(&new_b)[tid - 32];
+  } else if (tid < kHistCols) {
     // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
     const bool have = tid < 3 || tid >= 6 || do_sim;
     p.hist[kHistCols * (step_s % p.hist_len) + tid] =
@@ -527,38 +577,13 @@ __device__ void tail(const StepArgs &p, const ForceRegion &reg) {
     p.counts[0] += 1;
   } else if (tid == 17 && do_sim) {
     p.counts[1] += 1;
-  } else if (tid == 32) {
-    new_b = old_b;
-    ForceRegion nreg = reg;
-    if (old_b.moving) {
-      const bool sim = old_b.estimator == VPLBM_SIM;
-      const double F[3] = {sim ? tot[3] : tot[0], sim ? tot[4] : tot[1], sim ? tot[5] : tot[2]};
-      rigid_update(new_b, F);
-      nreg = make_region(p.L, new_b.xg, new_b.yg, 0.5 * new_b.length, p.ntiles_x, p.ntiles_y,
-                         p.tile_w);
-      if (nreg.error || nreg.count > p.region_slots || nreg.count > p.region_capacity ||
-          fabs(new_b.xg - old_b.xg) >= 1.0 || fabs(new_b.yg - old_b.yg) >= 1.0) {
-        // the body left the lattice or moved a node in one step: keep it
-        // where it was and flag the run as unstable
-        atomicOr(p.status, kStatusUnstable);
-        new_b = old_b;
-        nreg = reg;
-      }
-    }
-    *p.reg_dst = nreg;
+  } else if (tid == 64) {
     *p.dev_step = step_s + 1;
   }
-  __syncthreads();
-  if (tid >= 32 && tid < 32 + kBodyWords)
-    reinterpret_cast<unsigned long long *>(p.body_dst)[tid - 32] =
-        reinterpret_cast<const unsigned long long *>(&new_b)[tid - 32];
-  __syncthreads();
-  if (tid < kAccWords) p.acc[tid] = 0ull;
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    *p.ticket = 0u;
-  }
+  // every read of the sums above precedes the barrier; the next launch sees
+  // all of this block's stores
+  if (tid >= 96 && tid < 96 + kAccWords) p.acc[tid - 96] = 0ull;
+  if (tid == 160) *p.ticket = 0u;
 }
 
 // ---------------------------------------------------------------------------
@@ -1096,6 +1121,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) special_kernel(const Ste
   using T = typename Store<S>::T;
   __shared__ int is_last;
   __shared__ TileMask tmask;
+  __shared__ RigidConst rigid;
   const Lattice &L = p.L;
   const int tid = threadIdx.y * kTileX + threadIdx.x;
   const ForceRegion reg = *p.reg_src;
@@ -1106,6 +1132,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) special_kernel(const Ste
     finalize<T>(p);
     return;
   }
+
+  if (!p.defer && tid >= kThreads - 32 && tid < kThreads - 29 && p.body_src->moving)
+    rigid_const(*p.body_src, rigid, tid - (kThreads - 32));
 
   if (b < p.sim_blocks) {
     // ---- SIM points of this level ----
@@ -1181,7 +1210,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) special_kernel(const Ste
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  tail<T>(p, reg);
+  tail<T>(p, reg, rigid);
 }
 
 // ---------------------------------------------------------------------------

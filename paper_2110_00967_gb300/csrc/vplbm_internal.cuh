@@ -397,6 +397,32 @@ __device__ __forceinline__ bool body_contains(const BodyState &b, int i, int j) 
   return false;
 }
 
+// The same predicate for a disk, decided in FP32 wherever that is certain: the
+// squared distance, with coordinates taken relative to the node below the
+// centre, has a relative error below 1e-6, and only nodes closer to the circle
+// than 1e-5 of r^2 need the FP64 form (none in most warps).  GB300 has two FP64
+// lanes per SM: evaluated everywhere in FP64, the mask of a moving disk took
+// 1.8 us of its 12 us step.
+struct NearTest {
+  int i0, j0;
+  float fx, fy, r2;
+  __device__ __forceinline__ explicit NearTest(const BodyState &b) {
+    const double x0 = floor(b.xg), y0 = floor(b.yg);
+    i0 = (int)x0;
+    j0 = (int)y0;
+    fx = (float)(b.xg - x0);
+    fy = (float)(b.yg - y0);
+    const float r = 0.5f * (float)b.length;
+    r2 = r * r;
+  }
+};
+__device__ __forceinline__ bool disk_contains(const BodyState &b, const NearTest &t, int i, int j) {
+  const float dx = (float)(i - t.i0) - t.fx, dy = (float)(j - t.j0) - t.fy;
+  const float d2 = dx * dx + dy * dy, diff = d2 - t.r2;
+  if (fabsf(diff) > 1e-5f * (d2 + t.r2) + 1e-5f) return diff < 0.0f;
+  return body_contains(b, i, j);
+}
+
 // neighbour of (i, j) along a inside the lattice (periodic sides wrap);
 // false when it lies beyond a non-periodic side
 __device__ __forceinline__ bool neighbour(const Lattice &L, int a, int i, int j, int &ni, int &nj) {
