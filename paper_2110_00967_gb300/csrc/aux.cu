@@ -1,5 +1,7 @@
 // aux.cu -- mask rasterisation (Eq. fcar), interface flags, initial state and
 // the conversions between the stored offsets and FP64 fields.
+#include <cmath>
+
 #include "vplbm_internal.cuh"
 
 namespace vplbm {
@@ -82,36 +84,114 @@ __global__ void get_f_kernel(Lattice L, const S *buf, const typename Store<S>::T
       out[(a - a0) * n + k] = (double)pre_pop<S, kGather>(buf, prev, L, a, i, j) + L.E[a];
 }
 
-// macroscopic fields of Eqs. updatestep and updatestepm, FP64
+// Moments of FP32 offsets, exactly: each offset as a 64-bit integer multiple of
+// 2^-60 (FP32 values above 2^-37 in magnitude exactly, smaller ones cut off
+// below 1e-18), summed as integers with the reference state's part.  rho and j
+// are scaled by 2^60, which their quotient does not see.
+constexpr int kFixBits = 60;
+__device__ __forceinline__ long long fixed60(float h) {
+  const uint32_t bits = __float_as_uint(h);
+  const int e = (int)(bits >> 23 & 0xffu);
+  const unsigned long long m = (unsigned long long)((bits & 0x7fffffu) | 0x800000u) << 35;
+  const long long v = (long long)(m >> min(max(125 - e, 0), 63));  // |h| < 1/2: e <= 125
+  return (int)bits < 0 ? -v : v;
+}
+
+// The double nearest v (a tie away from zero), by integer operations: the
+// conversion instruction shares the FP64 lanes.
+__device__ __forceinline__ double to_double(long long v) {
+  const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
+  if (u == 0) return 0.0;
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = u << lz;                          // leading bit 63
+  const unsigned long long r = (m >> 11) + (m >> 10 & 1ull);     // 53 bits, rounded
+  // the leading bit of r adds one to the exponent
+  return __longlong_as_double((long long)((((unsigned long long)(1085 - lz) << 52) + r) |
+                                          ((unsigned long long)v & 0x8000000000000000ull)));
+}
+
+// 1/a for a normal a by one third-order iteration from the hardware's
+// approximation (relative error below 2^-20, cubed): three FMAs
+__device__ __forceinline__ double near_rcp(double a) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  const double e = fma(-a, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Macroscopic fields of Eqs. updatestep and updatestepm, FP64.  (ox, oy): the
+// part of j that the offsets leave out, u_ref plus half the body force, for FP32
+// offsets in units of 2^-60.  GB300's two FP64 lanes per SM bound this kernel
+// (about 140 FP64 operations per node for nine conversions, the moments and two
+// divisions: 246 us for 2048 x 1024, where its traffic takes 19 us); FP32 offsets
+// are therefore summed as integers, which rounds less, and a node is left with
+// five FP64 operations.
 template <typename S, bool kGather>
-__global__ void get_fields_kernel(Lattice L, const S *buf, const typename Store<S>::T *prev,
-                                  const uint8_t *chi, const BodyState *body, double half_pen,
-                                  double *rho_o, double *ux_o, double *uy_o, int j0, int rows) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t n = (int64_t)L.nx * rows;
-  if (k >= n) return;
-  const int i = (int)(k % L.nx), j = j0 + (int)(k / L.nx);
-  double rho = 0.0, jx = 0.0, jy = 0.0;
+__global__ void __launch_bounds__(kAuxThreads)
+    get_fields_kernel(Lattice L, const S *buf, const typename Store<S>::T *prev,
+                      const uint8_t *chi, const BodyState *body, double half_pen, double *rho_o,
+                      double *ux_o, double *uy_o, int j0, int rows, long long ox, long long oy) {
+  using T = typename Store<S>::T;
+  const int i = blockIdx.x * kAuxThreads + threadIdx.x;
+  if (i >= L.nx) return;
+  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+    const int j = j0 + r;
+    const int64_t node = (int64_t)j * L.pitch + i, k = (int64_t)r * L.nx + i;
+    T h[9];
+    if (kGather && i > 0 && i < L.nx - 1 && j > 0 && j < L.ny - 1) {
 #pragma unroll
-  for (int a = 0; a < 9; ++a) {
-    const double f = (double)pre_pop<S, kGather>(buf, prev, L, a, i, j) + L.E[a];
-    rho += f;
-    jx += cx_of(a) * f;
-    jy += cy_of(a) * f;
+      for (int a = 0; a < 9; ++a)
+        h[a] = pop_at(buf, L, a, i - cx_of(a), j - cy_of(a));
+    } else {
+#pragma unroll
+      for (int a = 0; a < 9; ++a) h[a] = pre_pop<S, kGather>(buf, prev, L, a, i, j);
+    }
+    const uint8_t m = chi[node];
+    double rho, jx, jy;  // FP32 offsets: scaled by 2^60
+    bool exact = false, near_one;  // near_one: rho between 2^-10 and 2^10
+    if constexpr (sizeof(T) == 4) {
+      float big = 0.f;
+#pragma unroll
+      for (int a = 0; a < 9; ++a) big = fmaxf(big, fabsf(h[a]));
+      long long v[9];
+#pragma unroll
+      for (int a = 0; a < 9; ++a) v[a] = fixed60(h[a]);
+      const long long s = v[0] + v[1] + v[2] + v[3] + v[4] + v[5] + v[6] + v[7] + v[8] + (1ll << kFixBits);
+      // (NaN offsets fail the sum's comparison: fmaxf drops them)
+      exact = big < 0.4f && s > (1ll << (kFixBits - 10)) && h[0] + h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8] < 4.f;
+      if (exact) {
+        rho = to_double(s);
+        jx = to_double(v[1] - v[3] + v[5] - v[6] + v[8] - v[7] + ox);
+        jy = to_double(v[2] - v[4] + v[5] - v[7] + v[6] - v[8] + oy);
+      }
+    }
+    if (!exact) {
+      rho = 1.0 + ((((double)h[0] + (double)h[1]) + ((double)h[2] + (double)h[3])) +
+                   (((double)h[4] + (double)h[5]) + ((double)h[6] + (double)h[7])) + (double)h[8]);
+      jx = ((double)h[1] - (double)h[3]) + ((double)h[5] - (double)h[6]) + ((double)h[8] - (double)h[7]);
+      jy = ((double)h[2] - (double)h[4]) + ((double)h[5] - (double)h[7]) + ((double)h[6] - (double)h[8]);
+      jx += L.ur[0] + 0.5 * L.bf[0];
+      jy += L.ur[1] + 0.5 * L.bf[1];
+    }
+    near_one = exact || (uint32_t)(__double2hiint(rho) - (1013 << 20)) < (uint32_t)(20 << 20);
+    if (m & kSolid) {
+      const BodyState b = *body;
+      const double usx = b.ux - b.omega * ((double)j - b.yg);
+      const double usy = b.uy + b.omega * ((double)i - b.xg);
+      ux_o[k] = (jx + half_pen * rho * usx) / (rho + half_pen * rho);
+      uy_o[k] = (jy + half_pen * rho * usy) / (rho + half_pen * rho);
+    } else if (near_one) {
+      const double inv = near_rcp(rho);
+      ux_o[k] = jx * inv;
+      uy_o[k] = jy * inv;
+    } else {
+      ux_o[k] = jx / rho;
+      uy_o[k] = jy / rho;
+    }
+    // 2^-60 rho: the exponent alone (rho is normal)
+    rho_o[k] = exact ? __hiloint2double(__double2hiint(rho) - (kFixBits << 20), __double2loint(rho))
+                     : rho;
   }
-  jx += 0.5 * L.bf[0];
-  jy += 0.5 * L.bf[1];
-  double ux = jx / rho, uy = jy / rho;
-  if (chi[(int64_t)j * L.pitch + i] & kSolid) {
-    const BodyState b = *body;
-    const double usx = b.ux - b.omega * ((double)j - b.yg);
-    const double usy = b.uy + b.omega * ((double)i - b.xg);
-    ux = (jx + half_pen * rho * usx) / (rho + half_pen * rho);
-    uy = (jy + half_pen * rho * usy) / (rho + half_pen * rho);
-  }
-  rho_o[k] = rho;
-  ux_o[k] = ux;
-  uy_o[k] = uy;
 }
 
 template <typename S>
@@ -165,13 +245,16 @@ cudaError_t get_fields_t(bool gather, const Lattice &L, const void *buf, const v
                          double *ux, double *uy, int j0, int rows, cudaStream_t s) {
   using T = typename Store<S>::T;
   const T *prev = static_cast<const T *>(prev_v);
-  const int g = blocks_for((int64_t)L.nx * rows);
+  const dim3 g((L.nx + kAuxThreads - 1) / kAuxThreads, rows < 65535 ? rows : 65535);
+  const double unit = (double)(1ll << kFixBits);
+  const long long ox = llrint((L.ur[0] + 0.5 * L.bf[0]) * unit);
+  const long long oy = llrint((L.ur[1] + 0.5 * L.bf[1]) * unit);
   if (gather)
     get_fields_kernel<S, true><<<g, kAuxThreads, 0, s>>>(L, (const S *)buf, prev, chi, body,
-                                                         half_pen, rho, ux, uy, j0, rows);
+                                                         half_pen, rho, ux, uy, j0, rows, ox, oy);
   else
     get_fields_kernel<S, false><<<g, kAuxThreads, 0, s>>>(L, (const S *)buf, prev, chi, body,
-                                                          half_pen, rho, ux, uy, j0, rows);
+                                                          half_pen, rho, ux, uy, j0, rows, ox, oy);
   return cudaGetLastError();
 }
 
