@@ -388,6 +388,8 @@ StepArgs step_args(vplbm_ctx *c, int src, bool do_sim) {
   a.f_a_plus = (float)a.a_plus;
   a.f_a_minus = (float)a.a_minus;
   a.f_half_pen = (float)a.half_pen;
+  a.pen = -2.0 * c->half_pen / (1.0 + c->half_pen);
+  a.f_pen = (float)a.pen;
   a.f_sim_s = (float)(1.0 - 0.5 / a.tau_plus);
   a.tile_w = kTileX;
   a.ntiles_x = (c->L.nx + kTileX - 1) / kTileX;

@@ -110,15 +110,6 @@ __device__ __forceinline__ double to_double(long long v) {
                                           ((unsigned long long)v & 0x8000000000000000ull)));
 }
 
-// 1/a for a normal a by one third-order iteration from the hardware's
-// approximation (relative error below 2^-20, cubed): three FMAs
-__device__ __forceinline__ double near_rcp(double a) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  const double e = fma(-a, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
 // Macroscopic fields of Eqs. updatestep and updatestepm, FP64.  (ox, oy): the
 // part of j that the offsets leave out, u_ref plus half the body force, for FP32
 // offsets in units of 2^-60.  GB300's two FP64 lanes per SM bound this kernel

@@ -267,20 +267,6 @@ __device__ __forceinline__ void stored_pops(float (&o)[9], uint32_t level, uint3
   }
 }
 
-// MEM and volume-integral terms of one box node, from its values before
-// rounding, added to the sums of its step
-__device__ __forceinline__ void box_terms(const StepArgs &p, const float (&o)[9], int i, int j,
-                                          bool solid, uint32_t links, float pen_x, float pen_y,
-                                          FixAcc<float> &acc, FixAcc<float> &vol) {
-  if (links) {
-    Offsets<float> post;
-#pragma unroll
-    for (int a = 0; a < 9; ++a) post.h[a] = o[a];
-    acc = mem_terms<float>(p, post, i, j, solid, links);
-  }
-  if (solid) vol = vol_terms<float>(BodyRef<float>(*p.body_src), i, j, pen_x, pen_y);
-}
-
 // the first step's tile in shared memory, read by unwrapped node coordinates
 struct TileSrc {
   const float (*post)[kPairThreads];
@@ -314,7 +300,7 @@ __host__ __device__ inline PairGrid pair_grid(const StepArgs &p) {
 template <typename S, bool kForce, bool kSR>
 __device__ __forceinline__ void pair_special(const StepArgs &p, const PairGrid &g, int b,
                                              float (*post)[kPairThreads],
-                                             float (*old)[kPairThreads]) {
+                                             float (*old)[kPairThreads], LinkList<float> *list) {
   const Lattice &L = p.L;
   const int tid = threadIdx.x, lane = tid & 31;
   const BodyState *body = p.body_src;
@@ -463,6 +449,7 @@ __device__ __forceinline__ void pair_special(const StepArgs &p, const PairGrid &
       if (sim2) m = p.chi[node];
       bad |= update_node<S, kForce>(h, m, gi, gj, L, body, cst, o, px, py) && own;
     }
+    __syncwarp();  // fluid and solid lanes meet again
     const uint32_t level = kSR ? sr_level(p, second ? 1 : 0) : 0u;
     if (sim2) {
       // the populations streaming into (qi, qj), exchanged within the group
@@ -492,10 +479,11 @@ __device__ __forceinline__ void pair_special(const StepArgs &p, const PairGrid &
       continue;
     }
     if (!frame) {
-      FixAcc<float> acc, vol;
-      if (own) box_terms(p, o, i, j, m & kSolid, links, px, py, acc, vol);
+      // from the values before rounding
       unsigned long long *sums = second ? p.acc2 : p.acc;
-      warp_add(acc, sums, 0);
+      warp_add(mem_terms<float, true>(p, o, i, j, m & kSolid, own ? links : 0u, list), sums, 0);
+      FixAcc<float> vol;
+      if (own && (m & kSolid)) vol = vol_terms<float>(BodyRef<float>(*body), i, j, px, py);
       warp_add(vol, sums, 6);
     }
     if (!second) {
@@ -525,7 +513,8 @@ __device__ __forceinline__ void pair_special(const StepArgs &p, const PairGrid &
 template <typename S, bool kForce, bool kSR>
 __global__ void __launch_bounds__(kPairThreads, kPairMinBlocks) pair_kernel(const StepArgs p) {
   using Raw = typename Cell<S>::Raw;
-  constexpr size_t kTileBytes = 12 * kPairThreads * sizeof(float);
+  constexpr size_t kPopBytes = 12 * kPairThreads * sizeof(float);
+  constexpr size_t kTileBytes = kPopBytes + kPairWarps * sizeof(LinkList<float>);
   constexpr size_t kRingBytes = kRing<S> ? sizeof(Raw[kPairStages][9][kPairThreads]) : 0;
   __shared__ __align__(16) unsigned char smem[kRingBytes > kTileBytes ? kRingBytes : kTileBytes];
   const PairGrid g = pair_grid(p);
@@ -533,7 +522,8 @@ __global__ void __launch_bounds__(kPairThreads, kPairMinBlocks) pair_kernel(cons
   if (kSR && b == 0 && threadIdx.x == 0) *p.rng_dst = *p.rng_src + 2ull;  // the next launch's counter
   if (b < g.special) {
     float(*post)[kPairThreads] = reinterpret_cast<float(*)[kPairThreads]>(smem);
-    pair_special<S, kForce, kSR>(p, g, b, post, post + 9);
+    LinkList<float> *lists = reinterpret_cast<LinkList<float> *>(smem + kPopBytes);
+    pair_special<S, kForce, kSR>(p, g, b, post, post + 9, lists + (threadIdx.x >> 5));
     return;
   }
   pair_bulk<S, kForce, kSR>(p, (b - g.special) % p.pair_bx, (b - g.special) / p.pair_bx,

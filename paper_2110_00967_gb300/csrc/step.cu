@@ -78,17 +78,7 @@ __device__ __forceinline__ void warp_add(const FixAcc<T> &a, unsigned long long 
     }
 }
 
-// the nine populations of a node, passed by value
-template <typename T>
-struct Offsets {
-  T h[9];
-};
-
-// ---------------------------------------------------------------------------
-// SIM (Sec. 2.3.2)
-// ---------------------------------------------------------------------------
-
-// The SIM terms are written with named roundings, so that a state gives the
+// The force terms are written with named roundings, so that a state gives the
 // same bits in a single step and in either step of a pair, whatever the
 // compiler would fuse around them.
 __device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
@@ -99,6 +89,16 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ double rrcp(double a) { return __drcp_rn(a); }
+
+// the nine populations of a node, passed by value
+template <typename T>
+struct Offsets {
+  T h[9];
+};
+
+// ---------------------------------------------------------------------------
+// SIM (Sec. 2.3.2)
+// ---------------------------------------------------------------------------
 
 // The part of the stress beyond -(1/3) I at a fluid node,
 // sigma + (1/3) I = -(rho - 1)/3 I - (1 - 1/(2 tau+)) sum c c (f - feq),
@@ -314,12 +314,29 @@ struct TileMask {
   uint8_t s[kTileY + 2][kTileX + 2];
 };
 
-__device__ __forceinline__ void tile_solid(const StepArgs &p, int ti, int tj, TileMask &tm) {
+// A block of the special kernel takes a tile of kThreads nodes, or with FP64
+// storage one of its eight 32-node slices: the FP64 lanes of an SM (two) are what
+// its blocks wait for, and one warp per block spreads them over all SMs (the
+// disk channel's step, 20 tiles: 32 -> 28 us, and 15 us with one link per lane
+// in mem_terms; FP32 tiles in slices of 128 or 64 gain nothing and a moving
+// disk's step loses 0.3 and 0.7 us of 10.0).  Nodes are numbered within the tile,
+// x fastest.
+template <typename S>
+constexpr int kSlices = sizeof(S) == 8 ? 8 : 1;
+struct Slice {
+  int first, count;  // the block's nodes of the tile
+};
+
+__device__ __forceinline__ void tile_solid(const StepArgs &p, int ti, int tj, Slice sl,
+                                           TileMask &tm) {
   const Lattice &L = p.L;
-  const int tid = threadIdx.y * kTileX + threadIdx.x;
   const NearTest near(*p.body_src);
-  for (int q = tid; q < (kTileY + 2) * (kTileX + 2); q += kThreads) {
-    const int hx = q % (kTileX + 2), hy = q / (kTileX + 2);
+  // the slice's rows and columns with their halo (a slice shorter than a row
+  // lies within one)
+  const int x0 = sl.first % kTileX, y0 = sl.first / kTileX;
+  const int w = min(sl.count, kTileX) + 2, h = (sl.count + kTileX - 1) / kTileX + 2;
+  for (int q = threadIdx.x; q < w * h; q += blockDim.x) {
+    const int hx = x0 + q % w, hy = y0 + q / w;
     int gi = ti * kTileX + hx - 1, gj = tj * kTileY + hy - 1;
     // halo nodes across a periodic side are the nodes there; beyond another
     // side they are never a neighbour (neighbour() gives false)
@@ -353,7 +370,7 @@ __device__ __forceinline__ uint8_t tile_mask_byte(const Lattice &L, const TileMa
 // own.  Off the edges the eight bytes are loaded together with the node's own
 // populations: the links' latency is then not added to theirs.
 __device__ __forceinline__ uint32_t node_links(const StepArgs &p, int i, int j, bool solid,
-                                               const TileMask *tm) {
+                                               const TileMask *tm, int tx = 0, int ty = 0) {
   const Lattice &L = p.L;
   const uint8_t self = solid ? kSolid : (uint8_t)0;
   uint32_t links = 0;
@@ -369,43 +386,112 @@ __device__ __forceinline__ uint32_t node_links(const StepArgs &p, int i, int j, 
   for (int a = 1; a < 9; ++a) {
     int ni, nj;
     if (!neighbour(L, a, i, j, ni, nj)) continue;
-    const uint8_t m = tm ? tm->s[threadIdx.y + 1 + cy_of(a)][threadIdx.x + 1 + cx_of(a)]
+    const uint8_t m = tm ? tm->s[ty + 1 + cy_of(a)][tx + 1 + cx_of(a)]
                          : p.chi[(int64_t)nj * L.pitch + ni];
     links |= (uint32_t)((m ^ self) & kSolid) << a;
   }
   return links;
 }
 
-// The link terms of one interface node (Eq. MMEL): for each lattice
+// The link terms of a warp's interface nodes (Eq. MMEL): for each lattice
 // neighbour of the other phase, the fluid end adds (c_a - u_Gamma) f~_a and
 // the solid end subtracts its own (c_a - u_Gamma) f~_a, with x_Gamma the link
 // midpoint and u_Gamma the rigid velocity there; torques about the reference
 // point (Eq. fluidtorque).  f~ = h~ + E is split so that the E parts, which
 // cancel in pairs around a fixed body, are rounded exactly.
+//
+// A warp holds a few interface nodes with a few links each: walking the eight
+// directions with most lanes idle was the longest part of a special block
+// (2.7 us in FP32, some 400 FP64 operations in FP64).  Every lane takes one link
+// of the warp instead: listed in shared memory, or without a list (nullptr)
+// found from the lanes' link counts by shuffles, for kernels that run beside
+// others which need the L1 that the list would take (the FP16 batch 12.9 us per
+// lattice step without lists, 13.5 with them).  Every lane of the warp calls; a
+// lane's sums are of the links it took (their order and place do not matter: the
+// sums are exact).
 template <typename T>
-__device__ __forceinline__ FixAcc<T> mem_terms(const StepArgs &p, const Offsets<T> post, int i, int j,
-                                            bool solid, uint32_t links) {
-  const T(&o)[9] = post.h;
+struct LinkList {
+  T post[8][32];       // o[1 .. 8] of the lanes with links
+  uint16_t link[256];  // lane | direction << 5 | solid << 9
+};
+template <typename T, bool kList>
+__device__ __forceinline__ FixAcc<T> mem_terms(const StepArgs &p, const T (&o)[9], int i, int j,
+                                               bool solid, uint32_t links, LinkList<T> *list) {
   FixAcc<T> acc;
+  __syncwarp();  // the lanes come from divergent updates; unmerged they would run all this in turn
+  if (!__any_sync(kFull, links != 0)) return acc;
+  const int lane = threadIdx.x & 31;
+  const int n = __popc(links);
+  int end = n;  // links of the lanes up to this one
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int v = __shfl_up_sync(kFull, end, d);
+    if (lane >= d) end += v;
+  }
+  const int total = __shfl_sync(kFull, end, 31);
+  if constexpr (kList) {
+    int at = end - n;
+#pragma unroll
+    for (int a = 1; a < 9; ++a)
+      if (links >> a & 1u) {
+        list->post[a - 1][lane] = o[a];
+        list->link[at++] = (uint16_t)(lane | a << 5 | (solid ? 1 << 9 : 0));
+      }
+    __syncwarp();
+  }
+  const uint32_t mine = links | (solid ? 1u : 0u);  // bit 0: the node's phase
   const Lattice &L = p.L;
   const BodyRef<T> b(*p.body_src);
-  const T sg = solid ? (T)-1 : (T)1;
+#pragma unroll 1
+  for (int first = 0; first < total; first += 32) {
+    const int t = first + lane;
+    int from = 0, a = 1;  // the link's lane and direction
+    bool in_solid;
+    T post;
+    if constexpr (kList) {
+      const uint32_t e = t < total ? list->link[t] : 1u << 5;
+      from = (int)(e & 31u);
+      a = (int)(e >> 5 & 15u);
+      in_solid = e >> 9;
+      post = list->post[a - 1][from];
+    } else {
+      // the lane of link t is the first whose end lies beyond t
 #pragma unroll
-  for (int a = 1; a < 9; ++a) {
-    if (!(links >> a & 1u)) continue;
-    const T rx = ((T)i - b.xg) + (T)(0.5 * cx_of(a));
-    const T ry = ((T)j - b.yg) + (T)(0.5 * cy_of(a));
-    const T vx = (T)cx_of(a) - (b.ux - b.om * ry);
-    const T vy = (T)cy_of(a) - (b.uy + b.om * rx);
-    const T ah = sg * o[a], aw = sg * LatC<T>::E(L, a);
-    const T lxh = vx * ah, lyh = vy * ah, lxw = vx * aw, lyw = vy * aw;
+      for (int d = 16; d > 0; d >>= 1)
+        if (__shfl_sync(kFull, end, from + d - 1) <= t) from += d;
+      from &= 31;
+      const uint32_t bits = __shfl_sync(kFull, mine, from);
+      const int before = __shfl_sync(kFull, end - n, from);
+      uint32_t rest = bits & ~1u;  // its directions from the one taken on
+#pragma unroll
+      for (int k = 0; k < 7; ++k)
+        if (k < t - before) rest &= rest - 1u;
+      a = __ffs((int)rest) - 1;
+      in_solid = bits & 1u;
+      post = __shfl_sync(kFull, o[1], from);
+#pragma unroll
+      for (int q = 2; q < 9; ++q) {
+        const T v = __shfl_sync(kFull, o[q], from);
+        if (a == q) post = v;
+      }
+    }
+    const int ni = __shfl_sync(kFull, i, from), nj = __shfl_sync(kFull, j, from);
+    if (t >= total) continue;
+    const T cx = (T)cx_of(a), cy = (T)cy_of(a);
+    const T sg = in_solid ? (T)-1 : (T)1;
+    const T rx = radd(radd((T)ni, -b.xg), rmul((T)0.5, cx));
+    const T ry = radd(radd((T)nj, -b.yg), rmul((T)0.5, cy));
+    const T vx = radd(cx, -rfma(-b.om, ry, b.ux)), vy = radd(cy, -rfma(b.om, rx, b.uy));
+    const T ah = rmul(sg, post), aw = rmul(sg, LatC<T>::E(L, a));
+    const T lxh = rmul(vx, ah), lyh = rmul(vy, ah), lxw = rmul(vx, aw), lyw = rmul(vy, aw);
     acc.add(0, lxh);
     acc.add(0, lxw);
     acc.add(1, lyh);
     acc.add(1, lyw);
-    acc.add(2, rx * lyh - ry * lxh);
-    acc.add(2, rx * lyw - ry * lxw);
+    acc.add(2, rfma(rx, lyh, -rmul(ry, lxh)));
+    acc.add(2, rfma(rx, lyw, -rmul(ry, lxw)));
   }
+  if constexpr (kList) __syncwarp();
   return acc;
 }
 
@@ -418,7 +504,7 @@ __device__ __forceinline__ FixAcc<T> vol_terms(const BodyRef<T> b, int i, int j,
   const T fx = -pen_x, fy = -pen_y;
   vol.add(0, fx);
   vol.add(1, fy);
-  vol.add(2, ((T)i - b.xg) * fy - ((T)j - b.yg) * fx);
+  vol.add(2, rfma(radd((T)i, -b.xg), fy, -rmul(radd((T)j, -b.yg), fx)));
   return vol;
 }
 
@@ -450,45 +536,48 @@ __device__ __forceinline__ void rigid_const(const BodyState &b, RigidConst &c, i
 // call.  Loads are spread over threads and issued together.
 template <typename T>
 __device__ void finalize(const StepArgs &p) {
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int tid = threadIdx.x;
   const int rows = p.prev_rows;
   __shared__ double tot[2][kAccSlots];
   __shared__ long long step_s;
   const bool do_sim = p.prev_sim != 0;
-  const int row = tid >> 5, col = tid & 31;  // warps 0 and 1: the rows
-  if (row < rows && col < kAccSlots) {
-    const unsigned long long *acc = row ? p.acc2_prev : p.acc_prev;
-    const long long w0 = (long long)__ldcg(acc + 2 * col);
-    const long long w1 = (long long)__ldcg(acc + 2 * col + 1);
-    double v = Fix<T>::value(w0, w1);
-    if (col >= 3 && col < 6) v += p.sim_const[col - 3];
-    tot[row][col] = v;
-  } else if (tid == 64) {
-    step_s = __ldcg(p.dev_step);
-  }
+  // a warp per row, or one warp for both in turn
+  const int col = tid & 31, stride = blockDim.x >> 5;
+  for (int row = tid >> 5; row < rows; row += stride)
+    if (col < kAccSlots) {
+      const unsigned long long *acc = row ? p.acc2_prev : p.acc_prev;
+      const long long w0 = (long long)__ldcg(acc + 2 * col);
+      const long long w1 = (long long)__ldcg(acc + 2 * col + 1);
+      double v = Fix<T>::value(w0, w1);
+      if (col >= 3 && col < 6) v += p.sim_const[col - 3];
+      tot[row][col] = v;
+    }
+  if (tid == 31) step_s = __ldcg(p.dev_step);
   __syncthreads();
-  if (row < rows && col < kHistCols) {
-    // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
-    const bool have = col < 3 || col >= 6 || do_sim;
-    p.hist[kHistCols * ((step_s + row) % p.hist_len) + col] =
-        have ? tot[row][col] : __longlong_as_double(0x7ff8000000000000LL);
+  for (int row = tid >> 5; row < rows; row += stride) {
+    if (col < kHistCols) {
+      // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
+      const bool have = col < 3 || col >= 6 || do_sim;
+      p.hist[kHistCols * ((step_s + row) % p.hist_len) + col] =
+          have ? tot[row][col] : __longlong_as_double(0x7ff8000000000000LL);
+    }
+    // every read of the sums above precedes the barrier
+    if (col < kAccWords) (row ? p.acc2_prev : p.acc_prev)[col] = 0ull;
   }
-  if (tid >= 64 && tid < 64 + 6) {
-    const int q = tid - 64;
+  if (tid >= 16 && tid < 22) {
+    const int q = tid - 16;
     if (q < 3 || do_sim) {
       double v = p.sums[q] + tot[0][q];
       if (rows > 1) v += tot[1][q];
       p.sums[q] = v;
     }
-  } else if (tid == 80) {
+  } else if (tid == 22) {
     p.counts[0] += rows;
-  } else if (tid == 81 && do_sim) {
+  } else if (tid == 23 && do_sim) {
     p.counts[1] += rows;
-  } else if (tid == 96) {
+  } else if (tid == 24) {
     *p.dev_step = step_s + rows;
   }
-  // every read of the sums above precedes the barrier
-  if (row < rows && col < kAccWords) (row ? p.acc2_prev : p.acc_prev)[col] = 0ull;
 }
 
 // The last participating block: the step's forces from the fixed-point sums
@@ -500,7 +589,7 @@ template <typename T>
 __device__ void tail(const StepArgs &p, const ForceRegion &reg, const RigidConst &rc) {
   constexpr int kBodyWords = (int)(sizeof(BodyState) / sizeof(unsigned long long));
   static_assert(sizeof(BodyState) % sizeof(unsigned long long) == 0, "BodyState in 8-byte words");
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int tid = threadIdx.x;
   __shared__ double tot[kAccSlots];
   __shared__ BodyState old_b, new_b;
   __shared__ long long step_s;
@@ -512,18 +601,19 @@ __device__ void tail(const StepArgs &p, const ForceRegion &reg, const RigidConst
     double v = Fix<T>::value(w0, w1);
     if (tid >= 3 && tid < 6) v += p.sim_const[tid - 3];
     tot[tid] = v;
-  } else if (tid >= 32 && tid < 32 + kBodyWords) {
+  } else if (tid < kAccSlots + kBodyWords) {
+    const int q = tid - kAccSlots;
     const unsigned long long w =
-        __ldcg(reinterpret_cast<const unsigned long long *>(p.body_src) + (tid - 32));
-    reinterpret_cast<unsigned long long *>(&old_b)[tid - 32] = w;
-    reinterpret_cast<unsigned long long *>(&new_b)[tid - 32] = w;
-  } else if (tid == 64) {
+        __ldcg(reinterpret_cast<const unsigned long long *>(p.body_src) + q);
+    reinterpret_cast<unsigned long long *>(&old_b)[q] = w;
+    reinterpret_cast<unsigned long long *>(&new_b)[q] = w;
+  } else if (tid == 31) {
     step_s = __ldcg(p.dev_step);
   }
   __syncthreads();
-  if (tid >= 32 && tid < 64) {
-    // the warp of the body: lanes 0, 1, 2 update x, y and the rotation
-    const int k = min(tid - 32, 2);
+  if (tid < 32) {
+    // the first warp: lanes 0, 1, 2 update x, y and the rotation
+    const int k = min(tid, 2);
     const bool sim = old_b.estimator == VPLBM_SIM;
     const double v0 = k == 0 ? old_b.ux : k == 1 ? old_b.uy : old_b.omega;
     const double x0 = k == 0 ? old_b.xg : k == 1 ? old_b.yg : old_b.theta;
@@ -540,23 +630,23 @@ __device__ void tail(const StepArgs &p, const ForceRegion &reg, const RigidConst
              fabs(x - old_b.xg) >= 1.0 || fabs(y - old_b.yg) >= 1.0);
     }
     if (old_b.moving && ok) {
-      if (tid == 32) {
+      if (tid == 0) {
         new_b.ux = v1;
         new_b.xg = x1;
         new_b.f_ux = (float)v1;
         new_b.f_xg = (float)x1;
-      } else if (tid == 33) {
+      } else if (tid == 1) {
         new_b.uy = v1;
         new_b.yg = x1;
         new_b.f_uy = (float)v1;
         new_b.f_yg = (float)x1;
-      } else if (tid == 34) {
+      } else if (tid == 2) {
         new_b.omega = v1;
         new_b.theta = x1;
         new_b.f_omega = (float)v1;
       }
     }
-    if (tid == 32) {
+    if (tid == 0) {
       if (!ok) {
         atomicOr(p.status, kStatusUnstable);
         nreg = reg;
@@ -564,26 +654,32 @@ __device__ void tail(const StepArgs &p, const ForceRegion &reg, const RigidConst
       *p.reg_dst = nreg;
     }
     __syncwarp();
-    if (tid < 32 + kBodyWords)
-      reinterpret_cast<unsigned long long *>(p.body_dst)[tid - 32] =
-          reinterpret_cast<const unsigned long long *>(&new_b)[tid - 32];
-  } else if (tid < kHistCols) {
-    // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
-    const bool have = tid < 3 || tid >= 6 || do_sim;
-    p.hist[kHistCols * (step_s % p.hist_len) + tid] =
-        have ? tot[tid] : __longlong_as_double(0x7ff8000000000000LL);
-    if (have && tid < 6) p.sums[tid] += tot[tid];
-  } else if (tid == 16) {
-    p.counts[0] += 1;
-  } else if (tid == 17 && do_sim) {
-    p.counts[1] += 1;
-  } else if (tid == 64) {
-    *p.dev_step = step_s + 1;
+    if (tid < kBodyWords)
+      reinterpret_cast<unsigned long long *>(p.body_dst)[tid] =
+          reinterpret_cast<const unsigned long long *>(&new_b)[tid];
   }
-  // every read of the sums above precedes the barrier; the next launch sees
-  // all of this block's stores
-  if (tid >= 96 && tid < 96 + kAccWords) p.acc[tid - 96] = 0ull;
-  if (tid == 160) *p.ticket = 0u;
+  // the bookkeeping: a second warp where there is one
+  const int q = tid - (blockDim.x > 32 ? 32 : 0);
+  if (q >= 0 && q < 32) {
+    if (q < kHistCols) {
+      // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
+      const bool have = q < 3 || q >= 6 || do_sim;
+      p.hist[kHistCols * (step_s % p.hist_len) + q] =
+          have ? tot[q] : __longlong_as_double(0x7ff8000000000000LL);
+      if (have && q < 6) p.sums[q] += tot[q];
+    } else if (q == 16) {
+      p.counts[0] += 1;
+    } else if (q == 17 && do_sim) {
+      p.counts[1] += 1;
+    } else if (q == 18) {
+      *p.dev_step = step_s + 1;
+    } else if (q == 19) {
+      *p.ticket = 0u;
+    }
+    // every read of the sums above precedes the barrier; the next launch sees
+    // all of this block's stores
+    if (q < kAccWords) p.acc[q] = 0ull;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -663,12 +759,10 @@ __device__ __forceinline__ bool rho_bad(float r) { return !(r > 0.f) || !isfinit
 __device__ __forceinline__ bool rho_bad(double r) { return !(r > 0.0) || !isfinite(r); }
 
 // 1 / a by Newton's iteration y <- y + y (1 - a y) from the hardware's
-// approximation (relative error below 2^-22 in FP32, about 2^-20 in FP64; the
-// error squares at each iteration): one iteration in FP32, two in FP64, each
-// two FMAs, where the correctly rounded division's range checks and fix-ups
-// cost several times that.  In FP32 the result is the correctly rounded one for
-// every float between 2^-20 and 2^20 (all of them were compared with
-// __frcp_rn); densities are near 1.
+// approximation (relative error below 2^-22; the error squares), two FMAs, where
+// the correctly rounded division's range checks and fix-ups cost several times
+// that.  The result is the correctly rounded one for every float between 2^-20
+// and 2^20 (all of them were compared with __frcp_rn); densities are near 1.
 __device__ __forceinline__ F2 vrcp(F2 a) {
   float x, y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(a.v.x));
@@ -676,13 +770,7 @@ __device__ __forceinline__ F2 vrcp(F2 a) {
   const F2 r = vpair(x, y);
   return vfma(r, vfma(vmul(a, vsame(-1.0f)), r, vsame(1.0f)), r);
 }
-__device__ __forceinline__ double vrcp(double a) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-#pragma unroll
-  for (int k = 0; k < 2; ++k) r = vfma(r, vfma(-a, r, 1.0), r);
-  return r;
-}
+__device__ __forceinline__ double vrcp(double a) { return near_rcp(a); }
 
 // Sums and differences of the opposite pairs (a, opp(a)), a = 1, 2, 5, 6, and
 // the moments of the offsets: drho = rho - 1 and (djx, djy) = j - u_ref.
@@ -726,20 +814,26 @@ struct Moments {
 // o_0 = h_0 - 2 sum (even change of a pair's population): equal to the
 // relaxation of h_0 towards heq_0 (plus F_0) in exact arithmetic, and
 // conserving mass exactly up to the rounding of that sum.  kForce = false
-// drops the forcing term (G = 0: a fluid node without body force).
-template <typename V, bool kForce>
+// drops the forcing term (G = 0: a fluid node without body force), kRef = false
+// the terms of u_ref (zero).
+template <typename V, bool kForce, bool kRef = true>
 __device__ __forceinline__ void collide(const V (&h)[9], const Moments<V> &m, V djx, V djy, V ux,
                                         V uy, V dux, V duy, V gx, V gy,
                                         const Consts<typename Val<V>::T> &c, V (&o)[9]) {
   using T = typename Val<V>::T;
   auto k = [](T v) { return Val<V>::splat(v); };
-  const V X = vfma(djx, ux, vmul(k(c.urx), dux));
-  const V Y = vfma(djy, uy, vmul(k(c.ury), duy));
-  const V P = vfma(djx, uy, vmul(k(c.urx), duy));
+  const V X = kRef ? vfma(djx, ux, vmul(k(c.urx), dux)) : vmul(djx, ux);
+  const V Y = kRef ? vfma(djy, uy, vmul(k(c.ury), duy)) : vmul(djy, uy);
+  const V P = kRef ? vfma(djx, uy, vmul(k(c.urx), duy)) : vmul(djx, uy);
   const V t = vadd(X, Y);
   const V axis = vmul(k(c.sp_w1), vfma(k((T)-1.5), t, m.drho));
   const V diag = vmul(k(c.sp_w5), vfma(k((T)3), t, m.drho));
   V even{};
+  // FP64 (bound by its operation count) writes the pair as half its sum and half
+  // its difference, o_a,b = P +- M, and the rest population as what they leave of
+  // rho: eight operations fewer.  FP32 adds the small changes to h, which rounds
+  // less.
+  constexpr bool kHalves = std::is_same<V, double>::value;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int a = q < 2 ? q + 1 : q + 3, b = opp_of(a);
@@ -749,8 +843,9 @@ __device__ __forceinline__ void collide(const V (&h)[9], const Moments<V> &m, V 
                  : q == 2 ? vfma(k(c.sp_9w5), P, diag)
                           : vfma(k(-c.sp_9w5), P, diag);
     const V cdj = q == 0 ? djx : q == 1 ? djy : q == 2 ? vadd(djx, djy) : vsub(djy, djx);
-    V dp = vfma(k(c.nsp_half), m.s[q], ep);
-    V dm = vfma(k(c.nsm_half), m.d[q], vmul(k(q < 2 ? c.sm_k1 : c.sm_k2), cdj));
+    V dp = vfma(k(kHalves ? (T)0.5 + c.nsp_half : c.nsp_half), m.s[q], ep);
+    V dm = vfma(k(kHalves ? (T)0.5 + c.nsm_half : c.nsm_half), m.d[q],
+                vmul(k(q < 2 ? c.sm_k1 : c.sm_k2), cdj));
     if (kForce) {
       // F_a = w [3 c.G + 9 (c.u)(c.G) - 3 u.G], even and odd parts
       const V cu = q == 0 ? ux : q == 1 ? uy : q == 2 ? vadd(ux, uy) : vsub(uy, ux);
@@ -761,17 +856,18 @@ __device__ __forceinline__ void collide(const V (&h)[9], const Moments<V> &m, V 
       dm = vfma(k(c.a_minus), vmul(k(odd_w<T>(a)), cg), dm);
     }
     even = q == 0 ? dp : vadd(even, dp);
-    o[a] = vadd(vadd(h[a], dp), dm);
-    o[b] = vsub(vadd(h[b], dp), dm);
+    o[a] = vadd(kHalves ? dp : vadd(h[a], dp), dm);
+    o[b] = vsub(kHalves ? dp : vadd(h[b], dp), dm);
   }
-  o[0] = vfma(k((T)-2), even, h[0]);
+  o[0] = vfma(k((T)-2), even, kHalves ? m.drho : h[0]);
 }
 
 // The update of fluid nodes (no penalization): moments, velocity and the
 // collision, from the pre-collision offsets h of a node (FP64), a node pair or
-// one node in both lanes (FP32); kForce adds the uniform body force.  Returns
-// rho.
-template <typename V, bool kForce>
+// one node in both lanes (FP32); kForce adds the uniform body force, kRef = false
+// leaves out u_ref = 0 (seven operations; FP64 lattices store offsets from rest).
+// Returns rho.
+template <typename V, bool kForce, bool kRef = true>
 __device__ __forceinline__ V fluid_update(const Lattice &L, const Consts<typename Val<V>::T> &cst,
                                           const V (&h)[9], V (&o)[9]) {
   using T = typename Val<V>::T;
@@ -785,10 +881,11 @@ __device__ __forceinline__ V fluid_update(const Lattice &L, const Consts<typenam
     djx = vfma(Val<V>::splat((T)0.5), gx, djx);
     djy = vfma(Val<V>::splat((T)0.5), gy, djy);
   }
-  const V dux = vmul(vfma(m.drho, Val<V>::splat(-cst.urx), djx), inv);
-  const V duy = vmul(vfma(m.drho, Val<V>::splat(-cst.ury), djy), inv);
-  collide<V, kForce>(h, m, djx, djy, vadd(Val<V>::splat(cst.urx), dux),
-                     vadd(Val<V>::splat(cst.ury), duy), dux, duy, gx, gy, cst, o);
+  const V dux = vmul(kRef ? vfma(m.drho, Val<V>::splat(-cst.urx), djx) : djx, inv);
+  const V duy = vmul(kRef ? vfma(m.drho, Val<V>::splat(-cst.ury), djy) : djy, inv);
+  const V ux = kRef ? vadd(Val<V>::splat(cst.urx), dux) : dux;
+  const V uy = kRef ? vadd(Val<V>::splat(cst.ury), duy) : duy;
+  collide<V, kForce, kRef>(h, m, djx, djy, ux, uy, dux, duy, gx, gy, cst, o);
   return rho;
 }
 
@@ -900,6 +997,9 @@ __device__ __forceinline__ V update_fluid(const Lattice &L,
                                           const V (&h)[9], V (&o)[9]) {
   if constexpr (sizeof(S) == 2)
     return fluid_update16<kForce>(L, cst, h, o);
+  else if constexpr (sizeof(S) == 8)
+    return cst.urx == 0.0 && cst.ury == 0.0 ? fluid_update<V, kForce, false>(L, cst, h, o)
+                                            : fluid_update<V, kForce>(L, cst, h, o);
   else
     return fluid_update<V, kForce>(L, cst, h, o);
 }
@@ -955,19 +1055,30 @@ __device__ __forceinline__ bool update_node(const T (&h)[9], uint8_t mask, int i
     // u - u_ref = (j + k rho u_s)/(rho (1 + k)) - u_ref, written as
     // (u_s - u_ref) + (j - rho u_s)/(rho (1 + k)): the large part is exact
     // and the small one keeps its relative precision (k rho u_s alone
-    // would carry an FP32 rounding of 1e-3 into the division by k rho)
-    const T dux = (usx - cst.urx) + defx / den, duy = (usy - cst.ury) + defy / den;
+    // would carry an FP32 rounding of 1e-3 into the division by k rho);
     // G = -(chi/eta)(j - rho u_s)/(1 + k)
-    const T pen = (T)2 * k;
-    pen_x = -pen * defx / ((T)1 + k);
-    pen_y = -pen * defy / ((T)1 + k);
+    T ex, ey;
+    if constexpr (sizeof(S) == 2) {
+      ex = defx / den;
+      ey = defy / den;
+      const T pen = (T)2 * k;
+      pen_x = -pen * defx / ((T)1 + k);
+      pen_y = -pen * defy / ((T)1 + k);
+    } else {
+      const T inv = N::get(vrcp(Val<V>::splat(den)));
+      ex = defx * inv;
+      ey = defy * inv;
+      pen_x = cst.pen * defx;
+      pen_y = cst.pen * defy;
+    }
+    const T dux = (usx - cst.urx) + ex, duy = (usy - cst.ury) + ey;
     const V vx = Val<V>::splat(dux), vy = Val<V>::splat(duy);
     const V gx = Val<V>::splat(bfx + pen_x), gy = Val<V>::splat(bfy + pen_y);
     if constexpr (sizeof(S) == 2) {
       collide16<true>(hv, drho, vx, vy, gx, gy, cst, ov);
     } else {
       // rho u - u_ref with the penalized velocity
-      const V ux = Val<V>::splat(usx + defx / den), uy = Val<V>::splat(usy + defy / den);
+      const V ux = Val<V>::splat(usx + ex), uy = Val<V>::splat(usy + ey);
       collide<V, true>(hv, m, vfma(drho, ux, vx), vfma(drho, uy, vy), ux, uy, vx, vy, gx, gy, cst, ov);
     }
   }
@@ -1038,13 +1149,21 @@ __device__ __forceinline__ void edge_pops(const S *src, const typename Store<S>:
   for (int a = 0; a < 9; ++a) h[a] = pre_pop<S, kGather>(src, prev, L, a, i, j);
 }
 
+// What a node of the force region leaves for its warp's force terms: its
+// post-collision values, links and penalization force.
+template <typename T>
+struct NodeForces {
+  T o[9], pen_x = 0, pen_y = 0;
+  uint32_t links = 0;
+  bool solid = false;
+};
+
 // One node of the special kernel: pull (with the side conditions where
-// needed), keep the outlet column, update, store, and the MEM link terms of
-// an interface node of the force region.
+// needed), keep the outlet column, update and store.
 template <typename S, bool kGather>
 __device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bool in_reg,
-                                             const TileMask *tm, FixAcc<typename Store<S>::T> &acc,
-                                             FixAcc<typename Store<S>::T> &vol) {
+                                             const TileMask *tm, int tx, int ty,
+                                             NodeForces<typename Store<S>::T> &nf) {
   using T = typename Store<S>::T;
   const Lattice &L = p.L;
   const S *__restrict__ src = static_cast<const S *>(p.src);
@@ -1070,19 +1189,21 @@ __device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bo
   if (tm) {
     // a moving body's tile: its mask byte from the tile's predicate, kept in
     // chi for the read-backs
-    m = tile_mask_byte(L, *tm, i, j, threadIdx.x, threadIdx.y);
+    m = tile_mask_byte(L, *tm, i, j, tx, ty);
     p.chi[node] = m;
   } else {
     m = p.chi[node];
   }
   // FP64's long update hides the links' loads; elsewhere only interface nodes
   // look for theirs
-  const uint32_t links = in_reg && ((sizeof(S) == 8 && !tm) || (m & kInterface))
-                             ? node_links(p, i, j, m & kSolid, tm)
-                             : 0u;
-  T o[9], pen_x, pen_y;
-  const bool bad = L.has_bf ? update_node<S, true>(h, m, i, j, L, p.body_src, Consts<T>(p), o, pen_x, pen_y)
-                            : update_node<S, false>(h, m, i, j, L, p.body_src, Consts<T>(p), o, pen_x, pen_y);
+  if (in_reg && ((sizeof(S) == 8 && !tm) || (m & kInterface)))
+    nf.links = node_links(p, i, j, m & kSolid, tm, tx, ty);
+  nf.solid = m & kSolid;
+  T(&o)[9] = nf.o;
+  const Consts<T> cst(p);
+  const bool bad =
+      L.has_bf ? update_node<S, true>(h, m, i, j, L, p.body_src, cst, o, nf.pen_x, nf.pen_y)
+               : update_node<S, false>(h, m, i, j, L, p.body_src, cst, o, nf.pen_x, nf.pen_y);
   if (sizeof(S) == 2 && p.sr) {
     const SrBits r(sr_level(p), (uint32_t)node >> 1);
 #pragma unroll
@@ -1093,13 +1214,6 @@ __device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bo
     for (int a = 0; a < 9; ++a)
       store_pop<S, false>(dst + (int64_t)a * L.plane + node, o[a], nullptr, a, (uint32_t)node);
   }
-  if (links) {
-    Offsets<T> post;
-#pragma unroll
-    for (int a = 0; a < 9; ++a) post.h[a] = o[a];
-    acc = mem_terms<T>(p, post, i, j, m & kSolid, links);
-  }
-  if (in_reg && (m & kSolid)) vol = vol_terms<T>(BodyRef<T>(*p.body_src), i, j, pen_x, pen_y);
   return bad;
 }
 
@@ -1117,24 +1231,29 @@ template <typename S>
 constexpr int kSpecialMinBlocks = sizeof(S) <= 4 ? 4 : 1;
 
 template <typename S, bool kGather, int kMinBlocks>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) special_kernel(const StepArgs p) {
+__global__ void __launch_bounds__(kThreads / kSlices<S>, kMinBlocks)
+    special_kernel(const StepArgs p) {
   using T = typename Store<S>::T;
+  constexpr int kBlock = kThreads / kSlices<S>;
   __shared__ int is_last;
   __shared__ TileMask tmask;
   __shared__ RigidConst rigid;
+  // (the capped form runs beside other lattices' bulk kernels)
+  constexpr bool kList = kMinBlocks == 1;
+  __shared__ LinkList<T> lists[kList ? kBlock / 32 : 1];
   const Lattice &L = p.L;
-  const int tid = threadIdx.y * kTileX + threadIdx.x;
+  const int b = blockIdx.x / kSlices<S>;
+  const Slice slice{(int)(blockIdx.x % kSlices<S>) * kBlock, kBlock};
+  const int tid = slice.first + threadIdx.x;  // within the tile's nodes
   const ForceRegion reg = *p.reg_src;
-  const int b = blockIdx.x;
   if (p.sr && b == 0 && tid == 0) *p.rng_dst = *p.rng_src + 1ull;  // the next level's counter
-  if (p.finalize_prev && b == (int)gridDim.x - 1) {
+  if (p.finalize_prev && b == (int)(gridDim.x / kSlices<S>) - 1) {
     // the previous step's force sums, beside this step's work
-    finalize<T>(p);
+    if (slice.first == 0) finalize<T>(p);
     return;
   }
-
-  if (!p.defer && tid >= kThreads - 32 && tid < kThreads - 29 && p.body_src->moving)
-    rigid_const(*p.body_src, rigid, tid - (kThreads - 32));
+  if (!p.defer && threadIdx.x >= kBlock - 3 && p.body_src->moving)
+    rigid_const(*p.body_src, rigid, threadIdx.x - (kBlock - 3));
 
   if (b < p.sim_blocks) {
     // ---- SIM points of this level ----
@@ -1158,8 +1277,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) special_kernel(const Ste
       const int ti = i / kTileX, tj = j / kTileY;
       const bool in_reg = ti >= reg.ti0 && ti <= reg.ti1 && tj >= reg.tj0 && tj <= reg.tj1;
       if (!in_reg) {
-        FixAcc<T> unused, unused_vol;
-        bad = special_node<S, kGather>(p, i, j, false, nullptr, unused, unused_vol);
+        NodeForces<T> unused;
+        bad = special_node<S, kGather>(p, i, j, false, nullptr, 0, 0, unused);
       }
     }
     if (__any_sync(kFull, bad) && (tid & 31) == 0) atomicOr(p.status, kStatusUnstable);
@@ -1179,21 +1298,26 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) special_kernel(const Ste
       tj = reg.tj0 + k / rw;
     }
     const bool in_reg = ti >= reg.ti0 && ti <= reg.ti1 && tj >= reg.tj0 && tj <= reg.tj1;
-    const int i = ti * kTileX + threadIdx.x;
-    const int j = tj * kTileY + threadIdx.y;
+    const int tx = tid % kTileX, ty = tid / kTileX;
+    const int i = ti * kTileX + tx, j = tj * kTileY + ty;
     // a moving body: the region tiles rasterise its mask at this level
     const bool raster = p.raster && in_reg;  // uniform over the block
     if (raster) {
-      tile_solid(p, ti, tj, tmask);
+      tile_solid(p, ti, tj, slice, tmask);
       __syncthreads();
     }
     bool bad = false;
-    FixAcc<T> acc, vol;
+    NodeForces<T> nf;
     if (i < L.nx && j < L.ny)
-      bad = special_node<S, kGather>(p, i, j, in_reg, raster ? &tmask : nullptr, acc, vol);
+      bad = special_node<S, kGather>(p, i, j, in_reg, raster ? &tmask : nullptr, tx, ty, nf);
+    __syncwarp();
     if (__any_sync(kFull, bad) && (tid & 31) == 0) atomicOr(p.status, kStatusUnstable);
     if (!in_reg) return;  // uniform over the block
-    warp_add(acc, p.acc, 0);
+    LinkList<T> *list = nullptr;
+    if constexpr (kList) list = lists + (threadIdx.x >> 5);
+    warp_add(mem_terms<T, kList>(p, nf.o, i, j, nf.solid, nf.links, list), p.acc, 0);
+    FixAcc<T> vol;
+    if (nf.solid) vol = vol_terms<T>(BodyRef<T>(*p.body_src), i, j, nf.pen_x, nf.pen_y);
     warp_add(vol, p.acc, 6);
   }
 
@@ -1201,9 +1325,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) special_kernel(const Ste
 
   // ---- ticket among the SIM blocks and the force-region tiles ----
   __syncthreads();
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     __threadfence();
-    const unsigned int expected = (unsigned int)(p.sim_blocks + reg.count);
+    const unsigned int expected = (unsigned int)(kSlices<S> * (p.sim_blocks + reg.count));
     const unsigned int prev = atomicAdd(p.ticket, 1u);
     is_last = (prev == expected - 1);
   }
@@ -1541,16 +1665,17 @@ __global__ void __launch_bounds__(32 * kTileY, 12) bulk16x4_kernel(const StepArg
 template <typename S, bool kGather>
 cudaError_t special_t(const StepArgs &a, cudaStream_t s) {
   const int tiles = a.all_tiles ? a.ntiles_x * a.ntiles_y : a.edge_blocks + a.region_slots;
-  const int blocks = a.sim_blocks + tiles + (a.finalize_prev ? 1 : 0);
+  const int blocks = (a.sim_blocks + tiles + (a.finalize_prev ? 1 : 0)) * kSlices<S>;
+  constexpr int kBlock = kThreads / kSlices<S>;
   if (a.raster || kSpecialMinBlocks<S> == 1)
-    special_kernel<S, kGather, 1><<<blocks, dim3(kTileX, kTileY), 0, s>>>(a);
+    special_kernel<S, kGather, 1><<<blocks, kBlock, 0, s>>>(a);
   else
-    special_kernel<S, kGather, kSpecialMinBlocks<S>><<<blocks, dim3(kTileX, kTileY), 0, s>>>(a);
+    special_kernel<S, kGather, kSpecialMinBlocks<S>><<<blocks, kBlock, 0, s>>>(a);
   return cudaGetLastError();
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads) finalize_kernel(const StepArgs p) {
+__global__ void __launch_bounds__(64) finalize_kernel(const StepArgs p) {
   finalize<T>(p);
 }
 
@@ -1563,11 +1688,12 @@ __global__ void __launch_bounds__(kThreads) mask_kernel(const StepArgs p) {
   if (k >= reg.count) return;
   const int rw = reg.ti1 - reg.ti0 + 1;
   const int ti = reg.ti0 + k % rw, tj = reg.tj0 + k / rw;
-  tile_solid(p, ti, tj, tm);
+  tile_solid(p, ti, tj, Slice{0, kThreads}, tm);
   __syncthreads();
-  const int i = ti * kTileX + threadIdx.x, j = tj * kTileY + threadIdx.y;
+  const int tx = threadIdx.x % kTileX, ty = threadIdx.x / kTileX;
+  const int i = ti * kTileX + tx, j = tj * kTileY + ty;
   if (i < p.L.nx && j < p.L.ny)
-    p.chi[(int64_t)j * p.L.pitch + i] = tile_mask_byte(p.L, tm, i, j, threadIdx.x, threadIdx.y);
+    p.chi[(int64_t)j * p.L.pitch + i] = tile_mask_byte(p.L, tm, i, j, tx, ty);
 }
 
 template <typename S, bool kForce, bool kSR>
@@ -1634,14 +1760,14 @@ cudaError_t launch_pair(int dtype, const StepArgs &a, cudaStream_t s) {
 
 cudaError_t launch_finalize(int dtype, const StepArgs &a, cudaStream_t s) {
   if (dtype == VPLBM_F64)
-    finalize_kernel<double><<<1, dim3(kTileX, kTileY), 0, s>>>(a);
+    finalize_kernel<double><<<1, 64, 0, s>>>(a);
   else
-    finalize_kernel<float><<<1, dim3(kTileX, kTileY), 0, s>>>(a);
+    finalize_kernel<float><<<1, 64, 0, s>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_mask(const StepArgs &a, cudaStream_t s) {
-  mask_kernel<<<a.region_slots, dim3(kTileX, kTileY), 0, s>>>(a);
+  mask_kernel<<<a.region_slots, kThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -60,6 +60,15 @@ constexpr uint8_t kInterface = 2;  // some lattice neighbour has the other phase
 constexpr int kStatusUnstable = 1;
 constexpr int kStatusSimMissing = 2;
 
+// 1/a for a normal a by one third-order iteration from the hardware's
+// approximation (relative error below 2^-20, cubed): three FMAs
+__device__ __forceinline__ double near_rcp(double a) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  const double e = fma(-a, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // ---------------------------------------------------------------------------
 // storage conversions: populations are stored as offsets h = f - w
 // ---------------------------------------------------------------------------
@@ -193,13 +202,29 @@ template <typename T>
 struct Fix;
 template <>
 struct Fix<double> {
-  // two words: round(v 2^30) and the exact remainder at 2^-82 (|sum| < 2^33)
+  // two words, units 2^-30 and 2^-82 (|sum| < 2^33): the magnitude rounded down
+  // to a multiple of 2^-82, both words with the value's sign.  Integer
+  // operations on the value's bits, which have their own lanes: GB300's FP64
+  // conversions wait for its two FP64 lanes per SM.
   static constexpr int kWords = 2;
   static __device__ __forceinline__ void split(double v, long long (&w)[2]) {
-    const long long hi = __double2ll_rn(v * 1073741824.0);              // 2^30
-    const double rem = v - (double)hi * 9.313225746154785e-10;          // exact
-    w[0] = hi;
-    w[1] = __double2ll_rn(rem * 4835703278458516698824704.0);           // 2^82
+    const long long bits = __double_as_longlong(v);
+    const int e = (int)(bits >> 52) & 0x7ff;
+    const unsigned long long m = ((unsigned long long)bits & 0xfffffffffffffull) | 0x10000000000000ull;
+    // |v| = m 2^(e - 1075); hi = |v| 2^30 rounded down, lo = the rest in 2^-82
+    const int s = 1045 - e;  // hi = m >> s; |v| < 2^33 keeps s >= -10
+    unsigned long long hi, lo;
+    if (s > 0) {
+      hi = s < 64 ? m >> s : 0ull;
+      const unsigned long long rest = s < 64 ? m & ((1ull << s) - 1ull) : m;
+      lo = s <= 52 ? rest << (52 - s) : (s < 116 ? rest >> (s - 52) : 0ull);
+    } else {
+      hi = m << min(-s, 63);
+      lo = 0ull;
+    }
+    if (e == 0) hi = lo = 0ull;  // zero (denormals round to it)
+    w[0] = bits < 0 ? -(long long)hi : (long long)hi;
+    w[1] = bits < 0 ? -(long long)lo : (long long)lo;
   }
   static __host__ __device__ double value(long long w0, long long w1) {
     return (double)w0 * 9.313225746154785e-10 + (double)w1 * 2.0679515313825692e-25;
@@ -502,7 +527,8 @@ struct StepArgs {
   double half_pen;         // dt/(2 eta)
   double tau_plus;
   double sim_const[3];     // -(1/3) sum S n and its moment: the SIM constant part
-  float f_s_plus, f_s_minus, f_a_plus, f_a_minus, f_half_pen, f_sim_s;
+  double pen;              // -(1/eta)/(1 + half_pen): G = pen (j - rho u_s)
+  float f_s_plus, f_s_minus, f_a_plus, f_a_minus, f_half_pen, f_sim_s, f_pen;
   // the collision's folded coefficients (CollideC), in either precision
   CollideC<double> coll;
   CollideC<float> f_coll;
@@ -609,17 +635,17 @@ template <typename T>
 struct Consts;
 template <>
 struct Consts<double> : CollideC<double> {
-  double a_plus, a_minus, half_pen, sim_s, urx, ury;
+  double a_plus, a_minus, half_pen, pen, sim_s, urx, ury;
   __device__ __forceinline__ explicit Consts(const StepArgs &p)
       : CollideC<double>(p.coll), a_plus(p.a_plus), a_minus(p.a_minus), half_pen(p.half_pen),
-        sim_s(1.0 - 0.5 / p.tau_plus), urx(p.L.ur[0]), ury(p.L.ur[1]) {}
+        pen(p.pen), sim_s(1.0 - 0.5 / p.tau_plus), urx(p.L.ur[0]), ury(p.L.ur[1]) {}
 };
 template <>
 struct Consts<float> : CollideC<float> {
-  float s_plus, s_minus, a_plus, a_minus, half_pen, sim_s, urx, ury;
+  float s_plus, s_minus, a_plus, a_minus, half_pen, pen, sim_s, urx, ury;
   __device__ __forceinline__ explicit Consts(const StepArgs &p)
       : CollideC<float>(p.f_coll), s_plus(p.f_s_plus), s_minus(p.f_s_minus), a_plus(p.f_a_plus), a_minus(p.f_a_minus),
-        half_pen(p.f_half_pen), sim_s(p.f_sim_s), urx(p.L.ur_f[0]), ury(p.L.ur_f[1]) {}
+        half_pen(p.f_half_pen), pen(p.f_pen), sim_s(p.f_sim_s), urx(p.L.ur_f[0]), ury(p.L.ur_f[1]) {}
 };
 
 // tile range of the force region of a body whose bounding box is
