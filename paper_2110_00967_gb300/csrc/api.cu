@@ -235,10 +235,12 @@ int default_sim_points(const vplbm_body &b) {
 
 }  // namespace
 
-// How a call's step graphs step: one step per launch pair, or two steps per
-// launch (pair.cuh) with the run lengths of a lattice alone or of one among
-// many.  The results are the same bit for bit.
-enum StepMode { kSingle = 0, kPairAlone = 1, kPairBatch = 2, kStepModes = 3 };
+// How a call's step graphs step: one step per special and bulk kernel, or two
+// steps per launch (pair.cuh), each as one lattice among many or alone.  The
+// results are the same bit for bit.
+enum StepMode { kSingle = 0, kSingleAlone, kPair, kPairAlone, kStepModes };
+bool takes_pairs(int mode) { return mode >= kPair; }
+bool is_alone(int mode) { return mode == kSingleAlone || mode == kPairAlone; }
 
 struct vplbm_ctx {
   vplbm_config cfg;
@@ -391,15 +393,13 @@ StepArgs step_args(vplbm_ctx *c, int src, bool do_sim) {
   a.pen = -2.0 * c->half_pen / (1.0 + c->half_pen);
   a.f_pen = (float)a.pen;
   a.f_sim_s = (float)(1.0 - 0.5 / a.tau_plus);
-  a.tile_w = kTileX;
   a.ntiles_x = (c->L.nx + kTileX - 1) / kTileX;
   a.ntiles_y = (c->L.ny + kTileY - 1) / kTileY;
   a.all_tiles = 0;
-  a.n_edge = edge_count(c->L.nx, c->L.ny);
-  a.edge_blocks = (a.n_edge + kThreads - 1) / kThreads;
+  a.edge_blocks = (edge_count(c->L.nx, c->L.ny) + kThreads - 1) / kThreads;
   a.region_slots = c->region_slots;
-  a.region_capacity = kRegionCapacity;
   a.raster = c->body_host.moving ? 1 : 0;
+  a.uncapped = c->body_host.moving || is_alone(c->mode) ? 1 : 0;
   a.sr = stochastic_dtype(c->cfg.dtype) ? 1 : 0;
   a.rng_src = c->rng + src;
   a.rng_dst = c->rng + (1 - src);
@@ -477,7 +477,7 @@ constexpr int64_t kPairSmall = 700000;
 // 13.05 / 12.8; 512 x 256 (6 / 12 / 16 rows) 3.9 / 4.4 / 5.0.
 int pair_rows(const vplbm_ctx *c) {
   if (c->bulk_variant > 0) return c->bulk_variant == 1 ? 12 : 24;
-  if (c->mode == kPairBatch) return 20;
+  if (!is_alone(c->mode)) return 20;
   return (int64_t)c->L.nx * c->L.ny < kPairSmall || elem_bytes(c->cfg.dtype) == 2 ? 6 : 8;
 }
 
@@ -498,9 +498,9 @@ cudaError_t queue_pair(vplbm_ctx *c, cudaStream_t s, int src, bool do_sim) {
 // a graph of n steps: its moves of the state to the other buffer (one per
 // pair of steps, or per step), and its launches (one per pair, two per single
 // step, and those that end the run)
-int graph_moves(const vplbm_ctx *c, int n) { return c->mode != kSingle ? n / 2 + (n & 1) : n; }
+int graph_moves(const vplbm_ctx *c, int n) { return takes_pairs(c->mode) ? n / 2 + (n & 1) : n; }
 int graph_launches(const vplbm_ctx *c, int n) {
-  return (c->mode != kSingle ? n / 2 + 2 * (n & 1) : 2 * n) + 1 + (c->body_host.moving ? 1 : 0);
+  return (takes_pairs(c->mode) ? n / 2 + 2 * (n & 1) : 2 * n) + 1 + (c->body_host.moving ? 1 : 0);
 }
 // the buffer holding the state after a graph of n steps from buffer cur
 int buffer_after(const vplbm_ctx *c, int cur, int n) { return cur ^ (graph_moves(c, n) & 1); }
@@ -583,10 +583,10 @@ constexpr int64_t kPair16Nodes = 1500000;
 constexpr int64_t kPairBatchNodes = 4000000;  // a full GPU: longer runs
 void choose_mode(vplbm_ctx *c, int64_t call_nodes) {
   const int64_t own = (int64_t)c->L.nx * c->L.ny;
-  if (!c->pair_ok || (elem_bytes(c->cfg.dtype) == 2 && call_nodes > kPair16Nodes))
-    c->mode = kSingle;
-  else
-    c->mode = call_nodes >= 2 * own && call_nodes > kPairBatchNodes ? kPairBatch : kPairAlone;
+  const bool pairs =
+      c->pair_ok && !(elem_bytes(c->cfg.dtype) == 2 && call_nodes > kPair16Nodes);
+  const bool alone = call_nodes < 2 * own || (pairs && call_nodes <= kPairBatchNodes);
+  c->mode = pairs ? (alone ? kPairAlone : kPair) : (alone ? kSingleAlone : kSingle);
 }
 // ... for a lattice stepped by itself
 void choose_mode(vplbm_ctx *c) { choose_mode(c, (int64_t)c->L.nx * c->L.ny); }
@@ -630,7 +630,7 @@ vplbm_status ensure_graphs(vplbm_ctx *c, cudaStream_t s) {
       const int cur = c->cur;
       c->cur = buffer_after(c, p, n);  // where the graph ends, for the end-of-run work
       for (int q = 0, u = p; q < n && e == cudaSuccess; u ^= 1)
-        if (c->mode != kSingle && n - q >= 2) {
+        if (takes_pairs(c->mode) && n - q >= 2) {
           e = queue_pair(c, c->capture_stream, u, do_sim);
           q += 2;
         } else {

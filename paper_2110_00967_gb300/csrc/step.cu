@@ -539,44 +539,42 @@ __device__ void finalize(const StepArgs &p) {
   const int tid = threadIdx.x;
   const int rows = p.prev_rows;
   __shared__ double tot[2][kAccSlots];
-  __shared__ long long step_s;
   const bool do_sim = p.prev_sim != 0;
-  // a warp per row, or one warp for both in turn
-  const int col = tid & 31, stride = blockDim.x >> 5;
-  for (int row = tid >> 5; row < rows; row += stride)
-    if (col < kAccSlots) {
-      const unsigned long long *acc = row ? p.acc2_prev : p.acc_prev;
-      const long long w0 = (long long)__ldcg(acc + 2 * col);
-      const long long w1 = (long long)__ldcg(acc + 2 * col + 1);
-      double v = Fix<T>::value(w0, w1);
-      if (col >= 3 && col < 6) v += p.sim_const[col - 3];
-      tot[row][col] = v;
-    }
-  if (tid == 31) step_s = __ldcg(p.dev_step);
-  __syncthreads();
-  for (int row = tid >> 5; row < rows; row += stride) {
-    if (col < kHistCols) {
+  // A warp per row (or one warp for both in turn).  Each row's words and the
+  // step counter are loaded together; the code is kept short, since a lone
+  // finalizing launch mostly waits for its instructions.
+  const int lane = tid & 31;
+#pragma unroll 1
+  for (int row = tid >> 5; row < rows; row += blockDim.x >> 5) {
+    unsigned long long *acc = row ? p.acc2_prev : p.acc_prev;
+    long long step = 0;
+    double v = 0.0;
+    if (lane < kHistCols) {
+      const long long w0 = (long long)__ldcg(acc + 2 * lane);
+      const long long w1 = (long long)__ldcg(acc + 2 * lane + 1);
+      step = __ldcg(p.dev_step) + row;
+      v = Fix<T>::value(w0, w1);
+      const bool is_sim = lane >= 3 && lane < 6;
+      if (is_sim) v += p.sim_const[lane - 3];
       // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
-      const bool have = col < 3 || col >= 6 || do_sim;
-      p.hist[kHistCols * ((step_s + row) % p.hist_len) + col] =
-          have ? tot[row][col] : __longlong_as_double(0x7ff8000000000000LL);
+      p.hist[kHistCols * (step % p.hist_len) + lane] =
+          !is_sim || do_sim ? v : __longlong_as_double(0x7ff8000000000000LL);
+      tot[row][lane] = v;
     }
-    // every read of the sums above precedes the barrier
-    if (col < kAccWords) (row ? p.acc2_prev : p.acc_prev)[col] = 0ull;
+    __syncwarp();
+    if (lane < kAccWords) acc[lane] = 0ull;
   }
-  if (tid >= 16 && tid < 22) {
-    const int q = tid - 16;
-    if (q < 3 || do_sim) {
-      double v = p.sums[q] + tot[0][q];
-      if (rows > 1) v += tot[1][q];
-      p.sums[q] = v;
+  __syncthreads();
+  if (tid < 6) {
+    if (tid < 3 || do_sim) {
+      double v = p.sums[tid] + tot[0][tid];
+      if (rows > 1) v += tot[1][tid];
+      p.sums[tid] = v;
     }
-  } else if (tid == 22) {
-    p.counts[0] += rows;
-  } else if (tid == 23 && do_sim) {
-    p.counts[1] += rows;
-  } else if (tid == 24) {
-    *p.dev_step = step_s + rows;
+  } else if (tid == 6 || (tid == 7 && do_sim)) {
+    p.counts[tid - 6] += rows;
+  } else if (tid == 8) {
+    *p.dev_step += rows;  // read above by both rows before the barrier
   }
 }
 
@@ -623,10 +621,10 @@ __device__ void tail(const StepArgs &p, const ForceRegion &reg, const RigidConst
     ForceRegion nreg = reg;
     bool ok = true;
     if (old_b.moving) {
-      nreg = make_region(p.L, x, y, 0.5 * old_b.length, p.ntiles_x, p.ntiles_y, p.tile_w);
+      nreg = make_region(p.L, x, y, 0.5 * old_b.length, p.ntiles_x, p.ntiles_y, kTileX);
       // the body left the lattice or moved a node in one step: keep it where
       // it was and flag the run as unstable
-      ok = !(nreg.error || nreg.count > p.region_slots || nreg.count > p.region_capacity ||
+      ok = !(nreg.error || nreg.count > p.region_slots || nreg.count > kRegionCapacity ||
              fabs(x - old_b.xg) >= 1.0 || fabs(y - old_b.yg) >= 1.0);
     }
     if (old_b.moving && ok) {
@@ -1223,14 +1221,15 @@ __device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bo
 // ---------------------------------------------------------------------------
 // The special kernels of lattices stepped side by side share the SMs with the
 // bulk kernels, whose bytes in flight need the register file: for a fixed
-// body with FP32 compute the special kernel is capped at 64 registers (four
-// blocks per SM), at the price of a few spilled values.  A moving body's
-// special kernel is on the step's critical path (its force feeds the next
-// step), so it keeps all the registers it wants (kMinBlocks 1).
+// body with FP32 compute the special kernel is then capped at 64 registers (four
+// blocks per SM), at the price of a few spilled values.  A moving body's special
+// kernel is on the step's critical path (its force feeds the next step), and so
+// is that of a lattice stepped alone: they keep all the registers they want
+// (kMinBlocks 1).
 template <typename S>
 constexpr int kSpecialMinBlocks = sizeof(S) <= 4 ? 4 : 1;
 
-template <typename S, bool kGather, int kMinBlocks>
+template <typename S, bool kGather, int kMinBlocks, bool kList>
 __global__ void __launch_bounds__(kThreads / kSlices<S>, kMinBlocks)
     special_kernel(const StepArgs p) {
   using T = typename Store<S>::T;
@@ -1238,8 +1237,6 @@ __global__ void __launch_bounds__(kThreads / kSlices<S>, kMinBlocks)
   __shared__ int is_last;
   __shared__ TileMask tmask;
   __shared__ RigidConst rigid;
-  // (the capped form runs beside other lattices' bulk kernels)
-  constexpr bool kList = kMinBlocks == 1;
   __shared__ LinkList<T> lists[kList ? kBlock / 32 : 1];
   const Lattice &L = p.L;
   const int b = blockIdx.x / kSlices<S>;
@@ -1271,7 +1268,7 @@ __global__ void __launch_bounds__(kThreads / kSlices<S>, kMinBlocks)
     // ---- one edge node per thread (nodes of force-region tiles excluded) ----
     const int e = (b - p.sim_blocks) * kThreads + tid;
     bool bad = false;
-    if (e < p.n_edge) {
+    if (e < edge_count(L.nx, L.ny)) {
       int i, j;
       edge_node(e, L.nx, L.ny, i, j);
       const int ti = i / kTileX, tj = j / kTileY;
@@ -1667,10 +1664,12 @@ cudaError_t special_t(const StepArgs &a, cudaStream_t s) {
   const int tiles = a.all_tiles ? a.ntiles_x * a.ntiles_y : a.edge_blocks + a.region_slots;
   const int blocks = (a.sim_blocks + tiles + (a.finalize_prev ? 1 : 0)) * kSlices<S>;
   constexpr int kBlock = kThreads / kSlices<S>;
-  if (a.raster || kSpecialMinBlocks<S> == 1)
-    special_kernel<S, kGather, 1><<<blocks, kBlock, 0, s>>>(a);
+  if (a.raster || sizeof(S) == 8)
+    special_kernel<S, kGather, 1, true><<<blocks, kBlock, 0, s>>>(a);
+  else if (a.uncapped)
+    special_kernel<S, kGather, 1, false><<<blocks, kBlock, 0, s>>>(a);
   else
-    special_kernel<S, kGather, kSpecialMinBlocks<S>><<<blocks, kBlock, 0, s>>>(a);
+    special_kernel<S, kGather, kSpecialMinBlocks<S>, false><<<blocks, kBlock, 0, s>>>(a);
   return cudaGetLastError();
 }
 

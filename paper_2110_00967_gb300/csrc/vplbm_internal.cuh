@@ -515,7 +515,6 @@ struct StepArgs {
   int32_t sim_per_block; // SIM points per block (a multiple of 32)
   double *hist;          // [hist_len][6]
   int32_t hist_len;
-  int32_t pad0;
   double *sums;          // [6]
   long long *counts;     // [2]
   long long *dev_step;   // steps completed
@@ -533,15 +532,13 @@ struct StepArgs {
   CollideC<double> coll;
   CollideC<float> f_coll;
   int32_t ntiles_x, ntiles_y;
-  int32_t region_capacity;  // most force-region tiles a step may hold
-  int32_t tile_w;           // nodes along x of one tile
   int32_t all_tiles;        // 1: the special kernel updates every tile (first step)
-  int32_t n_edge;           // nodes on the lattice edges
   int32_t edge_blocks;      // special-kernel blocks for the edge nodes
   int32_t region_slots;     // special-kernel blocks reserved for force-region tiles
   int32_t raster;           // 1 (a moving body): the force-region tiles rasterise chi
                             // from body_src themselves, and SIM tests nodes with the
                             // predicate instead of reading chi
+  int32_t uncapped;         // 1: the special kernel may use all the registers it wants
   int32_t sr;               // 1: 16-bit stores round stochastically
   // ---- a pair of steps in one launch (fixed or no body; api.cu: pair_ok) ----
   unsigned long long *acc2;       // sums of the pair's second step
