@@ -51,7 +51,7 @@ size_t elem_bytes(int dtype) {
 
 struct Layout {
   size_t buf[2], prev[2], chi, sim_pts, sim_nodes, hist, body[2], region[2], sums, counts,
-      dev_step, ticket, status, acc, rng, snap_end, acc2, total;
+      dev_step, rigid, status, acc, rng, snap_end, acc2, total;
 };
 
 int effective_max_sim(const vplbm_config &c) { return c.max_sim_points > 0 ? c.max_sim_points : 4096; }
@@ -93,7 +93,7 @@ Layout make_layout(const vplbm_config &c) {
   l.sums = take(6 * sizeof(double));
   l.counts = take(2 * sizeof(long long));
   l.dev_step = take(sizeof(long long));
-  l.ticket = take(sizeof(unsigned int));
+  l.rigid = take(sizeof(RigidConst));
   l.status = take(sizeof(int32_t));
   l.acc = take(2 * kAccWords * sizeof(unsigned long long));  // by step parity
   l.rng = take(2 * sizeof(unsigned long long));                // rounding counter, by parity
@@ -265,13 +265,15 @@ struct vplbm_ctx {
   double *sums;
   long long *counts;
   long long *dev_step;
-  unsigned int *ticket;
+  RigidConst *rigid;
   int32_t *status;
   int cur = 0;        // buffer holding the state
   bool pre = true;    // the state is a pre-collision field (first step reads in place)
   bool pending = false;      // the last queued step's force sums still await finalizing
   bool pending_sim = false;  // ... and that step evaluated SIM
   int pending_rows = 1;      // ... of one step, or of the two of a pair
+  int turn = 0;              // a moving body's set of sums for the next step
+  RigidConst rigid_host{};
   bool pair_ok = false;      // two steps per launch are possible (pair_plan)
   int mode = 0;              // how the current call steps (StepMode)
   int box[4] = {0, -1, 0, -1};  // nodes around the body (StepArgs::box)
@@ -364,11 +366,20 @@ StepArgs step_args(vplbm_ctx *c, int src, bool do_sim) {
   a.prev_dst = c->prev[1 - src];
   a.chi = c->chi;
   a.body_src = c->body[src];
-  a.body_dst = c->body[1 - src];
+  a.body_prev = c->body[1 - src];
+  a.rigid = c->rigid;
   a.reg_src = c->region[src];
   a.reg_dst = c->region[1 - src];
   a.acc = c->acc + kAccWords * src;
   a.acc_prev = c->acc + kAccWords * (1 - src);
+  if (c->body_host.moving) {
+    // every block of a launch reads the previous step's sums while this step's
+    // are added: three sets in turn, the next one cleared meanwhile
+    unsigned long long *sets[3] = {c->acc, c->acc + kAccWords, c->acc2};
+    a.acc = sets[c->turn];
+    a.acc_prev = sets[(c->turn + 2) % 3];
+    a.acc_next = sets[(c->turn + 1) % 3];
+  }
   a.acc2 = c->acc2 + kAccWords * src;
   a.acc2_prev = c->acc2 + kAccWords * (1 - src);
   a.prev_rows = c->pending_rows;
@@ -385,7 +396,6 @@ StepArgs step_args(vplbm_ctx *c, int src, bool do_sim) {
   a.sums = c->sums;
   a.counts = c->counts;
   a.dev_step = c->dev_step;
-  a.ticket = c->ticket;
   a.status = c->status;
   a.coll = collide_coeffs<double>(c->s_plus, c->s_minus);
   a.f_coll = collide_coeffs<float>(c->s_plus, c->s_minus);
@@ -424,13 +434,15 @@ bool sim_due(const vplbm_ctx *c, long long step) {
 // blocks) runs on the context's high-priority side stream beside the bulk
 // kernel (all other nodes, bandwidth-bound) on s; the two write disjoint
 // nodes, and s waits for both before the next step.
-// Finalizes the force sums of the last queued step if they were deferred: one
-// block on s (history row, running sums, step counter).
+// Finalizes the force sums of the last queued step or pair, if pending: one
+// block on s (history rows, running sums, step counter, a moving body's state).
 cudaError_t flush_forces(vplbm_ctx *c, cudaStream_t s) {
   if (!c->pending) return cudaSuccess;
   StepArgs a = step_args(c, c->cur, false);  // acc_prev: the last step's sums
+  a.finalize_prev = 1;
   a.prev_sim = c->pending_sim ? 1 : 0;
   c->pending = false;
+  c->turn = 0;  // a moving body's sums are all clear now
   ++c->launches;
   return launch_finalize(storage_dtype(c->cfg.dtype), a, s);
 }
@@ -447,32 +459,31 @@ cudaError_t refresh_mask(vplbm_ctx *c, cudaStream_t s) {
 
 cudaError_t queue_step(vplbm_ctx *c, cudaStream_t s, int src, bool pre, bool do_sim) {
   if (c->body_host.moving) c->mask_stale = true;
-  if (pre) {
-    cudaError_t e = flush_forces(c, s);
-    StepArgs a = step_args(c, src, do_sim);
-    a.all_tiles = 1;
-    ++c->launches;
-    if (e == cudaSuccess) e = launch_special(storage_dtype(c->cfg.dtype), false, a, s);
-    return e;
-  }
+  cudaError_t e = cudaSuccess;
+  if (pre) e = flush_forces(c, s);
+  // the step's force sums are finalized by the next step's special kernel (one
+  // extra block beside its work) or by flush_forces
   StepArgs a = step_args(c, src, do_sim);
-  // a fixed body needs its force sums only after the call: the special kernel
-  // skips the ticket and tail, and the next step's special kernel (one extra
-  // block beside its work) or flush_forces finalizes them.  A moving body's
-  // update needs them within the step.
-  a.defer = c->body_host.moving ? 0 : 1;
   a.finalize_prev = c->pending ? 1 : 0;
   a.prev_sim = c->pending_sim ? 1 : 0;
-  cudaError_t e = cudaEventRecord(c->ev_fork, s);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
-  if (e == cudaSuccess) e = launch_special(storage_dtype(c->cfg.dtype), true, a, c->side);
-  if (e == cudaSuccess) e = cudaEventRecord(c->ev_join, c->side);
-  if (e == cudaSuccess) e = launch_bulk(storage_dtype(c->cfg.dtype), c->bulk_variant, a, s);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->ev_join, 0);
-  c->launches += 2;
-  c->pending = a.defer != 0;
+  a.all_tiles = pre ? 1 : 0;
+  const int st = storage_dtype(c->cfg.dtype);
+  if (pre) {
+    if (e == cudaSuccess) e = launch_special(st, false, a, s);
+    ++c->launches;
+  } else {
+    if (e == cudaSuccess) e = cudaEventRecord(c->ev_fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
+    if (e == cudaSuccess) e = launch_special(st, true, a, c->side);
+    if (e == cudaSuccess) e = cudaEventRecord(c->ev_join, c->side);
+    if (e == cudaSuccess) e = launch_bulk(st, c->bulk_variant, a, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->ev_join, 0);
+    c->launches += 2;
+  }
+  c->pending = true;
   c->pending_sim = do_sim;
   c->pending_rows = 1;
+  c->turn = (c->turn + 1) % 3;
   return e;
 }
 
@@ -492,7 +503,6 @@ int pair_rows(const vplbm_ctx *c) {
 // Two time steps in one launch on stream s (pair.cuh).
 cudaError_t queue_pair(vplbm_ctx *c, cudaStream_t s, int src, bool do_sim) {
   StepArgs a = step_args(c, src, do_sim);
-  a.defer = 1;
   a.finalize_prev = c->pending ? 1 : 0;
   a.prev_sim = c->pending_sim ? 1 : 0;
   a.pair_rows = pair_rows(c);
@@ -796,7 +806,7 @@ vplbm_status vplbm_create(const vplbm_config *cfg, void *dev_workspace, size_t b
   c->sums = (double *)(c->ws + lay.sums);
   c->counts = (long long *)(c->ws + lay.counts);
   c->dev_step = (long long *)(c->ws + lay.dev_step);
-  c->ticket = (unsigned int *)(c->ws + lay.ticket);
+  c->rigid = (RigidConst *)(c->ws + lay.rigid);
   c->status = (int32_t *)(c->ws + lay.status);
 
   Lattice &L = c->L;
@@ -1028,6 +1038,8 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   // histories, sums, counters, status
   VPLBM_CUDA(c, cudaMemsetAsync(c->ws + c->lay.hist, 0, c->lay.body[0] - c->lay.hist, s));
   VPLBM_CUDA(c, cudaMemsetAsync(c->ws + c->lay.sums, 0, c->lay.total - c->lay.sums, s));
+  c->rigid_host = b->moving ? rigid_const(c->body_host) : RigidConst{};
+  VPLBM_CUDA(c, cudaMemcpyAsync(c->rigid, &c->rigid_host, sizeof(RigidConst), cudaMemcpyHostToDevice, s));
   VPLBM_CUDA(c, cudaMemsetAsync(c->prev[0], 0, 3 * (size_t)L.ny * sizeof(double), s));
   VPLBM_CUDA(c, cudaMemsetAsync(c->prev[1], 0, 3 * (size_t)L.ny * sizeof(double), s));
   VPLBM_CUDA(c, cudaGetLastError());
@@ -1035,6 +1047,7 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   c->pre = true;
   c->steps = 0;
   c->pending = false;  // the accumulators were cleared with the other counters
+  c->turn = 0;
   c->mask_stale = false;
   c->has_body = true;
   return sync(c);
@@ -1455,6 +1468,8 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
   const char *in = static_cast<const char *>(host);
   VPLBM_CUDA(c, cudaMemcpyAsync(c->ws + c->lay.prev[0], in + hb, tb, cudaMemcpyHostToDevice, c->stream));
   VPLBM_CUDA(c, cudaMemcpyAsync(c->buf[h.cur], in + hb + tb, pb, cudaMemcpyHostToDevice, c->stream));
+  c->rigid_host = h.body_host.moving ? rigid_const(h.body_host) : RigidConst{};
+  VPLBM_CUDA(c, cudaMemcpyAsync(c->rigid, &c->rigid_host, sizeof(RigidConst), cudaMemcpyHostToDevice, c->stream));
   if (vplbm_status st = sync(c)) return st;
   c->body_cfg = h.body_cfg;
   c->body_host = h.body_host;
@@ -1476,6 +1491,7 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
   }
   c->pending = false;
   c->pending_sim = false;
+  c->turn = 0;
   c->mask_stale = false;
   c->has_body = true;
   drop_graphs(c);

@@ -319,7 +319,7 @@ __device__ __forceinline__ void pair_special(const StepArgs &p, const PairGrid &
     const int q = (b - (g.special - (p.finalize_prev ? 1 : 0) - g.sim1)) * kPairThreads + tid;
     FixAcc<float> acc;
     bool missing = false;
-    if (q < p.n_sim) acc = sim_point<S, true>(p, src, body->xg, body->yg, q, missing);
+    if (q < p.n_sim) acc = sim_point<S, true>(p, src, *body, q, missing);
     if (__any_sync(kFull, missing) && lane == 0) atomicOr(p.status, kStatusSimMissing);
     warp_add(acc, p.acc, 3);
     return;
@@ -481,7 +481,7 @@ __device__ __forceinline__ void pair_special(const StepArgs &p, const PairGrid &
     if (!frame) {
       // from the values before rounding
       unsigned long long *sums = second ? p.acc2 : p.acc;
-      warp_add(mem_terms<float, true>(p, o, i, j, m & kSolid, own ? links : 0u, list), sums, 0);
+      warp_add(mem_terms<float, true>(p, *body, o, i, j, m & kSolid, own ? links : 0u, list), sums, 0);
       FixAcc<float> vol;
       if (own && (m & kSolid)) vol = vol_terms<float>(BodyRef<float>(*body), i, j, px, py);
       warp_add(vol, sums, 6);

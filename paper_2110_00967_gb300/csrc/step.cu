@@ -7,12 +7,11 @@
 //     conditions of Sec. 3.1/3.2), and the tiles of the force region around
 //     the body (penalized nodes and the MEM link terms of Eq. MMEL /
 //     Eq. fluidtorque).  Its SIM and region blocks add their force terms into
-//     exact fixed-point sums.  For a moving body the region tiles rasterise
-//     the mask of the body's current position themselves (each tile with a
-//     one-node halo), the blocks take a ticket and the last of them records
-//     the step's forces and applies the FP64 rigid-body update (Eqs. dep1,
-//     theta2); for a fixed body one extra block of the next step's launch
-//     records them.
+//     exact fixed-point sums, which one extra block of the next step's launch
+//     records.  For a moving body every block of that launch applies the FP64
+//     rigid-body update (Eqs. dep1, theta2) for itself, and the region tiles
+//     rasterise the mask of the body's current position (each tile with a
+//     one-node halo).
 //   * the bulk kernel: every other node -- pull streaming (Eq. eqBd) and the
 //     BGK/TRT collision (Eq. TRT) of fluid nodes whose sources all lie inside
 //     the lattice; no mask, no side conditions, no forces.  It comes in
@@ -148,7 +147,7 @@ struct FieldNode {
 // moving body (a disk; t given) the predicate of Eq. fcar on the current body, since
 // the force-region tiles rewrite chi during the step
 __device__ __forceinline__ uint8_t solid_at(const StepArgs &p, const NearTest *t, int i, int j) {
-  if (t) return disk_contains(*p.body_src, *t, i, j) ? kSolid : (uint8_t)0;
+  if (t) return disk_contains(*t, i, j) ? kSolid : (uint8_t)0;
   return p.chi[(int64_t)j * p.L.pitch + i];
 }
 
@@ -290,12 +289,14 @@ __device__ __forceinline__ FixAcc<T> sim_terms(const StepArgs &p, const NearTest
 // One SIM integration point: its sampled nodes (walked now, or for a fixed
 // body found when it was placed) and its force terms.
 template <typename S, bool kGather>
-__device__ __noinline__ FixAcc<typename Store<S>::T> sim_point(const StepArgs &p, const S *buf, double bxg, double byg,
-                                         int q, bool &missing) {
+__device__ __noinline__ FixAcc<typename Store<S>::T> sim_point(const StepArgs &p, const S *buf,
+                                                               const BodyState &body, int q,
+                                                               bool &missing) {
   using T = typename Store<S>::T;
   const SimPoint &sp = p.sim_pts[q];
   uint32_t cand[4] = {sp.cand[0], sp.cand[1], sp.cand[2], sp.cand[3]};
-  const NearTest near(*p.body_src);
+  const double bxg = body.xg, byg = body.yg;
+  const NearTest near(body);
   const NearTest *t = p.raster ? &near : nullptr;  // a moving body: its predicate, not chi
   const int n = sp.n_cand >= 0 ? sp.n_cand : sim_candidates(p, t, sp, bxg, byg, cand);
   missing = n <= 0;
@@ -327,10 +328,10 @@ struct Slice {
   int first, count;  // the block's nodes of the tile
 };
 
-__device__ __forceinline__ void tile_solid(const StepArgs &p, int ti, int tj, Slice sl,
-                                           TileMask &tm) {
+__device__ __forceinline__ void tile_solid(const StepArgs &p, const BodyState &body, int ti,
+                                           int tj, Slice sl, TileMask &tm) {
   const Lattice &L = p.L;
-  const NearTest near(*p.body_src);
+  const NearTest near(body);
   // the slice's rows and columns with their halo (a slice shorter than a row
   // lies within one)
   const int x0 = sl.first % kTileX, y0 = sl.first / kTileX;
@@ -343,7 +344,7 @@ __device__ __forceinline__ void tile_solid(const StepArgs &p, int ti, int tj, Sl
     if (L.bc[0] == VPLBM_PERIODIC) gi = gi < 0 ? gi + L.nx : (gi >= L.nx ? gi - L.nx : gi);
     if (L.bc[2] == VPLBM_PERIODIC) gj = gj < 0 ? gj + L.ny : (gj >= L.ny ? gj - L.ny : gj);
     const bool in = gi >= 0 && gi < L.nx && gj >= 0 && gj < L.ny;
-    tm.s[hy][hx] = (in && disk_contains(*p.body_src, near, gi, gj)) ? kSolid : (uint8_t)0;
+    tm.s[hy][hx] = (in && disk_contains(near, gi, gj)) ? kSolid : (uint8_t)0;
   }
 }
 
@@ -415,8 +416,9 @@ struct LinkList {
   uint16_t link[256];  // lane | direction << 5 | solid << 9
 };
 template <typename T, bool kList>
-__device__ __forceinline__ FixAcc<T> mem_terms(const StepArgs &p, const T (&o)[9], int i, int j,
-                                               bool solid, uint32_t links, LinkList<T> *list) {
+__device__ __forceinline__ FixAcc<T> mem_terms(const StepArgs &p, const BodyState &body,
+                                               const T (&o)[9], int i, int j, bool solid,
+                                               uint32_t links, LinkList<T> *list) {
   FixAcc<T> acc;
   __syncwarp();  // the lanes come from divergent updates; unmerged they would run all this in turn
   if (!__any_sync(kFull, links != 0)) return acc;
@@ -441,7 +443,7 @@ __device__ __forceinline__ FixAcc<T> mem_terms(const StepArgs &p, const T (&o)[9
   }
   const uint32_t mine = links | (solid ? 1u : 0u);  // bit 0: the node's phase
   const Lattice &L = p.L;
-  const BodyRef<T> b(*p.body_src);
+  const BodyRef<T> b(body);
 #pragma unroll 1
   for (int first = 0; first < total; first += 32) {
     const int t = first + lane;
@@ -512,23 +514,105 @@ __device__ __forceinline__ FixAcc<T> vol_terms(const BodyRef<T> b, int i, int j,
 // rigid body and the tail
 // ---------------------------------------------------------------------------
 
-// What the rigid-body update of a disk of density ratio rho_s/rho in a fluid of
-// density 1 needs of its constants: 1/m, 1/m, 1/I and the buoyant acceleration
-// (1 - 1/rho_r) g of the three coordinates.  Computed by three lanes of every
-// block that may turn out the last, while its other warps work: the tail's
-// chain of FP64 operations (some 60 cycles each) is then four operations long,
-// where it held the mass, the inertia and four divisions.
-struct RigidConst {
-  double inv[3], acc[3];
-};
-__device__ __forceinline__ void rigid_const(const BodyState &b, RigidConst &c, int k) {
-  const double r = 0.5 * b.length;
-  const double m = b.density_ratio * 3.14159265358979323846 * r * r;
-  c.inv[k] = 1.0 / (k == 2 ? 0.5 * m * r * r : m);
-  c.acc[k] = k == 2 ? 0.0 : (1.0 - 1.0 / b.density_ratio) * (k == 0 ? b.gx : b.gy);
+// A moving body at the step's time level, into b (shared memory), by one warp.
+// With the previous step's sums pending (finalize_prev) it is the previous
+// level's state updated with them (Eqs. dep1 and theta2, explicit trapezoid in
+// time), lanes 0, 1 and 2 taking x, y and the rotation; lanes 0 .. 8 return that
+// step's nine totals.  Every block of a launch computes it for itself: the
+// earlier scheme, in which the last block of the step (found by a ticket) did
+// this for all, added a fence, two rounds to L2 and a half-empty GPU to every
+// step's chain.
+template <typename T>
+__device__ __forceinline__ double moving_body(const StepArgs &p, BodyState &b, bool &ok) {
+  constexpr int kBodyWords = (int)(sizeof(BodyState) / sizeof(unsigned long long));
+  static_assert(sizeof(BodyState) % sizeof(unsigned long long) == 0 && kBodyWords <= 32,
+                "BodyState in 8-byte words, one per lane");
+  const int lane = threadIdx.x & 31, k = min(lane, 2);
+  const BodyState *from = p.finalize_prev ? p.body_prev : p.body_src;
+  // all loads are issued together
+  unsigned long long w = 0;
+  long long w0 = 0, w1 = 0;
+  if (lane < kBodyWords) w = __ldcg(reinterpret_cast<const unsigned long long *>(from) + lane);
+  if (p.finalize_prev && lane < kAccSlots) {
+    w0 = (long long)__ldcg(p.acc_prev + 2 * lane);
+    if (Fix<T>::kWords > 1) w1 = (long long)__ldcg(p.acc_prev + 2 * lane + 1);
+  }
+  const double inv = __ldg(p.rigid->inv + k), acc = __ldg(p.rigid->acc + k);
+  if (lane < kBodyWords) reinterpret_cast<unsigned long long *>(&b)[lane] = w;
+  __syncwarp();
+  ok = true;
+  if (!p.finalize_prev) return 0.0;
+  double tot = Fix<T>::value(w0, w1);
+  if (lane >= 3 && lane < 6) tot += p.sim_const[lane - 3];
+  const double force = __shfl_sync(kFull, tot, b.estimator == VPLBM_SIM ? 3 + k : k);
+  const double v0 = k == 0 ? b.ux : k == 1 ? b.uy : b.omega;
+  const double x0 = k == 0 ? b.xg : k == 1 ? b.yg : b.theta;
+  const double v1 = v0 + fma(force, inv, acc);
+  const double x1 = x0 + 0.5 * (v0 + v1);
+  // a body that left the lattice or moved a node in one step stays where it was
+  // (and one block flags the run as unstable)
+  const double r = 0.5 * b.length, far = (double)((k == 0 ? p.L.nx : p.L.ny) - 1);
+  const bool fine = k == 2 || (x1 - r >= 0.0 && x1 + r <= far && fabs(x1 - x0) < 1.0);
+  ok = __all_sync(kFull, fine);
+  __syncwarp();
+  if (ok) {
+    if (lane == 0) {
+      b.ux = v1;
+      b.xg = x1;
+      b.f_ux = (float)v1;
+      b.f_xg = (float)x1;
+    } else if (lane == 1) {
+      b.uy = v1;
+      b.yg = x1;
+      b.f_uy = (float)v1;
+      b.f_yg = (float)x1;
+    } else if (lane == 2) {
+      b.omega = v1;
+      b.theta = x1;
+      b.f_omega = (float)v1;
+    }
+  }
+  __syncwarp();
+  return tot;
 }
 
-// Force bookkeeping of a launch whose tail was deferred (a fixed body): the
+// The bookkeeping of a moving body's step by one warp: with sums pending, the
+// body at this level, the history row, running sums and step counter; and the
+// force region of this level's body, for the next launch.
+template <typename T>
+__device__ __forceinline__ void record_moving(const StepArgs &p, BodyState &b,
+                                              ForceRegion *region) {
+  const int lane = threadIdx.x & 31;
+  bool ok;
+  const double tot = moving_body<T>(p, b, ok);
+  if (lane == 0)
+    *region = make_region(p.L, b.xg, b.yg, 0.5 * b.length, p.ntiles_x, p.ntiles_y, kTileX);
+  if (!p.finalize_prev) return;
+  constexpr int kBodyWords = (int)(sizeof(BodyState) / sizeof(unsigned long long));
+  if (lane < kBodyWords)
+    reinterpret_cast<unsigned long long *>(p.body_src)[lane] =
+        reinterpret_cast<const unsigned long long *>(&b)[lane];
+  const bool do_sim = p.prev_sim != 0;
+  const long long step = __ldcg(p.dev_step);
+  __syncwarp();
+  if (lane < kHistCols) {
+    // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
+    const bool have = lane < 3 || lane >= 6 || do_sim;
+    p.hist[kHistCols * (step % p.hist_len) + lane] =
+        have ? tot : __longlong_as_double(0x7ff8000000000000LL);
+    if (have && lane < 6) p.sums[lane] += tot;
+  } else if (lane == 16) {
+    p.counts[0] += 1;
+  } else if (lane == 17 && do_sim) {
+    p.counts[1] += 1;
+  } else if (lane == 18) {
+    *p.dev_step = step + 1;
+  } else if (lane == 19 && !ok) {
+    atomicOr(p.status, kStatusUnstable);
+  }
+}
+
+// Force bookkeeping of the previous launch (a fixed body): the
 // fixed-point sums of its step, or of the two steps of a pair, become the
 // steps' history rows and are added to the running sums in step order; the
 // step counter advances and the sums are cleared for reuse two launches later.
@@ -575,108 +659,6 @@ __device__ void finalize(const StepArgs &p) {
     p.counts[tid - 6] += rows;
   } else if (tid == 8) {
     *p.dev_step += rows;  // read above by both rows before the barrier
-  }
-}
-
-// The last participating block: the step's forces from the fixed-point sums
-// (plus the polygon's constant SIM part), histories, running sums, body
-// (Eqs. dep1 and theta2, explicit trapezoid in time).  Its loads are spread over
-// threads and issued together, and the three coordinates of the body are updated
-// by three lanes side by side.
-template <typename T>
-__device__ void tail(const StepArgs &p, const ForceRegion &reg, const RigidConst &rc) {
-  constexpr int kBodyWords = (int)(sizeof(BodyState) / sizeof(unsigned long long));
-  static_assert(sizeof(BodyState) % sizeof(unsigned long long) == 0, "BodyState in 8-byte words");
-  const int tid = threadIdx.x;
-  __shared__ double tot[kAccSlots];
-  __shared__ BodyState old_b, new_b;
-  __shared__ long long step_s;
-  const bool do_sim = p.sim_blocks > 0;
-  if (tid < kAccSlots) {
-    // the sums were added by other SMs: read them through L2
-    const long long w0 = (long long)__ldcg(p.acc + 2 * tid);
-    const long long w1 = (long long)__ldcg(p.acc + 2 * tid + 1);
-    double v = Fix<T>::value(w0, w1);
-    if (tid >= 3 && tid < 6) v += p.sim_const[tid - 3];
-    tot[tid] = v;
-  } else if (tid < kAccSlots + kBodyWords) {
-    const int q = tid - kAccSlots;
-    const unsigned long long w =
-        __ldcg(reinterpret_cast<const unsigned long long *>(p.body_src) + q);
-    reinterpret_cast<unsigned long long *>(&old_b)[q] = w;
-    reinterpret_cast<unsigned long long *>(&new_b)[q] = w;
-  } else if (tid == 31) {
-    step_s = __ldcg(p.dev_step);
-  }
-  __syncthreads();
-  if (tid < 32) {
-    // the first warp: lanes 0, 1, 2 update x, y and the rotation
-    const int k = min(tid, 2);
-    const bool sim = old_b.estimator == VPLBM_SIM;
-    const double v0 = k == 0 ? old_b.ux : k == 1 ? old_b.uy : old_b.omega;
-    const double x0 = k == 0 ? old_b.xg : k == 1 ? old_b.yg : old_b.theta;
-    const double v1 = v0 + fma(tot[sim ? 3 + k : k], rc.inv[k], rc.acc[k]);
-    const double x1 = x0 + 0.5 * (v0 + v1);
-    const double x = __shfl_sync(kFull, x1, 0), y = __shfl_sync(kFull, x1, 1);
-    ForceRegion nreg = reg;
-    bool ok = true;
-    if (old_b.moving) {
-      nreg = make_region(p.L, x, y, 0.5 * old_b.length, p.ntiles_x, p.ntiles_y, kTileX);
-      // the body left the lattice or moved a node in one step: keep it where
-      // it was and flag the run as unstable
-      ok = !(nreg.error || nreg.count > p.region_slots || nreg.count > kRegionCapacity ||
-             fabs(x - old_b.xg) >= 1.0 || fabs(y - old_b.yg) >= 1.0);
-    }
-    if (old_b.moving && ok) {
-      if (tid == 0) {
-        new_b.ux = v1;
-        new_b.xg = x1;
-        new_b.f_ux = (float)v1;
-        new_b.f_xg = (float)x1;
-      } else if (tid == 1) {
-        new_b.uy = v1;
-        new_b.yg = x1;
-        new_b.f_uy = (float)v1;
-        new_b.f_yg = (float)x1;
-      } else if (tid == 2) {
-        new_b.omega = v1;
-        new_b.theta = x1;
-        new_b.f_omega = (float)v1;
-      }
-    }
-    if (tid == 0) {
-      if (!ok) {
-        atomicOr(p.status, kStatusUnstable);
-        nreg = reg;
-      }
-      *p.reg_dst = nreg;
-    }
-    __syncwarp();
-    if (tid < kBodyWords)
-      reinterpret_cast<unsigned long long *>(p.body_dst)[tid] =
-          reinterpret_cast<const unsigned long long *>(&new_b)[tid];
-  }
-  // the bookkeeping: a second warp where there is one
-  const int q = tid - (blockDim.x > 32 ? 32 : 0);
-  if (q >= 0 && q < 32) {
-    if (q < kHistCols) {
-      // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
-      const bool have = q < 3 || q >= 6 || do_sim;
-      p.hist[kHistCols * (step_s % p.hist_len) + q] =
-          have ? tot[q] : __longlong_as_double(0x7ff8000000000000LL);
-      if (have && q < 6) p.sums[q] += tot[q];
-    } else if (q == 16) {
-      p.counts[0] += 1;
-    } else if (q == 17 && do_sim) {
-      p.counts[1] += 1;
-    } else if (q == 18) {
-      *p.dev_step = step_s + 1;
-    } else if (q == 19) {
-      *p.ticket = 0u;
-    }
-    // every read of the sums above precedes the barrier; the next launch sees
-    // all of this block's stores
-    if (q < kAccWords) p.acc[q] = 0ull;
   }
 }
 
@@ -1156,26 +1138,34 @@ struct NodeForces {
   bool solid = false;
 };
 
-// One node of the special kernel: pull (with the side conditions where
-// needed), keep the outlet column, update and store.
+// The pre-collision populations of a node of the special kernel (with the side
+// conditions where needed).
 template <typename S, bool kGather>
-__device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bool in_reg,
-                                             const TileMask *tm, int tx, int ty,
-                                             NodeForces<typename Store<S>::T> &nf) {
+__device__ __forceinline__ void special_load(const StepArgs &p, int i, int j,
+                                             typename Store<S>::T (&h)[9]) {
   using T = typename Store<S>::T;
   const Lattice &L = p.L;
   const S *__restrict__ src = static_cast<const S *>(p.src);
-  S *dst = static_cast<S *>(p.dst);
-  const T *prev = static_cast<const T *>(p.prev_src);
-  const int64_t node = (int64_t)j * L.pitch + i;
-  T h[9];
   if (kGather && i > 0 && i < L.nx - 1 && j > 0 && j < L.ny - 1) {
+    const int64_t node = (int64_t)j * L.pitch + i;
 #pragma unroll
     for (int a = 0; a < 9; ++a)
       h[a] = Store<S>::ld(src + (int64_t)a * L.plane + node - cy_of(a) * L.pitch - cx_of(a));
   } else {
-    edge_pops<S, kGather>(src, prev, L, i, j, h);
+    edge_pops<S, kGather>(src, static_cast<const T *>(p.prev_src), L, i, j, h);
   }
+}
+
+// One node of the special kernel: keep the outlet column, update and store.
+template <typename S>
+__device__ __forceinline__ bool special_node(const StepArgs &p, const BodyState *body,
+                                             const typename Store<S>::T (&h)[9], int i, int j,
+                                             bool in_reg, const TileMask *tm, int tx, int ty,
+                                             NodeForces<typename Store<S>::T> &nf) {
+  using T = typename Store<S>::T;
+  const Lattice &L = p.L;
+  S *dst = static_cast<S *>(p.dst);
+  const int64_t node = (int64_t)j * L.pitch + i;
   if (i == L.nx - 1 && L.bc[1] == VPLBM_OUTLET_CONVECTIVE) {
     // the outlet column's pre-collision values, for the next step
     T *pd = static_cast<T *>(p.prev_dst);
@@ -1200,8 +1190,8 @@ __device__ __forceinline__ bool special_node(const StepArgs &p, int i, int j, bo
   T(&o)[9] = nf.o;
   const Consts<T> cst(p);
   const bool bad =
-      L.has_bf ? update_node<S, true>(h, m, i, j, L, p.body_src, cst, o, nf.pen_x, nf.pen_y)
-               : update_node<S, false>(h, m, i, j, L, p.body_src, cst, o, nf.pen_x, nf.pen_y);
+      L.has_bf ? update_node<S, true>(h, m, i, j, L, body, cst, o, nf.pen_x, nf.pen_y)
+               : update_node<S, false>(h, m, i, j, L, body, cst, o, nf.pen_x, nf.pen_y);
   if (sizeof(S) == 2 && p.sr) {
     const SrBits r(sr_level(p), (uint32_t)node >> 1);
 #pragma unroll
@@ -1234,34 +1224,43 @@ __global__ void __launch_bounds__(kThreads / kSlices<S>, kMinBlocks)
     special_kernel(const StepArgs p) {
   using T = typename Store<S>::T;
   constexpr int kBlock = kThreads / kSlices<S>;
-  __shared__ int is_last;
   __shared__ TileMask tmask;
-  __shared__ RigidConst rigid;
+  __shared__ BodyState moving;
   __shared__ LinkList<T> lists[kList ? kBlock / 32 : 1];
   const Lattice &L = p.L;
   const int b = blockIdx.x / kSlices<S>;
   const Slice slice{(int)(blockIdx.x % kSlices<S>) * kBlock, kBlock};
   const int tid = slice.first + threadIdx.x;  // within the tile's nodes
   const ForceRegion reg = *p.reg_src;
+  const bool moves = kList && p.raster;  // a moving body (special_t)
   if (p.sr && b == 0 && tid == 0) *p.rng_dst = *p.rng_src + 1ull;  // the next level's counter
-  if (p.finalize_prev && b == (int)(gridDim.x / kSlices<S>) - 1) {
+  if ((p.finalize_prev || moves) && b == (int)(gridDim.x / kSlices<S>) - 1) {
     // the previous step's force sums, beside this step's work
-    if (slice.first == 0) finalize<T>(p);
+    if (slice.first != 0) return;
+    if (!moves) {
+      finalize<T>(p);
+    } else if (threadIdx.x < 32) {
+      if (threadIdx.x < kAccWords) p.acc_next[threadIdx.x] = 0ull;
+      record_moving<T>(p, moving, p.reg_dst);
+    }
     return;
   }
-  if (!p.defer && threadIdx.x >= kBlock - 3 && p.body_src->moving)
-    rigid_const(*p.body_src, rigid, threadIdx.x - (kBlock - 3));
+  // a moving body's state at this level, by the block's first warp
+  bool ok;
+  const BodyState *body = moves ? &moving : p.body_src;
 
   if (b < p.sim_blocks) {
     // ---- SIM points of this level ----
+    if (moves) {
+      if (threadIdx.x < 32) moving_body<T>(p, moving, ok);
+      __syncthreads();
+    }
     const int q = b * p.sim_per_block + tid;
     FixAcc<T> acc;
     bool missing = false;
-    if (tid < p.sim_per_block && q < p.n_sim) {
-      const BodyState *body = p.body_src;
-      acc = sim_point<S, kGather>(p, static_cast<const S *>(p.src), body->xg, body->yg, q,
-                                  missing);
-    }
+    if (tid < p.sim_per_block && q < p.n_sim)
+      acc = sim_point<S, kGather>(p, static_cast<const S *>(p.src), *body, q, missing);
+    __syncwarp();
     if (__any_sync(kFull, missing) && (tid & 31) == 0) atomicOr(p.status, kStatusSimMissing);
     warp_add(acc, p.acc, 3);
   } else if (!p.all_tiles && b < p.sim_blocks + p.edge_blocks) {
@@ -1275,11 +1274,12 @@ __global__ void __launch_bounds__(kThreads / kSlices<S>, kMinBlocks)
       const bool in_reg = ti >= reg.ti0 && ti <= reg.ti1 && tj >= reg.tj0 && tj <= reg.tj1;
       if (!in_reg) {
         NodeForces<T> unused;
-        bad = special_node<S, kGather>(p, i, j, false, nullptr, 0, 0, unused);
+        T h[9];
+        special_load<S, kGather>(p, i, j, h);
+        bad = special_node<S>(p, p.body_src, h, i, j, false, nullptr, 0, 0, unused);
       }
     }
     if (__any_sync(kFull, bad) && (tid & 31) == 0) atomicOr(p.status, kStatusUnstable);
-    return;
   } else {
     // ---- a whole tile: every tile (first step) or a force-region tile ----
     int ti, tj;
@@ -1297,41 +1297,32 @@ __global__ void __launch_bounds__(kThreads / kSlices<S>, kMinBlocks)
     const bool in_reg = ti >= reg.ti0 && ti <= reg.ti1 && tj >= reg.tj0 && tj <= reg.tj1;
     const int tx = tid % kTileX, ty = tid / kTileX;
     const int i = ti * kTileX + tx, j = tj * kTileY + ty;
-    // a moving body: the region tiles rasterise its mask at this level
-    const bool raster = p.raster && in_reg;  // uniform over the block
+    const bool inside = i < L.nx && j < L.ny;
+    T h[9];
+    if (inside) special_load<S, kGather>(p, i, j, h);
+    // a moving body: its state, and the region tiles rasterise its mask at this
+    // level, while the populations arrive
+    const bool raster = moves && in_reg;  // uniform over the block
     if (raster) {
-      tile_solid(p, ti, tj, slice, tmask);
+      if (threadIdx.x < 32) moving_body<T>(p, moving, ok);
+      __syncthreads();
+      tile_solid(p, moving, ti, tj, slice, tmask);
       __syncthreads();
     }
     bool bad = false;
     NodeForces<T> nf;
-    if (i < L.nx && j < L.ny)
-      bad = special_node<S, kGather>(p, i, j, in_reg, raster ? &tmask : nullptr, tx, ty, nf);
+    if (inside)
+      bad = special_node<S>(p, body, h, i, j, in_reg, raster ? &tmask : nullptr, tx, ty, nf);
     __syncwarp();
     if (__any_sync(kFull, bad) && (tid & 31) == 0) atomicOr(p.status, kStatusUnstable);
     if (!in_reg) return;  // uniform over the block
     LinkList<T> *list = nullptr;
     if constexpr (kList) list = lists + (threadIdx.x >> 5);
-    warp_add(mem_terms<T, kList>(p, nf.o, i, j, nf.solid, nf.links, list), p.acc, 0);
+    warp_add(mem_terms<T, kList>(p, *body, nf.o, i, j, nf.solid, nf.links, list), p.acc, 0);
     FixAcc<T> vol;
-    if (nf.solid) vol = vol_terms<T>(BodyRef<T>(*p.body_src), i, j, nf.pen_x, nf.pen_y);
+    if (nf.solid) vol = vol_terms<T>(BodyRef<T>(*body), i, j, nf.pen_x, nf.pen_y);
     warp_add(vol, p.acc, 6);
   }
-
-  if (p.defer) return;  // a later launch finalizes this step's sums
-
-  // ---- ticket among the SIM blocks and the force-region tiles ----
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned int expected = (unsigned int)(kSlices<S> * (p.sim_blocks + reg.count));
-    const unsigned int prev = atomicAdd(p.ticket, 1u);
-    is_last = (prev == expected - 1);
-  }
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  tail<T>(p, reg, rigid);
 }
 
 // ---------------------------------------------------------------------------
@@ -1662,7 +1653,7 @@ __global__ void __launch_bounds__(32 * kTileY, 12) bulk16x4_kernel(const StepArg
 template <typename S, bool kGather>
 cudaError_t special_t(const StepArgs &a, cudaStream_t s) {
   const int tiles = a.all_tiles ? a.ntiles_x * a.ntiles_y : a.edge_blocks + a.region_slots;
-  const int blocks = (a.sim_blocks + tiles + (a.finalize_prev ? 1 : 0)) * kSlices<S>;
+  const int blocks = (a.sim_blocks + tiles + (a.finalize_prev || a.raster ? 1 : 0)) * kSlices<S>;
   constexpr int kBlock = kThreads / kSlices<S>;
   if (a.raster || sizeof(S) == 8)
     special_kernel<S, kGather, 1, true><<<blocks, kBlock, 0, s>>>(a);
@@ -1675,7 +1666,20 @@ cudaError_t special_t(const StepArgs &a, cudaStream_t s) {
 
 template <typename T>
 __global__ void __launch_bounds__(64) finalize_kernel(const StepArgs p) {
-  finalize<T>(p);
+  __shared__ BodyState moving;
+  if (!p.raster) {
+    finalize<T>(p);
+    return;
+  }
+  // a moving body: into the state and region that the next launch starts from;
+  // all its sums are cleared, so that it starts at any of them
+  if (threadIdx.x >= 32) return;
+  record_moving<T>(p, moving, const_cast<ForceRegion *>(p.reg_src));
+  if (threadIdx.x < kAccWords) {
+    p.acc_prev[threadIdx.x] = 0ull;
+    p.acc[threadIdx.x] = 0ull;
+    p.acc_next[threadIdx.x] = 0ull;
+  }
 }
 
 // chi of a moving body on the force-region tiles, tile by tile as the special
@@ -1687,7 +1691,7 @@ __global__ void __launch_bounds__(kThreads) mask_kernel(const StepArgs p) {
   if (k >= reg.count) return;
   const int rw = reg.ti1 - reg.ti0 + 1;
   const int ti = reg.ti0 + k % rw, tj = reg.tj0 + k / rw;
-  tile_solid(p, ti, tj, Slice{0, kThreads}, tm);
+  tile_solid(p, *p.body_src, ti, tj, Slice{0, kThreads}, tm);
   __syncthreads();
   const int tx = threadIdx.x % kTileX, ty = threadIdx.x / kTileX;
   const int i = ti * kTileX + tx, j = tj * kTileY + ty;

@@ -429,9 +429,10 @@ __device__ __forceinline__ bool body_contains(const BodyState &b, int i, int j) 
 // lanes per SM: evaluated everywhere in FP64, the mask of a moving disk took
 // 1.8 us of its 12 us step.
 struct NearTest {
+  const BodyState &body;
   int i0, j0;
   float fx, fy, r2;
-  __device__ __forceinline__ explicit NearTest(const BodyState &b) {
+  __device__ __forceinline__ explicit NearTest(const BodyState &b) : body(b) {
     const double x0 = floor(b.xg), y0 = floor(b.yg);
     i0 = (int)x0;
     j0 = (int)y0;
@@ -441,11 +442,11 @@ struct NearTest {
     r2 = r * r;
   }
 };
-__device__ __forceinline__ bool disk_contains(const BodyState &b, const NearTest &t, int i, int j) {
+__device__ __forceinline__ bool disk_contains(const NearTest &t, int i, int j) {
   const float dx = (float)(i - t.i0) - t.fx, dy = (float)(j - t.j0) - t.fy;
   const float d2 = dx * dx + dy * dy, diff = d2 - t.r2;
   if (fabsf(diff) > 1e-5f * (d2 + t.r2) + 1e-5f) return diff < 0.0f;
-  return body_contains(b, i, j);
+  return body_contains(t.body, i, j);
 }
 
 // neighbour of (i, j) along a inside the lattice (periodic sides wrap);
@@ -490,6 +491,19 @@ struct CollideC {
 // ---------------------------------------------------------------------------
 // parameters of the fused step kernel
 // ---------------------------------------------------------------------------
+// What the rigid-body update of a disk of density ratio rho_s/rho in a fluid of
+// density 1 needs of its constants: 1/m, 1/m, 1/I and the buoyant acceleration
+// (1 - 1/rho_r) g of the three coordinates (computed when the body is placed).
+struct RigidConst {
+  double inv[3], acc[3];
+};
+inline RigidConst rigid_const(const BodyState &b) {
+  const double r = 0.5 * b.length;
+  const double m = b.density_ratio * 3.14159265358979323846 * r * r;
+  const double buoy = 1.0 - 1.0 / b.density_ratio;
+  return RigidConst{{1.0 / m, 1.0 / m, 1.0 / (0.5 * m * r * r)}, {buoy * b.gx, buoy * b.gy, 0.0}};
+}
+
 struct StepArgs {
   Lattice L;
   const void *src;      // populations: post-collision of level n-1 (gather)
@@ -498,13 +512,18 @@ struct StepArgs {
   const void *prev_src;  // outlet column (compute type), pre-collision, level n-1
   void *prev_dst;        // outlet column, pre-collision, level n
   uint8_t *chi;
-  const BodyState *body_src;   // body at level n
-  BodyState *body_dst;         // body at level n + 1 (written by the tail)
-  const ForceRegion *reg_src;
-  ForceRegion *reg_dst;
+  // A fixed body: body_src, never written.  A moving one: the state at level n
+  // in body_src when nothing is pending; else body_prev holds level n - 1 and
+  // every block updates it with the previous step's sums for itself
+  // (moving_body), one block storing level n into body_src.
+  BodyState *body_src;
+  const BodyState *body_prev;
+  const RigidConst *rigid;     // a moving body's constants
+  const ForceRegion *reg_src;  // covers the body at level n (a moving one: by its margin,
+  ForceRegion *reg_dst;        // from level n - 1); ... at level n + 1, for the next launch
   unsigned long long *acc;       // [6][2] fixed-point sums of this step
   unsigned long long *acc_prev;  // the previous step's sums (finalized by this launch)
-  int32_t defer;                 // 1: no ticket and tail; a later launch finalizes the sums
+  unsigned long long *acc_next;  // a moving body's next sums, cleared by this launch
   int32_t finalize_prev;         // 1: an extra last block finalizes acc_prev first
   int32_t prev_sim;              // 1: the step being finalized evaluated SIM
   const SimPoint *sim_pts;
@@ -518,7 +537,6 @@ struct StepArgs {
   double *sums;          // [6]
   long long *counts;     // [2]
   long long *dev_step;   // steps completed
-  unsigned int *ticket;
   int32_t *status;
   // collision constants, FP64 and FP32 copies (FP32 paths must not convert
   // from FP64 per node: GB300 runs FP64 at a small fraction of FP32)
