@@ -40,17 +40,20 @@ NX, NY = 2048, 1024
 # populations read once and written once per node: 9 x 4 B + 9 x 4 B for FP32 storage,
 # 9 x 2 B + 9 x 2 B for the 16-bit offset forms
 BYTES_PER_LUP = {"f32": 72, "f16": 36, "bf16": 36, "f16sr": 36, "bf16sr": 36}
-STORAGE_NAME = {"f32": "float", "f16": "__half", "bf16": "__nv_bfloat16", "f16sr": "__half",
-                "bf16sr": "__nv_bfloat16"}
 # the arithmetic of the step: FP32, with the 16-bit forms storing FP16 / BF16
 # offsets and colliding in FP32 (force sums FP64 in every form)
 DTYPE_NAME = {"f32": "f32", "f16": "f16-storage/f32-compute", "bf16": "bf16-storage/f32-compute",
               "f16sr": "f16-storage-stochastic/f32-compute",
               "bf16sr": "bf16-storage-stochastic/f32-compute"}
-# the bulk kernel of each storage form (the special kernel runs beside it)
-BULK_NAME = {"f32": "bulk32x2_kernel", "f16": "bulk16_kernel<__half>",
-             "bf16": "bulk16_kernel<__nv_bfloat16>", "f16sr": "bulk16_kernel<__half, sr>",
-             "bf16sr": "bulk16_kernel<__nv_bfloat16, sr>"}
+# time steps per pass over the populations on the workloads below with a fixed
+# body: FP32 lattices take two steps in one launch, 16-bit ones of this size one
+STEPS_PER_PASS = {"f32": 2, "f16": 1, "bf16": 1, "f16sr": 1, "bf16sr": 1}
+# the kernels of one lattice step
+STEP_NAME = {"f32": "half of a pair_kernel<float> launch (two steps in one pass)",
+             "f16": "bulk16_kernel<__half>, special_kernel<__half> beside it",
+             "bf16": "bulk16_kernel<__nv_bfloat16>, special_kernel<__nv_bfloat16> beside it",
+             "f16sr": "bulk16_kernel<__half, sr>, special_kernel<__half> beside it",
+             "bf16sr": "bulk16_kernel<__nv_bfloat16, sr>, special_kernel<__nv_bfloat16> beside it"}
 PROFILE = os.path.join(ROOT, "profiles", "step_kernel_naca2048_f32.md")
 KERNEL_SOURCES = ("paper_2110_00967_gb300/csrc/step.cu",
                   "paper_2110_00967_gb300/csrc/pair.cuh",
@@ -71,7 +74,7 @@ def config_block(dtype: str = "f32", extra=None):
          "storage": "f32" if dtype == "f32" else f"{dtype} offsets from feq(1, u_in)",
          "forces_per_step": ["mem", "sim-849"],
          "l2": f"inputs larger than L2: 5 lattices x {mb} MB ping-pong, stepped side by side"
-               + (" (ncu range replay: DRAM traffic 151.9 MB per lattice step, 151.0 algorithmic)"
+               + (" (ncu range replay: DRAM traffic 78.4 MB per lattice step, 75.5 algorithmic at two steps per pass)"
                   if dtype == "f32" else "")}
     if extra:
         c.update(extra)
@@ -321,7 +324,7 @@ def run_ours(args, rank, world, local_rank):
     value = world * nodes * args.steps / (elapsed_ms / 1e3) / 1e6
     e2e_value = world * nodes * e2e_steps / e2e_dt / 1e6
     peak, peak_kind = measured_hbm_peak()
-    bpl = BYTES_PER_LUP[args.dtype]
+    bpl = BYTES_PER_LUP[args.dtype] // STEPS_PER_PASS[args.dtype]
     achieved = bpl * NX * NY / (lattice_step_ms / 1e3) / 1e9
     traffic = profiled_traffic(args.dtype)
     if rank != 0:
@@ -336,9 +339,7 @@ def run_ours(args, rank, world, local_rank):
                                             "bulk_variant": variants}),
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
                      "unit": "GB/s", "frac": round(achieved / peak, 4), "traffic": traffic,
-                     "kernel": f"one lattice step: {BULK_NAME[args.dtype]} with "
-                               f"special_kernel<{STORAGE_NAME[args.dtype]}> beside it, timed over "
-                               "the region",
+                     "kernel": f"one lattice step: {STEP_NAME[args.dtype]}, timed over the region",
                      "kernel_avg_us": round(lattice_step_ms * 1e3, 3),
                      "bytes_per_lup": bpl, "peak_kind": peak_kind},
         "e2e": {"value": round(e2e_value, 1), "unit": "MLUPS",
@@ -564,7 +565,7 @@ def run_naca_large(args, rank, world, local_rank):
     lat.check()
     elapsed_ms = reduce_max(start.elapsed_time(end), world, dev)
     nodes = w.nx * w.ny
-    bpl = BYTES_PER_LUP[args.dtype]
+    bpl = BYTES_PER_LUP[args.dtype] // STEPS_PER_PASS[args.dtype]
     step_ms = elapsed_ms / args.steps
     achieved = bpl * nodes / (step_ms / 1e3) / 1e9
     peak, peak_kind = measured_hbm_peak()
@@ -578,11 +579,11 @@ def run_naca_large(args, rank, world, local_rank):
         "config": {"workload": f"naca0012-8192x4096-{args.dtype}-alpha10", "grid": [w.nx, w.ny],
                    "instances": 1, "chord": 800, "reynolds": 1000, "tau_plus": 0.62,
                    "storage": args.dtype, "bulk_variant": [variant],
-                   "l2": f"inputs larger than L2: {2 * bpl * nodes / 2 / 1e9:.1f} GB ping-pong",
+                   "l2": f"inputs larger than L2: {BYTES_PER_LUP[args.dtype] * nodes / 1e9:.1f} GB ping-pong",
                    "parallelism": f"replicas{world}"},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": None,
-                     "kernel": "one lattice step (bulk + special), timed over the region",
+                     "kernel": "one lattice step, timed over the region",
                      "kernel_avg_us": round(step_ms * 1e3, 3), "bytes_per_lup": bpl,
                      "peak_kind": peak_kind},
         "gpu_launches": lat.launches - l0,
@@ -725,7 +726,7 @@ def run_naca_paper(args, rank, world, local_rank, sim_variants=False):
             c["rel_to_n3393_order0"] = [(c["cd_sim"] - ref["cd_sim"]) / abs(ref["cd_sim"]),
                                         (c["cl_sim"] - ref["cl_sim"]) / abs(ref["cl_sim"])]
     nodes = works[0].nx * works[0].ny * len(lats)
-    bpl = BYTES_PER_LUP[args.dtype]
+    bpl = BYTES_PER_LUP[args.dtype] // STEPS_PER_PASS[args.dtype]
     lattice_step_ms = elapsed_ms / (args.steps * len(lats))
     achieved = bpl * nodes / len(lats) / (lattice_step_ms / 1e3) / 1e9
     peak, peak_kind = measured_hbm_peak()

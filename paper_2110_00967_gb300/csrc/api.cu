@@ -428,12 +428,6 @@ bool sim_due(const vplbm_ctx *c, long long step) {
   return c->sim_every > 0 && c->n_sim > 0 && step % c->sim_every == 0;
 }
 
-// One time step on stream s.  The first step after a pre-collision state
-// updates every tile with the special kernel.  Later steps split the nodes:
-// the special kernel (edge nodes, force region, SIM, tail: a few latency-bound
-// blocks) runs on the context's high-priority side stream beside the bulk
-// kernel (all other nodes, bandwidth-bound) on s; the two write disjoint
-// nodes, and s waits for both before the next step.
 // Finalizes the force sums of the last queued step or pair, if pending: one
 // block on s (history rows, running sums, step counter, a moving body's state).
 cudaError_t flush_forces(vplbm_ctx *c, cudaStream_t s) {
@@ -457,6 +451,12 @@ cudaError_t refresh_mask(vplbm_ctx *c, cudaStream_t s) {
   return launch_mask(step_args(c, c->cur, false), s);
 }
 
+// One time step on stream s.  The first step after a pre-collision state
+// updates every tile with the special kernel.  Later steps split the nodes: the
+// special kernel (edge nodes, force region, SIM: a few latency-bound blocks)
+// runs on the context's high-priority side stream beside the bulk kernel (all
+// other nodes, bandwidth-bound) on s; the two write disjoint nodes, and s waits
+// for both before the next step.
 cudaError_t queue_step(vplbm_ctx *c, cudaStream_t s, int src, bool pre, bool do_sim) {
   if (c->body_host.moving) c->mask_stale = true;
   cudaError_t e = cudaSuccess;
@@ -864,7 +864,7 @@ vplbm_status vplbm_create(const vplbm_config *cfg, void *dev_workspace, size_t b
 
   cudaError_t e = cudaMemsetAsync(c->ws, 0, lay.total, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  // the side stream runs the special kernel (forces, edges, tail) at the
+  // the side stream runs the special kernel (forces, edges) at the
   // highest priority so that its few blocks are dispatched ahead of the bulk
   int prio_lo = 0, prio_hi = 0;
   if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);

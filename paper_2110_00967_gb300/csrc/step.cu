@@ -15,8 +15,10 @@
 //   * the bulk kernel: every other node -- pull streaming (Eq. eqBd) and the
 //     BGK/TRT collision (Eq. TRT) of fluid nodes whose sources all lie inside
 //     the lattice; no mask, no side conditions, no forces.  It comes in
-//     several launch forms with identical results (bulk_kernel for FP32/FP64,
-//     bulk16_kernel and bulk16x4_kernel for 16-bit storage).
+//     several launch forms with identical results (bulk32x2_kernel for FP32,
+//     bulk_kernel for FP64, bulk16_kernel and bulk16x4_kernel for 16-bit storage).
+// Where the body stands still and the compute type is FP32, two time steps can
+// be one launch over the same nodes (pair.cuh).
 // For the first step after a pre-collision state the special kernel updates
 // every tile.
 #include "vplbm_internal.cuh"
@@ -511,7 +513,7 @@ __device__ __forceinline__ FixAcc<T> vol_terms(const BodyRef<T> b, int i, int j,
 }
 
 // ---------------------------------------------------------------------------
-// rigid body and the tail
+// rigid body and the force sums' bookkeeping
 // ---------------------------------------------------------------------------
 
 // A moving body at the step's time level, into b (shared memory), by one warp.

@@ -427,7 +427,7 @@ __device__ __forceinline__ bool body_contains(const BodyState &b, int i, int j) 
 // centre, has a relative error below 1e-6, and only nodes closer to the circle
 // than 1e-5 of r^2 need the FP64 form (none in most warps).  GB300 has two FP64
 // lanes per SM: evaluated everywhere in FP64, the mask of a moving disk took
-// 1.8 us of its 12 us step.
+// 1.8 us of a step (12 us then, 9.2 now).
 struct NearTest {
   const BodyState &body;
   int i0, j0;
@@ -703,7 +703,7 @@ void set_global_error(const std::string &msg);
 
 // launches (step.cu)
 // the special kernel: SIM blocks, edge nodes, force-region tiles and the
-// FP64 tail (or every tile, with all_tiles set)
+// block that finalizes the previous step (or every tile, with all_tiles set)
 cudaError_t launch_special(int dtype, bool gather, const StepArgs &a, cudaStream_t s);
 // one block that finalizes a deferred step's force sums (acc_prev): history
 // row, running sums, step counter
