@@ -487,17 +487,20 @@ cudaError_t queue_step(vplbm_ctx *c, cudaStream_t s, int src, bool pre, bool do_
   return e;
 }
 
-constexpr int64_t kPairSmall = 700000;
+constexpr int64_t kPairTiny = 400000, kPairSmall = 700000;
 // Rows per warp of the bulk blocks.  Long runs recompute fewer rim rows
 // ((rows + 2) / rows of the first step's work); short ones are more and shorter
-// blocks, which a lattice alone needs to fill 152 SMs and to keep its last wave
-// of blocks short.  us per step, FP32 (8 / 16 / 24 rows): 3614 x 1946 alone
-// 45.1 / 46.8 / 48.4, 2048 x 1024 alone 15.2 / 15.4 / 19.2, five of them 13.4 /
-// 13.05 / 12.8; 512 x 256 (6 / 12 / 16 rows) 3.9 / 4.4 / 5.0.
+// warps, which a lattice alone needs to fill 152 SMs and to keep its last wave
+// of blocks short.  us per step: 512 x 256 FP32 (5 / 6 / 8 rows) 3.89 / 3.92 / 3.98,
+// 768 x 384 FP16 4.80 / 4.89 / 5.30; 1024 x 512 FP32 (5 / 6 / 8) 5.3 / 4.9 / 5.8 and
+// FP16 6.0 / 5.7 / 6.7; 2048 x 1024 FP32 (6 / 8 / 10) 15.6 / 15.2 / 15.6, 3614 x 1946
+// (6 / 8 / 16) 45.4 / 44.9 / 46.3; five 2048 x 1024 (16 / 20 / 24) 12.91 / 12.76 / 12.78.
 int pair_rows(const vplbm_ctx *c) {
   if (c->bulk_variant > 0) return c->bulk_variant == 1 ? 12 : 24;
   if (!is_alone(c->mode)) return 20;
-  return (int64_t)c->L.nx * c->L.ny < kPairSmall || elem_bytes(c->cfg.dtype) == 2 ? 6 : 8;
+  const int64_t nodes = (int64_t)c->L.nx * c->L.ny;
+  if (nodes < kPairTiny) return 5;
+  return nodes < kPairSmall || elem_bytes(c->cfg.dtype) == 2 ? 6 : 8;
 }
 
 // Two time steps in one launch on stream s (pair.cuh).
@@ -589,14 +592,14 @@ PairPlan pair_plan(const vplbm_ctx *c, const vplbm_body &b, const std::vector<Si
 
 // Chooses how the lattices of a call step, from the nodes that the call steps
 // side by side.  FP32 steps in pairs wherever it can: it is bound by HBM, and a
-// pair halves the traffic (five 2048 x 1024 lattices 22.9 -> 13.0 us per step
+// pair halves the traffic (five 2048 x 1024 lattices 22.9 -> 12.8 us per step
 // each, one 512 x 256 lattice 7.3 -> 3.9).  16-bit storage already reads half
 // as much and is bound by its arithmetic once the GPU is full, where the rim
 // that a pair recomputes costs what the traffic saves (the serving mix of
 // five sizes, FP16 stochastic: 6.5 us per lattice step singly, 6.6 in pairs with
 // long runs, 7.6 with short ones); alone and up to about 1.5 M nodes the GPU is
-// not full, and half as many launches win (512 x 256: 9.7 -> 4.4 us, 1024 x 512:
-// 10.2 -> 7.0, 1536 x 768: 12.2 -> 10.7, 2048 x 1024: 16.5 -> 16.6).
+// not full, and half as many launches win (512 x 256: 9.7 -> 4.2 us, 1024 x 512:
+// 10.2 -> 5.7, 1536 x 768: 12.2 -> 9.8, 2048 x 1024: 16.5 -> 16.6).
 constexpr int64_t kPair16Nodes = 1500000;
 constexpr int64_t kPairBatchNodes = 4000000;  // a full GPU: longer runs
 void choose_mode(vplbm_ctx *c, int64_t call_nodes) {

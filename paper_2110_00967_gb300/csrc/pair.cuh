@@ -31,7 +31,7 @@
 // it is bound by the FMA pipe (62 % busy) and one row prefetched in registers is
 // enough.  Measured, us per step and lattice, five 2048 x 1024 lattices in FP32:
 // 22.9 in single steps (0.97 of the copy rate), 14.0 with the next row held in
-// registers, 12.9 with the ring, 11.3 being the traffic of a pair at the copy
+// registers, 12.8 with the ring, 11.3 being the traffic of a pair at the copy
 // rate; rings of three and four rows 13.15 and 13.8 (shared memory taken from
 // L1), five blocks per SM instead of four (96 registers, spilled in the special
 // blocks) 13.15 against 13.06.
@@ -111,7 +111,11 @@ __device__ __forceinline__ void cell_update(const StepArgs &p, const Consts<floa
   }
 }
 
-constexpr int kPairWarps = 4;    // warps (adjacent strips) per block
+// Warps per block, numbered over the whole grid (strips of a run of rows, then of
+// the next): with a block's four strips side by side the last block of a run held
+// up to three idle warps (1024 x 512, 17 strips: 5.8 us per step, 4.9 without;
+// 3614 x 1946, 61 strips: 45.5 and 44.9; 8192 x 4096, 137 strips: 204.2 and 202.3).
+constexpr int kPairWarps = 4;
 constexpr int kPairStore = 60;   // nodes a warp stores per row
 constexpr int kPairStages = 3;   // rows of the ring
 constexpr int kPairAhead = kPairStages - 1;
@@ -129,15 +133,14 @@ __device__ __forceinline__ void copy_async(Raw *smem, const void *global) {
 
 template <typename S, bool kForce, bool kSR>
 __device__ __forceinline__ void pair_bulk(
-    const StepArgs &p, int bx, int by,
+    const StepArgs &p, int strip, int run,
     typename Cell<S>::Raw (*ring)[9][32 * kPairWarps]) {
   using Raw = typename Cell<S>::Raw;
   const Lattice &L = p.L;
   const int lane = threadIdx.x & 31;
-  const int strip = bx * kPairWarps + (threadIdx.x >> 5);
   const int i = 2 + strip * kPairStore + 2 * (lane - 1);  // the lane's nodes i, i + 1
-  if (2 + strip * kPairStore > L.nx - 3) return;  // the warp lies beyond the last column
-  const int r0 = 2 + by * p.pair_rows;
+  const int r0 = 2 + run * p.pair_rows;
+  if (r0 >= L.ny - 2) return;  // the warp lies beyond the last run of rows
   const int r1 = min(r0 + p.pair_rows, L.ny - 2);
   // the nodes that the lane stores (bits), outside / inside the rows of the
   // box (its columns start and end on pairs)
@@ -526,16 +529,16 @@ __global__ void __launch_bounds__(kPairThreads, kPairMinBlocks) pair_kernel(cons
     pair_special<S, kForce, kSR>(p, g, b, post, post + 9, lists + (threadIdx.x >> 5));
     return;
   }
-  pair_bulk<S, kForce, kSR>(p, (b - g.special) % p.pair_bx, (b - g.special) / p.pair_bx,
+  const int warp = (b - g.special) * kPairWarps + (int)(threadIdx.x >> 5);
+  pair_bulk<S, kForce, kSR>(p, warp % p.pair_strips, warp / p.pair_strips,
                             reinterpret_cast<Raw(*)[9][kPairThreads]>(smem));
 }
 
 template <typename S, bool kForce>
 cudaError_t pair_f(StepArgs a, cudaStream_t s) {
-  const int strips = (a.L.nx - 4 + kPairStore - 1) / kPairStore;
-  a.pair_bx = (strips + kPairWarps - 1) / kPairWarps;
-  const int blocks =
-      pair_grid(a).special + a.pair_bx * ((a.L.ny - 4 + a.pair_rows - 1) / a.pair_rows);
+  a.pair_strips = (a.L.nx - 4 + kPairStore - 1) / kPairStore;
+  const int warps = a.pair_strips * ((a.L.ny - 4 + a.pair_rows - 1) / a.pair_rows);
+  const int blocks = pair_grid(a).special + (warps + kPairWarps - 1) / kPairWarps;
   if constexpr (sizeof(S) == 2) {
     if (a.sr) {
       pair_kernel<S, kForce, true><<<blocks, kPairThreads, 0, s>>>(a);

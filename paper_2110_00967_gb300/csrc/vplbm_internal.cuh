@@ -565,7 +565,7 @@ struct StepArgs {
   int32_t box[4];        // i0, i1, j0, j1 (inclusive): nodes around the body that the pair's
                          // special blocks update; i0 even, i1 odd; i1 < i0: none
   int32_t pair_rows;     // rows per warp of the bulk blocks
-  int32_t pair_bx;       // bulk blocks side by side (set at the launch)
+  int32_t pair_strips;   // strips side by side (set at the launch)
   const unsigned long long *rng_src;  // the rounding counter of this step's level
   unsigned long long *rng_dst;        // ... and of the next (written by the special kernel)
 };

@@ -77,6 +77,21 @@ def test_ragged_sizes(dtype, shape):
     run_both(w, (1, 4, 3))
 
 
+# rows per warp 5, 6 and 8 (by the lattice's size): a last run of one row, of a full
+# run and of all but one row, and 0, 2 and 3 warps in the last block of four
+RUNS = [(514, 5 * 41 + 5), (490, 5 * 43 + 4), (424, 5 * 48 + 8), (724, 6 * 93 + 5), (904, 8 * 97 + 5)]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16sr"])
+@pytest.mark.parametrize("shape", RUNS)
+def test_last_runs_and_warps(dtype, shape):
+    nx, ny = shape
+    body = W.Body("disk", length=17.0, x_c=80.4, y_c=0.5 * ny - 0.3)
+    w = W.Workload(name="runs", nx=nx, ny=ny, dtype=dtype, collision="trt", tau_plus=0.6, u_in=(0.04, 0.0),
+                   bc=("inlet", "outlet", "symmetry", "symmetry"), body=body, steps=1, u_ref=(0.04, 0.0))
+    run_both(w, (1, 4, 2))
+
+
 BCS = [("periodic", "periodic", "periodic", "periodic"), ("periodic", "periodic", "noslip", "noslip"),
        ("inlet", "outlet_free", "noslip", "noslip"), ("noslip", "noslip", "periodic", "periodic"),
        ("inlet", "noslip", "symmetry", "noslip"), ("inlet", "outlet", "periodic", "periodic")]
