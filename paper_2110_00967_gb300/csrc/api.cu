@@ -599,18 +599,23 @@ PairPlan pair_plan(const vplbm_ctx *c, const vplbm_body &b, const std::vector<Si
 // five sizes, FP16 stochastic: 6.5 us per lattice step singly, 6.6 in pairs with
 // long runs, 7.6 with short ones); alone and up to about 1.5 M nodes the GPU is
 // not full, and half as many launches win (512 x 256: 9.7 -> 4.2 us, 1024 x 512:
-// 10.2 -> 5.7, 1536 x 768: 12.2 -> 9.8, 2048 x 1024: 16.5 -> 16.6).
-constexpr int64_t kPair16Nodes = 1500000;
+// 10.2 -> 5.7, 1536 x 768: 12.2 -> 9.8, 2048 x 1024: 16.5 -> 16.6).  Every lattice
+// adds its frame and box on top of its nodes, counted as 100,000 nodes: FP16
+// stochastic, pairs against the older single steps, 4 lattices of 512 x 256 1.82
+// and 3.03, of 768 x 384 2.81 and 3.26, but 8 of 512 x 256 1.80 and 1.71 (1.71 as
+// single steps now).
+constexpr int64_t kPair16Nodes = 1600000, kPair16Lattice = 100000;
 constexpr int64_t kPairBatchNodes = 4000000;  // a full GPU: longer runs
-void choose_mode(vplbm_ctx *c, int64_t call_nodes) {
+void choose_mode(vplbm_ctx *c, int64_t call_nodes, int64_t lattices) {
   const int64_t own = (int64_t)c->L.nx * c->L.ny;
   const bool pairs =
-      c->pair_ok && !(elem_bytes(c->cfg.dtype) == 2 && call_nodes > kPair16Nodes);
+      c->pair_ok && !(elem_bytes(c->cfg.dtype) == 2 &&
+                      call_nodes + lattices * kPair16Lattice > kPair16Nodes);
   const bool alone = call_nodes < 2 * own || (pairs && call_nodes <= kPairBatchNodes);
   c->mode = pairs ? (alone ? kPairAlone : kPair) : (alone ? kSingleAlone : kSingle);
 }
 // ... for a lattice stepped by itself
-void choose_mode(vplbm_ctx *c) { choose_mode(c, (int64_t)c->L.nx * c->L.ny); }
+void choose_mode(vplbm_ctx *c) { choose_mode(c, (int64_t)c->L.nx * c->L.ny, 1); }
 
 bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
@@ -1663,7 +1668,7 @@ cudaError_t batch_join(vplbm_batch *b, cudaStream_t s) {
 void batch_modes(vplbm_batch *b) {
   int64_t nodes = 0;
   for (const vplbm_ctx *c : b->ctxs) nodes += (int64_t)c->L.nx * c->L.ny;
-  for (vplbm_ctx *c : b->ctxs) choose_mode(c, nodes);
+  for (vplbm_ctx *c : b->ctxs) choose_mode(c, nodes, (int64_t)b->ctxs.size());
 }
 
 // Every lattice replays step graphs (no per-step launches) from where it is.

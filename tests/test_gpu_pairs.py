@@ -170,3 +170,27 @@ def test_batch_of_lattices_stepped_in_pairs_and_singly():
         a.step(44)
         np.testing.assert_array_equal(a.get_f(), m.get_f())
         np.testing.assert_array_equal(a.history(V.MEM, 44), m.history(V.MEM, 44))
+
+
+@pytest.mark.parametrize("count, per_lattice", [(7, 4 + 1), (8, 2 * 8 + 1)])
+def test_sixteen_bit_batches_pair_up_to_their_nodes_and_lattices(count, per_lattice):
+    """16-bit lattices of 448 x 256 nodes: seven together step in pairs, eight do not
+    (each lattice weighs its nodes and a constant); the results are the same."""
+    works = [W.naca(2.0 * k, dtype="f16", nx=448, ny=256) for k in range(count)]
+    lats = [V.Lattice(V.config_of(w)) for w in works]
+    for lat, w in zip(lats, works):
+        lat.set_body(V.body_of(w))
+    batch = V.Batch(lats)
+    batch.step(1)
+    before = [lat.launches for lat in lats]
+    batch.step(8)
+    assert [lat.launches - b for lat, b in zip(lats, before)] == [per_lattice] * count
+    for lat, w in list(zip(lats, works))[:2]:
+        alone = V.Lattice(V.config_of(w))
+        alone.set_body(V.body_of(w))
+        for _ in range(9):
+            alone.step(1)
+        np.testing.assert_array_equal(lat.get_f(), alone.get_f())
+        for est in (V.MEM, V.SIM):
+            np.testing.assert_array_equal(lat.history(est, 9), alone.history(est, 9))
+    batch.close()
