@@ -60,7 +60,7 @@ __device__ __forceinline__ long long warp_sum(long long v) {
 }
 
 // adds the warp's fixed-point words into acc[slot][word] for the three
-// quantities starting at slot base
+// quantities starting at slot base (a low word as two: Fix<double>)
 template <typename T>
 __device__ __forceinline__ void warp_add(const FixAcc<T> &a, unsigned long long *acc, int base) {
   constexpr int W = Fix<T>::kWords;
@@ -75,7 +75,14 @@ __device__ __forceinline__ void warp_add(const FixAcc<T> &a, unsigned long long 
 #pragma unroll
     for (int k = 0; k < W; ++k) {
       const long long v = warp_sum(a.f[q][k]);
-      if ((threadIdx.x & 31) == 0 && v) atomicAdd(acc + 2 * (base + q) + k, (unsigned long long)v);
+      if ((threadIdx.x & 31) != 0 || !v) continue;
+      unsigned long long *word = acc + kSlotWords * (base + q) + k;
+      if (k == 0) {
+        atomicAdd(word, (unsigned long long)v);
+      } else {
+        atomicAdd(word, (unsigned long long)(v >> 26));
+        atomicAdd(word + 1, (unsigned long long)(v & Fix<double>::kLowMask));
+      }
     }
 }
 
@@ -533,18 +540,22 @@ __device__ __forceinline__ double moving_body(const StepArgs &p, BodyState &b, b
   const BodyState *from = p.finalize_prev ? p.body_prev : p.body_src;
   // all loads are issued together
   unsigned long long w = 0;
-  long long w0 = 0, w1 = 0;
+  long long w0 = 0, w1 = 0, w2 = 0;
   if (lane < kBodyWords) w = __ldcg(reinterpret_cast<const unsigned long long *>(from) + lane);
   if (p.finalize_prev && lane < kAccSlots) {
-    w0 = (long long)__ldcg(p.acc_prev + 2 * lane);
-    if (Fix<T>::kWords > 1) w1 = (long long)__ldcg(p.acc_prev + 2 * lane + 1);
+    const unsigned long long *slot = p.acc_prev + kSlotWords * lane;
+    w0 = (long long)__ldcg(slot);
+    if (Fix<T>::kWords > 1) {
+      w1 = (long long)__ldcg(slot + 1);
+      w2 = (long long)__ldcg(slot + 2);
+    }
   }
   const double inv = __ldg(p.rigid->inv + k), acc = __ldg(p.rigid->acc + k);
   if (lane < kBodyWords) reinterpret_cast<unsigned long long *>(&b)[lane] = w;
   __syncwarp();
   ok = true;
   if (!p.finalize_prev) return 0.0;
-  double tot = Fix<T>::value(w0, w1);
+  double tot = Fix<T>::value(w0, w1, w2);
   if (lane >= 3 && lane < 6) tot += p.sim_const[lane - 3];
   const double force = __shfl_sync(kFull, tot, b.estimator == VPLBM_SIM ? 3 + k : k);
   const double v0 = k == 0 ? b.ux : k == 1 ? b.uy : b.omega;
@@ -636,10 +647,12 @@ __device__ void finalize(const StepArgs &p) {
     long long step = 0;
     double v = 0.0;
     if (lane < kHistCols) {
-      const long long w0 = (long long)__ldcg(acc + 2 * lane);
-      const long long w1 = (long long)__ldcg(acc + 2 * lane + 1);
+      const unsigned long long *slot = acc + kSlotWords * lane;
+      const long long w0 = (long long)__ldcg(slot);
+      const long long w1 = (long long)__ldcg(slot + 1);
+      const long long w2 = (long long)__ldcg(slot + 2);
       step = __ldcg(p.dev_step) + row;
-      v = Fix<T>::value(w0, w1);
+      v = Fix<T>::value(w0, w1, w2);
       const bool is_sim = lane >= 3 && lane < 6;
       if (is_sim) v += p.sim_const[lane - 3];
       // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due

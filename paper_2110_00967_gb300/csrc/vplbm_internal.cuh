@@ -202,11 +202,16 @@ template <typename T>
 struct Fix;
 template <>
 struct Fix<double> {
-  // two words, units 2^-30 and 2^-82 (|sum| < 2^33): the magnitude rounded down
-  // to a multiple of 2^-82, both words with the value's sign.  Integer
-  // operations on the value's bits, which have their own lanes: GB300's FP64
-  // conversions wait for its two FP64 lanes per SM.
+  // Units 2^-30 and 2^-82 (|sum| < 2^33): the magnitude rounded to the nearest
+  // multiple of 2^-82, both words with the value's sign.  Integer operations on
+  // the value's bits, which have their own lanes: GB300's FP64 conversions wait
+  // for its two FP64 lanes per SM.  The low words of a body's terms add up (all of
+  // one sign they average 2^51, so some 4,000 would fill 64 bits, and a body has
+  // up to four million nodes): a warp's sum of them is added as two words, the
+  // multiples of 2^26 (unit 2^-56) and the rest (unit 2^-82, never negative),
+  // which leaves each 2^37 warps of headroom.
   static constexpr int kWords = 2;
+  static constexpr long long kLowMask = (1ll << 26) - 1;
   static __device__ __forceinline__ void split(double v, long long (&w)[2]) {
     const long long bits = __double_as_longlong(v);
     const int e = (int)(bits >> 52) & 0x7ff;
@@ -217,7 +222,7 @@ struct Fix<double> {
     if (s > 0) {
       hi = s < 64 ? m >> s : 0ull;
       const unsigned long long rest = s < 64 ? m & ((1ull << s) - 1ull) : m;
-      lo = s <= 52 ? rest << (52 - s) : (s < 116 ? rest >> (s - 52) : 0ull);
+      lo = s <= 52 ? rest << (52 - s) : (s < 116 ? (rest + (1ull << (s - 53))) >> (s - 52) : 0ull);
     } else {
       hi = m << min(-s, 63);
       lo = 0ull;
@@ -226,8 +231,12 @@ struct Fix<double> {
     w[0] = bits < 0 ? -(long long)hi : (long long)hi;
     w[1] = bits < 0 ? -(long long)lo : (long long)lo;
   }
-  static __host__ __device__ double value(long long w0, long long w1) {
-    return (double)w0 * 9.313225746154785e-10 + (double)w1 * 2.0679515313825692e-25;
+  // the sum of three accumulated words: the low ones are exact below one unit of
+  // the high one, so the value is rounded once (|sum| < 2^23)
+  static __host__ __device__ double value(long long w0, long long w1, long long w2) {
+    w1 += w2 >> 26;
+    const long long lo = (w1 & kLowMask) << 26 | (w2 & kLowMask);
+    return (double)(w0 + (w1 >> 26)) * 9.313225746154785e-10 + (double)lo * 2.0679515313825692e-25;
   }
 };
 template <>
@@ -243,15 +252,15 @@ struct Fix<float> {
   static __device__ __forceinline__ void split(float v, long long (&w)[1]) {
     w[0] = round_ll(v * 1099511627776.0f);  // 2^40
   }
-  static __host__ __device__ double value(long long w0, long long) {
+  static __host__ __device__ double value(long long w0, long long, long long) {
     return (double)w0 * 9.094947017729282e-13;  // 2^-40
   }
 };
-// accumulator words: (MEM Fx, Fy, T, SIM Fx, Fy, T) x two words
 // fixed-point sum slots: MEM F_x, F_y, T; SIM F_x, F_y, T; volume integral F_x, F_y, T
 constexpr int kAccSlots = 9;
 constexpr int kHistCols = 9;  // one history row per step: the same nine values
-constexpr int kAccWords = 2 * kAccSlots;
+constexpr int kSlotWords = 3;  // accumulator words per slot (FP32 compute uses the first)
+constexpr int kAccWords = kSlotWords * kAccSlots;
 
 // ---------------------------------------------------------------------------
 // lattice geometry and side conditions, shared by every kernel
@@ -521,7 +530,7 @@ struct StepArgs {
   const RigidConst *rigid;     // a moving body's constants
   const ForceRegion *reg_src;  // covers the body at level n (a moving one: by its margin,
   ForceRegion *reg_dst;        // from level n - 1); ... at level n + 1, for the next launch
-  unsigned long long *acc;       // [6][2] fixed-point sums of this step
+  unsigned long long *acc;       // [kAccSlots][kSlotWords] fixed-point sums of this step
   unsigned long long *acc_prev;  // the previous step's sums (finalized by this launch)
   unsigned long long *acc_next;  // a moving body's next sums, cleared by this launch
   int32_t finalize_prev;         // 1: an extra last block finalizes acc_prev first
