@@ -655,9 +655,12 @@ __device__ void finalize(const StepArgs &p) {
       v = Fix<T>::value(w0, w1, w2);
       const bool is_sim = lane >= 3 && lane < 6;
       if (is_sim) v += p.sim_const[lane - 3];
-      // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due
-      p.hist[kHistCols * (step % p.hist_len) + lane] =
-          !is_sim || do_sim ? v : __longlong_as_double(0x7ff8000000000000LL);
+      // MEM (0-2) and the volume integral (6-8) every step, SIM (3-5) when due;
+      // not the first of two steps in a ring of one row, which the second's warp
+      // writes with no order between them
+      if (rows - row <= p.hist_len)
+        p.hist[kHistCols * (step % p.hist_len) + lane] =
+            !is_sim || do_sim ? v : __longlong_as_double(0x7ff8000000000000LL);
       tot[row][lane] = v;
     }
     __syncwarp();

@@ -194,3 +194,25 @@ def test_sixteen_bit_batches_pair_up_to_their_nodes_and_lattices(count, per_latt
         for est in (V.MEM, V.SIM):
             np.testing.assert_array_equal(lat.history(est, 9), alone.history(est, 9))
     batch.close()
+
+
+@pytest.mark.parametrize("history_len", [1, 2, 3])
+def test_short_force_histories(history_len):
+    """A history of one row, of a pair's two, and of three: after every run the last
+    steps' forces are those of a lattice stepped one step per call."""
+    w = W.naca(9.0, dtype="f32", nx=517, ny=263)
+    runs, single = (V.Lattice(V.config_of(w, history_len=history_len)) for _ in range(2))
+    for lat in (runs, single):
+        lat.set_body(V.body_of(w))
+    for n in (1, 2, 6, 5, 32):
+        runs.step(n)
+        for _ in range(n):
+            single.step(1)
+        keep = min(history_len, runs.steps)
+        for est in (V.MEM, V.SIM, V.ANGOT):
+            np.testing.assert_array_equal(runs.history(est, keep), single.history(est, keep))
+        np.testing.assert_array_equal(runs.force_mem(), single.force_mem())
+        np.testing.assert_array_equal(runs.force_sim(), single.force_sim())
+        np.testing.assert_array_equal(runs.force_angot(), single.force_angot())
+        for a, b in zip(runs.sums(), single.sums()):
+            np.testing.assert_array_equal(a, b)
