@@ -1473,6 +1473,11 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
     return fail(c, VPLBM_EINVAL, "snapshot of a lattice with another configuration");
   if ((h.cur != 0 && h.cur != 1) || h.n_sim < 0 || h.n_sim > effective_max_sim(c->cfg))
     return fail(c, VPLBM_EINVAL, "corrupt snapshot header");
+  // everything that can be refused is looked at before the lattice is touched
+  std::vector<SimPoint> pts;
+  if (h.body_cfg.kind != VPLBM_BODY_NONE && !build_polygon(h.body_cfg, h.n_sim, pts))
+    return fail(c, VPLBM_EINVAL, "corrupt snapshot body");
+  const PairPlan plan = pair_plan(c, h.body_cfg, pts);
   const char *in = static_cast<const char *>(host);
   VPLBM_CUDA(c, cudaMemcpyAsync(c->ws + c->lay.prev[0], in + hb, tb, cudaMemcpyHostToDevice, c->stream));
   VPLBM_CUDA(c, cudaMemcpyAsync(c->buf[h.cur], in + hb + tb, pb, cudaMemcpyHostToDevice, c->stream));
@@ -1489,14 +1494,8 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
   c->n_sim = h.n_sim;
   c->sim_every = h.sim_every;
   c->region_slots = h.region_slots;
-  {
-    std::vector<SimPoint> pts;
-    if (h.body_cfg.kind != VPLBM_BODY_NONE && !build_polygon(h.body_cfg, h.n_sim, pts))
-      return fail(c, VPLBM_EINVAL, "corrupt snapshot body");
-    const PairPlan plan = pair_plan(c, h.body_cfg, pts);
-    c->pair_ok = plan.ok;
-    std::memcpy(c->box, plan.box, sizeof(plan.box));
-  }
+  c->pair_ok = plan.ok;
+  std::memcpy(c->box, plan.box, sizeof(plan.box));
   c->pending = false;
   c->pending_sim = false;
   c->turn = 0;

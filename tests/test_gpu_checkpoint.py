@@ -3,6 +3,8 @@ vplbm_load_state): a lattice restored from a snapshot continues bit for bit as
 the saved one did -- populations, outlet column, mask, force histories,
 running sums, step counter and the FP64 body state -- in FP32 and 16-bit
 storage, with a fixed airfoil and with a sedimenting disk."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -117,3 +119,26 @@ def test_snapshot_checks():
     with pytest.raises(V.VplbmError) as e:
         V.vplbm_save_state(bare.ctx)
     assert e.value.status == V.ESTATE
+
+
+def test_a_refused_snapshot_leaves_the_lattice_as_it_was():
+    """A header whose body has no polygon of the stored point count (a disk's 64 points
+    under an airfoil's kind): EINVAL, and the lattice goes on as if nothing had been
+    loaded."""
+    body = W.Body("disk", length=15.0, x_c=150.3, y_c=128.2, n_sim_points=64)
+    w = W.naca(5.0, dtype="f32", nx=512, ny=256).with_(body=body)
+    lat, twin = lattice(w), lattice(w)
+    lat.step(9)
+    bad = lat.save_state()
+    at = 16 + ctypes.sizeof(V.vplbm_config) + V.vplbm_body.kind.offset
+    assert bad[at:at + 4].view(np.int32)[0] == V.body_of(w).kind
+    bad[at:at + 4].view(np.int32)[0] = V.body_of(W.naca(5.0)).kind
+    lat.step(5)
+    twin.step(14)
+    with pytest.raises(V.VplbmError) as e:
+        lat.load_state(bad)
+    assert e.value.status == V.EINVAL
+    assert_same(record(lat, 14), record(twin, 14))
+    for x in (lat, twin):
+        x.step(7)
+    assert_same(record(lat, 21), record(twin, 21))
