@@ -116,12 +116,14 @@ __device__ __forceinline__ double to_double(long long v) {
 // (about 140 FP64 operations per node for nine conversions, the moments and two
 // divisions: 246 us for 2048 x 1024, where its traffic takes 19 us); FP32 offsets
 // are therefore summed as integers, which rounds less, and a node is left with
-// five FP64 operations.
+// five FP64 operations.  fixed: (ox, oy) fit beside the offsets' sums (six of
+// them, below 2.4 in magnitude, in 64 bits of unit 2^-60).
 template <typename S, bool kGather>
 __global__ void __launch_bounds__(kAuxThreads)
     get_fields_kernel(Lattice L, const S *buf, const typename Store<S>::T *prev,
                       const uint8_t *chi, const BodyState *body, double half_pen, double *rho_o,
-                      double *ux_o, double *uy_o, int j0, int rows, long long ox, long long oy) {
+                      double *ux_o, double *uy_o, int j0, int rows, long long ox, long long oy,
+                      bool fixed) {
   using T = typename Store<S>::T;
   const int i = blockIdx.x * kAuxThreads + threadIdx.x;
   if (i >= L.nx) return;
@@ -149,7 +151,7 @@ __global__ void __launch_bounds__(kAuxThreads)
       for (int a = 0; a < 9; ++a) v[a] = fixed60(h[a]);
       const long long s = v[0] + v[1] + v[2] + v[3] + v[4] + v[5] + v[6] + v[7] + v[8] + (1ll << kFixBits);
       // (NaN offsets fail the sum's comparison: fmaxf drops them)
-      exact = big < 0.4f && s > (1ll << (kFixBits - 10)) && h[0] + h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8] < 4.f;
+      exact = fixed && big < 0.4f && s > (1ll << (kFixBits - 10)) && h[0] + h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8] < 4.f;
       if (exact) {
         rho = to_double(s);
         jx = to_double(v[1] - v[3] + v[5] - v[6] + v[8] - v[7] + ox);
@@ -238,14 +240,15 @@ cudaError_t get_fields_t(bool gather, const Lattice &L, const void *buf, const v
   const T *prev = static_cast<const T *>(prev_v);
   const dim3 g((L.nx + kAuxThreads - 1) / kAuxThreads, rows < 65535 ? rows : 65535);
   const double unit = (double)(1ll << kFixBits);
-  const long long ox = llrint((L.ur[0] + 0.5 * L.bf[0]) * unit);
-  const long long oy = llrint((L.ur[1] + 0.5 * L.bf[1]) * unit);
+  const double mx = L.ur[0] + 0.5 * L.bf[0], my = L.ur[1] + 0.5 * L.bf[1];
+  const bool fixed = fabs(mx) < 4.0 && fabs(my) < 4.0;  // a body force may be larger
+  const long long ox = fixed ? llrint(mx * unit) : 0, oy = fixed ? llrint(my * unit) : 0;
   if (gather)
     get_fields_kernel<S, true><<<g, kAuxThreads, 0, s>>>(L, (const S *)buf, prev, chi, body,
-                                                         half_pen, rho, ux, uy, j0, rows, ox, oy);
+                                                         half_pen, rho, ux, uy, j0, rows, ox, oy, fixed);
   else
     get_fields_kernel<S, false><<<g, kAuxThreads, 0, s>>>(L, (const S *)buf, prev, chi, body,
-                                                          half_pen, rho, ux, uy, j0, rows, ox, oy);
+                                                          half_pen, rho, ux, uy, j0, rows, ox, oy, fixed);
   return cudaGetLastError();
 }
 
