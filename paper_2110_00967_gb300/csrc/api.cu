@@ -228,6 +228,12 @@ Extent extent_of(const vplbm_body &b, const std::vector<SimPoint> &pts) {
   return e;
 }
 
+// The polygon's place is finite: bounds taken over NaN points hold anything.
+bool finite_place(const vplbm_body &b) {
+  return std::isfinite(b.x_c) && std::isfinite(b.y_c) &&
+         (b.kind != VPLBM_BODY_NACA4 || std::isfinite(b.angle));
+}
+
 int default_sim_points(const vplbm_body &b) {
   if (b.n_sim_points > 0) return b.n_sim_points;
   if (b.kind == VPLBM_BODY_DISK) return (int)ceil(2.0 * M_PI * (0.5 * b.length) / 0.5);
@@ -924,6 +930,7 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
     if (b->kind != VPLBM_BODY_DISK && b->kind != VPLBM_BODY_NACA4)
       return fail(c, VPLBM_EINVAL, "unknown body kind");
     if (!(b->length > 0.0)) return fail(c, VPLBM_EINVAL, "body length must be > 0");
+    if (!finite_place(*b)) return fail(c, VPLBM_EINVAL, "non-finite body position or angle");
     if (b->kind == VPLBM_BODY_NACA4) {
       if (!(b->thickness > 0.0 && b->thickness < 0.5)) return fail(c, VPLBM_EINVAL, "bad NACA thickness");
       if (!(b->pivot_chord_frac >= 0.0 && b->pivot_chord_frac <= 1.0))
@@ -1475,7 +1482,8 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
     return fail(c, VPLBM_EINVAL, "corrupt snapshot header");
   // everything that can be refused is looked at before the lattice is touched
   std::vector<SimPoint> pts;
-  if (h.body_cfg.kind != VPLBM_BODY_NONE && !build_polygon(h.body_cfg, h.n_sim, pts))
+  if (h.body_cfg.kind != VPLBM_BODY_NONE &&
+      (!finite_place(h.body_cfg) || !build_polygon(h.body_cfg, h.n_sim, pts)))
     return fail(c, VPLBM_EINVAL, "corrupt snapshot body");
   const PairPlan plan = pair_plan(c, h.body_cfg, pts);
   const char *in = static_cast<const char *>(host);
