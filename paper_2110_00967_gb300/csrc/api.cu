@@ -234,6 +234,9 @@ bool finite_place(const vplbm_body &b) {
          (b.kind != VPLBM_BODY_NACA4 || std::isfinite(b.angle));
 }
 
+// an empty lattice has nothing to move, whatever the flag says
+bool moves(const vplbm_body &b) { return b.kind != VPLBM_BODY_NONE && b.moving != 0; }
+
 int default_sim_points(const vplbm_body &b) {
   if (b.n_sim_points > 0) return b.n_sim_points;
   if (b.kind == VPLBM_BODY_DISK) return (int)ceil(2.0 * M_PI * (0.5 * b.length) / 0.5);
@@ -579,7 +582,7 @@ struct PairPlan {
 PairPlan pair_plan(const vplbm_ctx *c, const vplbm_body &b, const std::vector<SimPoint> &pts) {
   PairPlan q;
   const Lattice &L = c->L;
-  if (c->cfg.dtype == VPLBM_F64 || b.moving || (int64_t)L.nx * L.ny < kPairMinNodes || L.nx < 64 ||
+  if (c->cfg.dtype == VPLBM_F64 || moves(b) || (int64_t)L.nx * L.ny < kPairMinNodes || L.nx < 64 ||
       L.ny < 32 || L.nx > 0xffff || L.ny > 0xffff || L.plane >= (int64_t)1 << 30)
     return q;
   if (b.kind != VPLBM_BODY_NONE) {
@@ -921,7 +924,7 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   bs.density_ratio = b->density_ratio;
   bs.gx = b->gravity[0];
   bs.gy = b->gravity[1];
-  bs.moving = b->moving;
+  bs.moving = moves(*b) ? b->moving : 0;
   bs.estimator = b->estimator;
   body_sync_f32(bs);
   std::vector<SimPoint> pts;
@@ -1002,7 +1005,7 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   // again, as a restarted solve does) keeps them: its geometry and state are
   // read from device memory at every step.
   const int new_slots = std::max(1, slots);
-  const int new_every = (b->moving && b->estimator == VPLBM_SIM) ? 1 : c->cfg.sim_every;
+  const int new_every = (moves(*b) && b->estimator == VPLBM_SIM) ? 1 : c->cfg.sim_every;
   const double new_const[3] = {cfx, cfy, ctq};
   const PairPlan plan = pair_plan(c, *b, pts);
   const bool keep_graphs = c->has_body && c->n_sim == n_sim && c->region_slots == new_slots &&
@@ -1053,7 +1056,7 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   // histories, sums, counters, status
   VPLBM_CUDA(c, cudaMemsetAsync(c->ws + c->lay.hist, 0, c->lay.body[0] - c->lay.hist, s));
   VPLBM_CUDA(c, cudaMemsetAsync(c->ws + c->lay.sums, 0, c->lay.total - c->lay.sums, s));
-  c->rigid_host = b->moving ? rigid_const(c->body_host) : RigidConst{};
+  c->rigid_host = moves(*b) ? rigid_const(c->body_host) : RigidConst{};
   VPLBM_CUDA(c, cudaMemcpyAsync(c->rigid, &c->rigid_host, sizeof(RigidConst), cudaMemcpyHostToDevice, s));
   VPLBM_CUDA(c, cudaMemsetAsync(c->prev[0], 0, 3 * (size_t)L.ny * sizeof(double), s));
   VPLBM_CUDA(c, cudaMemsetAsync(c->prev[1], 0, 3 * (size_t)L.ny * sizeof(double), s));
@@ -1489,6 +1492,7 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
   const char *in = static_cast<const char *>(host);
   VPLBM_CUDA(c, cudaMemcpyAsync(c->ws + c->lay.prev[0], in + hb, tb, cudaMemcpyHostToDevice, c->stream));
   VPLBM_CUDA(c, cudaMemcpyAsync(c->buf[h.cur], in + hb + tb, pb, cudaMemcpyHostToDevice, c->stream));
+  if (!moves(h.body_cfg)) h.body_host.moving = 0;
   c->rigid_host = h.body_host.moving ? rigid_const(h.body_host) : RigidConst{};
   VPLBM_CUDA(c, cudaMemcpyAsync(c->rigid, &c->rigid_host, sizeof(RigidConst), cudaMemcpyHostToDevice, c->stream));
   if (vplbm_status st = sync(c)) return st;
