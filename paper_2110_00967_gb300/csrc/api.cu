@@ -237,6 +237,14 @@ bool finite_place(const vplbm_body &b) {
 // an empty lattice has nothing to move, whatever the flag says
 bool moves(const vplbm_body &b) { return b.kind != VPLBM_BODY_NONE && b.moving != 0; }
 
+// Blocks reserved for the tiles of a body's force region (count tiles where it
+// stands): a moving body's box covers at most this many tiles anywhere.
+int region_slots_of(const vplbm_body &b, int count) {
+  if (!moves(b)) return std::max(1, count);
+  const double span = 2.0 * (0.5 * b.length + kRegionMargin) + 3.0;
+  return ((int)(span / kTileX) + 2) * ((int)(span / kTileY) + 2);
+}
+
 int default_sim_points(const vplbm_body &b) {
   if (b.n_sim_points > 0) return b.n_sim_points;
   if (b.kind == VPLBM_BODY_DISK) return (int)ceil(2.0 * M_PI * (0.5 * b.length) / 0.5);
@@ -982,14 +990,6 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   } else {
     reg.count = 1;
   }
-  // blocks reserved for region tiles: the region's tile count, or for a
-  // moving body the most tiles a box of its size can cover anywhere
-  int slots = reg.count;
-  if (b->kind != VPLBM_BODY_NONE && b->moving) {
-    const double span = 2.0 * (0.5 * b->length + kRegionMargin) + 3.0;
-    slots = ((int)(span / tw) + 2) * ((int)(span / kTileY) + 2);
-    slots = std::min(slots, kRegionCapacity);
-  }
   // the constant part of the SIM sum: -(1/3) sum S_i n_i and its moment
   // (zero for a closed polygon up to round-off), in FP64 in point order
   double cfx = 0.0, cfy = 0.0, ctq = 0.0;
@@ -1004,7 +1004,7 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   // it moves, the SIM cadence.  A body with the same ones (the same body placed
   // again, as a restarted solve does) keeps them: its geometry and state are
   // read from device memory at every step.
-  const int new_slots = std::max(1, slots);
+  const int new_slots = region_slots_of(*b, reg.count);
   const int new_every = (moves(*b) && b->estimator == VPLBM_SIM) ? 1 : c->cfg.sim_every;
   const double new_const[3] = {cfx, cfy, ctq};
   const PairPlan plan = pair_plan(c, *b, pts);
@@ -1505,7 +1505,7 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
   c->pre = h.pre != 0;
   c->n_sim = h.n_sim;
   c->sim_every = h.sim_every;
-  c->region_slots = h.region_slots;
+  c->region_slots = std::max(h.region_slots, region_slots_of(h.body_cfg, 1));
   c->pair_ok = plan.ok;
   std::memcpy(c->box, plan.box, sizeof(plan.box));
   c->pending = false;

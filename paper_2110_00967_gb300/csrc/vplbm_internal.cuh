@@ -44,7 +44,7 @@ __host__ __device__ __forceinline__ constexpr double w_of(int a) {
 constexpr int kTileX = 128;
 constexpr int kTileY = 2;
 constexpr int kThreads = kTileX * kTileY;
-constexpr int kRegionCapacity = 16384;  // force-region tiles
+constexpr int kRegionCapacity = 16384;  // force-region tiles of a body where it is placed
 // SIM points per block of the special kernel: a fixed body's points read
 // their cached nodes (memory latency only); a moving body's walk evaluates the
 // body's FP64 predicate, and GB300's FP64 rate per SM is low, so its points

@@ -62,3 +62,30 @@ def test_an_empty_lattice_has_nothing_to_move(dtype, length):
     np.testing.assert_array_equal(lat.get_f(), twin.get_f())
     assert not lat.get_mask().any()
     assert not lat.history(V.MEM, 7).any()
+
+
+def test_a_large_disk_moving_onto_one_more_column_of_tiles():
+    """A disk whose box covers 16 columns of tiles where it is placed and 17 a step later
+    (16,388 tiles): every node of the box is updated.  The same steps are taken by a
+    lattice set to each level's populations before its step, which updates every tile
+    of the lattice."""
+    body = W.Body("disk", length=1918.0, x_c=1084.0, y_c=980.0, moving=True, density_ratio=50.0, n_sim_points=1000)
+    w = W.Workload(name="wide", nx=2112, ny=1960, dtype="f32", collision="trt", tau_plus=0.7, u_in=(0.0, 0.0),
+                   bc=("noslip",) * 4, body=body, steps=1)
+    b = V.body_of(w)
+    b.u[0] = 0.2
+    runs, whole = V.Lattice(V.config_of(w)), V.Lattice(V.config_of(w))
+    f = W.random_field(5, (9, w.ny, w.nx), lo=0.10, hi=0.12)
+    for lat in (runs, whole):
+        lat.set_body(b)
+        lat.set_state(f, f, post_collision=False)
+    for _ in range(5):
+        runs.step(1)
+        whole.step(1)
+        f = runs.get_f()
+        # offsets of up to 0.4 read back and set again: one unit of FP32 at most
+        np.testing.assert_allclose(f, whole.get_f(), rtol=0, atol=2.0 ** -22)
+        np.testing.assert_allclose(runs.get_body(), whole.get_body(), rtol=1e-9, atol=1e-9)
+        whole.set_state(f, f, post_collision=False)
+    assert runs.get_body()[0] > 1084.5
+    runs.check()
