@@ -371,6 +371,7 @@ CollideC<T> collide_coeffs(double sp, double sm) {
   q.sp_w5 = (T)(sp * w_of(5));
   q.sp_45w1 = (T)(4.5 * sp * w_of(1));
   q.sp_9w5 = (T)(9.0 * sp * w_of(5));
+  q.halves = -q.nsm_half >= (T)0.25 ? 1 : 0;
   return q;
 }
 

@@ -814,7 +814,17 @@ struct Moments {
 // conserving mass exactly up to the rounding of that sum.  kForce = false
 // drops the forcing term (G = 0: a fluid node without body force), kRef = false
 // the terms of u_ref (zero).
-template <typename V, bool kForce, bool kRef = true>
+//
+// kHalves writes a pair as half its sum and half its difference, o_a,b = P +- M,
+// and the rest population as what they leave of rho: eight operations fewer than
+// adding the changes to h, for FP64 (bound by its operation count) where it rounds
+// no worse than the form with (c.u)^2.  That is s- >= 1/2: M then takes
+// (1 - s-)/2 <= 1/4 of the difference, an exact coefficient.  Below, the rounding
+// of the difference itself enters at half its size and the coefficient is rounded:
+// momentum error of a collision at s- = 0.17, in 1e-18: 3.2 with a bias of 1.7 for
+// halves, 1.6 for the form with (c.u)^2, 1.5 for changes added to h; at s- = 0.51
+// 2.6, 2.9 and 2.0; at s- = 1.5 4.7, 7.7 and 4.4.
+template <typename V, bool kForce, bool kRef = true, bool kHalves = false>
 __device__ __forceinline__ void collide(const V (&h)[9], const Moments<V> &m, V djx, V djy, V ux,
                                         V uy, V dux, V duy, V gx, V gy,
                                         const Consts<typename Val<V>::T> &c, V (&o)[9]) {
@@ -827,11 +837,6 @@ __device__ __forceinline__ void collide(const V (&h)[9], const Moments<V> &m, V 
   const V axis = vmul(k(c.sp_w1), vfma(k((T)-1.5), t, m.drho));
   const V diag = vmul(k(c.sp_w5), vfma(k((T)3), t, m.drho));
   V even{};
-  // FP64 (bound by its operation count) writes the pair as half its sum and half
-  // its difference, o_a,b = P +- M, and the rest population as what they leave of
-  // rho: eight operations fewer.  FP32 adds the small changes to h, which rounds
-  // less.
-  constexpr bool kHalves = std::is_same<V, double>::value;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int a = q < 2 ? q + 1 : q + 3, b = opp_of(a);
@@ -863,9 +868,9 @@ __device__ __forceinline__ void collide(const V (&h)[9], const Moments<V> &m, V 
 // The update of fluid nodes (no penalization): moments, velocity and the
 // collision, from the pre-collision offsets h of a node (FP64), a node pair or
 // one node in both lanes (FP32); kForce adds the uniform body force, kRef = false
-// leaves out u_ref = 0 (seven operations; FP64 lattices store offsets from rest).
-// Returns rho.
-template <typename V, bool kForce, bool kRef = true>
+// leaves out u_ref = 0 (seven operations; FP64 lattices store offsets from rest);
+// kHalves: see collide().  Returns rho.
+template <typename V, bool kForce, bool kRef = true, bool kHalves = false>
 __device__ __forceinline__ V fluid_update(const Lattice &L, const Consts<typename Val<V>::T> &cst,
                                           const V (&h)[9], V (&o)[9]) {
   using T = typename Val<V>::T;
@@ -883,7 +888,7 @@ __device__ __forceinline__ V fluid_update(const Lattice &L, const Consts<typenam
   const V duy = vmul(kRef ? vfma(m.drho, Val<V>::splat(-cst.ury), djy) : djy, inv);
   const V ux = kRef ? vadd(Val<V>::splat(cst.urx), dux) : dux;
   const V uy = kRef ? vadd(Val<V>::splat(cst.ury), duy) : duy;
-  collide<V, kForce, kRef>(h, m, djx, djy, ux, uy, dux, duy, gx, gy, cst, o);
+  collide<V, kForce, kRef, kHalves>(h, m, djx, djy, ux, uy, dux, duy, gx, gy, cst, o);
   return rho;
 }
 
@@ -996,8 +1001,9 @@ __device__ __forceinline__ V update_fluid(const Lattice &L,
   if constexpr (sizeof(S) == 2)
     return fluid_update16<kForce>(L, cst, h, o);
   else if constexpr (sizeof(S) == 8)
-    return cst.urx == 0.0 && cst.ury == 0.0 ? fluid_update<V, kForce, false>(L, cst, h, o)
-                                            : fluid_update<V, kForce>(L, cst, h, o);
+    return cst.urx != 0.0 || cst.ury != 0.0 ? fluid_update<V, kForce>(L, cst, h, o)
+           : cst.halves                     ? fluid_update<V, kForce, false, true>(L, cst, h, o)
+                                            : fluid_update<V, kForce, false>(L, cst, h, o);
   else
     return fluid_update<V, kForce>(L, cst, h, o);
 }

@@ -495,6 +495,7 @@ struct CollideC {
   T nsp_half, nsm_half;                 // -s+/2, -s-/2
   T sp_w1, sp_w5, sp_45w1, sp_9w5;      // s+ w1, s+ w5, 4.5 s+ w1, 9 s+ w5
   T sm_k1, sm_k2;
+  int32_t halves;  // 1: s- >= 1/2 (FP64 collision: step.cu, collide)
 };
 
 // ---------------------------------------------------------------------------
