@@ -70,20 +70,23 @@ __device__ __forceinline__ void warp_add(const FixAcc<T> &a, unsigned long long 
 #pragma unroll
     for (int k = 0; k < W; ++k) any |= a.f[q][k];
   if (!__any_sync(kFull, any != 0)) return;
+  // a lane per accumulator word: one instruction adds them all
+  const int lane = threadIdx.x & 31;
+  long long mine = 0;
 #pragma unroll
   for (int q = 0; q < 3; ++q)
 #pragma unroll
     for (int k = 0; k < W; ++k) {
       const long long v = warp_sum(a.f[q][k]);
-      if ((threadIdx.x & 31) != 0 || !v) continue;
-      unsigned long long *word = acc + kSlotWords * (base + q) + k;
       if (k == 0) {
-        atomicAdd(word, (unsigned long long)v);
+        if (lane == kSlotWords * q) mine = v;
       } else {
-        atomicAdd(word, (unsigned long long)(v >> 26));
-        atomicAdd(word + 1, (unsigned long long)(v & Fix<double>::kLowMask));
+        if (lane == kSlotWords * q + 1) mine = v >> 26;
+        if (lane == kSlotWords * q + 2) mine = v & Fix<double>::kLowMask;
       }
     }
+  if (lane < 3 * kSlotWords && mine)
+    atomicAdd(acc + kSlotWords * base + lane, (unsigned long long)mine);
 }
 
 // The force terms are written with named roundings, so that a state gives the
