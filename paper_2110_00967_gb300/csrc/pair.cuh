@@ -124,11 +124,14 @@ constexpr int kPairMinBlocks = 4;
 template <typename S>
 constexpr bool kRing = sizeof(S) == 4;
 
+// (the memory clobber keeps the ring's reads and later copies into the same stage
+// in program order)
 template <typename Raw>
 __device__ __forceinline__ void copy_async(Raw *smem, const void *global) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(
                    (uint32_t)__cvta_generic_to_shared(smem)),
-               "l"(global), "n"(sizeof(Raw)));
+               "l"(global), "n"(sizeof(Raw))
+               : "memory");
 }
 
 template <typename S, bool kForce, bool kSR>
