@@ -391,12 +391,14 @@ vplbm_status vplbm_batch_step(vplbm_batch *batch, int32_t nsteps);
  * stream).  It also builds a call of nsteps steps as one graph: every
  * lattice's run of step graphs as a chain of child graphs, the chains side by
  * side, for the lattices' current buffers and for the other ones (where they
- * stand after an odd step count).  A later vplbm_batch_step of nsteps steps
+ * stand after an odd step count; where some lattices take two steps per launch
+ * and some one, also for the buffers that such a call leaves them in).  A later vplbm_batch_step of nsteps steps
  * is then one graph launch on the batch's stream, as long as every lattice
  * starts from a buffer it was built for and none of the step graphs was
  * rebuilt since (vplbm_set_body, vplbm_load_state, a change of launch form);
  * other calls take the per-lattice path, with the same results.  At most
- * eight such graphs are kept per batch.  Synchronises.  ESTATE when a
+ * sixteen such graphs are kept per batch: the last four step counts prepared
+ * for a batch of both kinds of lattices, eight otherwise.  Synchronises.  ESTATE when a
  * lattice has no body placed. */
 vplbm_status vplbm_batch_prepare(vplbm_batch *batch, int32_t nsteps);
 

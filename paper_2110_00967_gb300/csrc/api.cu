@@ -1720,7 +1720,9 @@ const BatchGraph *find_batch_graph(const vplbm_batch *b, int n) {
   return nullptr;
 }
 
-constexpr size_t kBatchGraphsKept = 8;
+// a prepared step count has two graphs, or four where some lattices step in pairs
+// and some singly (vplbm_batch_prepare): four such counts are kept
+constexpr size_t kBatchGraphsKept = 16;
 
 // Builds (and uploads on s) the batch graph of n steps from the buffers cur.
 vplbm_status build_batch_graph(vplbm_batch *b, int n, const std::vector<int> &cur, cudaStream_t s) {

@@ -279,3 +279,37 @@ def test_batch_on_its_own_stream_orders_the_lattices_streams():
     other = lattice(w)
     other.step(1 + 16 + 7 + 2)
     same_state(other, members[1], 26)
+
+
+def test_four_prepared_counts_of_a_mixed_batch_are_kept():
+    """A lattice stepped two steps per launch beside one stepped singly: each of four
+    prepared step counts has four graphs (the lattices' buffers move apart).  Preparing
+    any of them again, after calls of all of them, finds its graphs: it builds nothing,
+    which takes well under a tenth of the first time."""
+    import time
+    works = [W.naca(7.0, dtype="f32", nx=512, ny=256), W.naca(7.0, dtype="f32", nx=256, ny=128)]
+    members, alone = [lattice(w) for w in works], [lattice(w) for w in works]
+    batch = V.Batch(members)
+    batch.step(1)
+    batch.prepare(4)  # the step graphs of the powers of two
+
+    def seconds(n):
+        batch.stream.synchronize()
+        t = time.perf_counter()
+        batch.prepare(n)
+        return time.perf_counter() - t
+
+    counts = (8, 10, 6, 14)
+    first = [seconds(n) for n in counts]
+    again = []
+    for _ in range(3):
+        for n in counts:
+            batch.step(n)
+        again.append([seconds(n) for n in counts])
+    for t0, t1 in zip(first, np.min(again, axis=0)):
+        assert t1 < 0.1 * t0, (first, again)
+    total = 1 + 3 * sum(counts)
+    for a, m in zip(alone, members):
+        a.step(total)
+        same_state(a, m, total)
+    batch.close()
