@@ -184,7 +184,10 @@ vplbm_status vplbm_set_body(vplbm_ctx *ctx, const vplbm_body *body);
  * Runs of steps are replayed from CUDA graphs of 1, 2, 4, ..., 32 steps,
  * captured (all of them, from either population buffer) at the first run
  * that can use one: when the lattice is past its first step and SIM runs
- * every step or never.  In these graphs a lattice with a fixed body or none,
+ * every step or never.  How a lattice is stepped also depends on how much the
+ * call steps beside it (vplbm_batch_step): alone or in a small batch, and in one
+ * that fills the GPU, it has graphs of their own, captured at the first call of
+ * each kind (about 1 ms per lattice) unless vplbm_prepare has captured them.  In these graphs a lattice with a fixed body or none,
  * FP32 or 16-bit storage and at least 100000 nodes takes two steps per launch
  * where that is faster; the results are those of single steps bit for bit.  The
  * call returns with the last step's forces in the history. */
@@ -194,8 +197,8 @@ vplbm_status vplbm_step(vplbm_ctx *ctx, int32_t nsteps);
  * (a run of more than 32 steps is replayed in 32-step graphs and one graph of
  * the remainder), so that the first run of that length pays for no capture
  * and replays one graph where it would otherwise replay several (20 steps:
- * one graph instead of 16 + 4).  No counterpart in the paper; it changes no
- * result.  The prepared length is kept until the context is destroyed (graphs
+ * one graph instead of 16 + 4), whether the lattice is then stepped alone or in
+ * a batch of any size.  No counterpart in the paper; it changes no result.  The prepared length is kept until the context is destroyed (graphs
  * dropped by vplbm_set_body or a change of launch form are captured again at
  * the next run).  Synchronises the stream.  ESTATE before vplbm_set_body.
  * Lattices whose SIM runs on some steps only (sim_every > 1) queue their
@@ -386,9 +389,10 @@ vplbm_status vplbm_batch_create(vplbm_ctx *const *ctxs, int32_t n, void *cuda_st
  * seen by the next call. */
 vplbm_status vplbm_batch_step(vplbm_batch *batch, int32_t nsteps);
 
-/* vplbm_prepare for every lattice of the batch (the runs of a batch call are
- * at most 32 steps per lattice; each graph is uploaded on its lattice's chain
- * stream).  It also builds a call of nsteps steps as one graph: every
+/* Captures and uploads, now, the step graphs that this batch's calls of nsteps
+ * steps use (the runs of a batch call are at most 32 steps per lattice; each
+ * graph is uploaded on its lattice's chain stream; the lengths are kept as by
+ * vplbm_prepare).  It also builds a call of nsteps steps as one graph: every
  * lattice's run of step graphs as a chain of child graphs, the chains side by
  * side, for the lattices' current buffers and for the other ones (where they
  * stand after an odd step count; where some lattices take two steps per launch

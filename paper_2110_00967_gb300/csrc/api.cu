@@ -630,10 +630,17 @@ void choose_mode(vplbm_ctx *c, int64_t call_nodes, int64_t lattices) {
       c->pair_ok && !(elem_bytes(c->cfg.dtype) == 2 &&
                       call_nodes + lattices * kPair16Lattice > kPair16Nodes);
   const bool alone = call_nodes < 2 * own || (pairs && call_nodes <= kPairBatchNodes);
-  c->mode = pairs ? (alone ? kPairAlone : kPair) : (alone ? kSingleAlone : kSingle);
+  if (pairs)
+    c->mode = alone ? kPairAlone : kPair;
+  else  // FP64 and moving bodies: the same kernels either way
+    c->mode = alone && c->cfg.dtype != VPLBM_F64 && !c->body_host.moving ? kSingleAlone : kSingle;
 }
 // ... for a lattice stepped by itself
 void choose_mode(vplbm_ctx *c) { choose_mode(c, (int64_t)c->L.nx * c->L.ny, 1); }
+// ... and for one among so many that the GPU is full
+void choose_mode_full(vplbm_ctx *c) {
+  choose_mode(c, std::max(kPairBatchNodes, 2 * (int64_t)c->L.nx * c->L.ny) + 1, 2);
+}
 
 bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
@@ -1106,6 +1113,10 @@ vplbm_status vplbm_prepare(vplbm_ctx *c, int32_t nsteps) {
   if (!c->has_body) return fail(c, VPLBM_ESTATE, "no body placed (vplbm_set_body)");
   want_length(c, nsteps);
   if (c->sim_every > 1) return VPLBM_OK;  // steps are queued one by one
+  // a lattice steps one way alone or in a small batch, and another in a large one:
+  // the graphs of both (0.6 to 1.5 ms each), so that no later call captures them
+  choose_mode_full(c);
+  if (vplbm_status st = ensure_graphs(c, c->stream)) return st;
   choose_mode(c);
   if (vplbm_status st = ensure_graphs(c, c->stream)) return st;
   return sync(c);

@@ -313,3 +313,32 @@ def test_four_prepared_counts_of_a_mixed_batch_are_kept():
         a.step(total)
         same_state(a, m, total)
     batch.close()
+
+
+@pytest.mark.parametrize("dtype,shape,count", [("f32", (1024, 512), 12), ("f16sr", (512, 256), 16), ("f64", (256, 128), 12)])
+def test_lattices_prepared_alone_are_prepared_for_a_batch(dtype, shape, count):
+    """vplbm_prepare on every lattice, then a batch of them large enough to be stepped in
+    another way than a lattice alone: the first call captures nothing (several
+    milliseconds for a dozen lattices that were not prepared), and the lattices end
+    as lone ones."""
+    import time
+    w = W.naca(7.0, dtype=dtype, nx=shape[0], ny=shape[1])
+    seconds = {}
+    for prepared in (False, True):
+        lats = [lattice(w) for _ in range(count)]
+        for lat in lats:
+            lat.step(1)
+            if prepared:
+                lat.prepare(20)
+        batch = V.Batch(lats)
+        batch.stream.synchronize()
+        t = time.perf_counter()
+        batch.step(20)
+        batch.stream.synchronize()
+        seconds[prepared] = time.perf_counter() - t
+        alone = lattice(w)
+        alone.step(21)
+        for lat in (lats[0], lats[-1]):
+            same_state(alone, lat, 21)
+        batch.close()
+    assert seconds[True] < 0.5 * seconds[False], seconds
