@@ -60,9 +60,8 @@ def test_airfoil_runs_equal_single_steps(dtype, force):
     assert launches[3] == 16 + 1
 
 
-# the two outermost columns, a strip of 30 cells (60 FP32 or 120 16-bit nodes), a
-# block of 4 strips, runs of 16 rows, frame tiles of 62 nodes: sizes one below,
-# at and one above their multiples
+# strips of 60 nodes between the two outermost columns on either side: widths one
+# below, at and one above their multiples, a narrow and a low lattice
 SIZES = [(4 * 60 + 4, 2 * 62 + 4 + 300), (4 * 60 + 5, 433), (8 * 60 + 3, 16 * 14 + 4), (62 * 8, 16 * 14 + 5),
          (62 * 8 + 1, 16 * 14 + 3), (2 * 480 + 4, 128), (1500, 70), (67, 1571)]
 
@@ -216,3 +215,52 @@ def test_short_force_histories(history_len):
         np.testing.assert_array_equal(runs.force_angot(), single.force_angot())
         for a, b in zip(runs.sums(), single.sums()):
             np.testing.assert_array_equal(a, b)
+
+
+# rows per warp 20, as batches of more than four million FP32 nodes take them: a last
+# run of 20, one and 19 rows, and two, three and one warps in the last block of four
+LARGE = [(2044, 20 * 51 + 4), (1500, 20 * 50 + 5), (2084, 20 * 38 + 23)]
+
+
+def test_large_batches_equal_single_steps():
+    works = [W.naca(4.0 + 5 * k, dtype="f32", nx=nx, ny=ny) for k, (nx, ny) in enumerate(LARGE)]
+    members, alone = ([V.Lattice(V.config_of(w)) for w in works] for _ in range(2))
+    for lats in (members, alone):
+        for lat, w in zip(lats, works):
+            lat.set_body(V.body_of(w))
+    batch = V.Batch(members)
+    batch.step(1)
+    batch.prepare(8)
+    before = [m.launches for m in members]
+    for n in (8, 3, 8):
+        batch.step(n)
+    # four launches and one that finalizes for 8 steps; one pair, one step and their
+    # finalizing launches for 3
+    assert [m.launches - b for m, b in zip(members, before)] == [5 + 2 + 3 + 5] * len(LARGE)
+    batch.close()
+    for a, m in zip(alone, members):
+        for _ in range(20):
+            a.step(1)
+        np.testing.assert_array_equal(a.get_f(), m.get_f())
+        for est in (V.MEM, V.SIM, V.ANGOT):
+            np.testing.assert_array_equal(a.history(est, 20), m.history(est, 20))
+        for p, q in zip(a.sums(), m.sums()):
+            np.testing.assert_array_equal(p, q)
+
+
+# frame tiles of 30 nodes along the rows and along the columns between them: sizes at,
+# one above and one below their multiples
+FRAMES = [(30 * 14, 30 * 10 + 4), (30 * 14 + 1, 30 * 10 + 5), (30 * 14 + 29, 30 * 10 + 33)]
+
+
+@pytest.mark.parametrize("length", range(15, 29))
+def test_ends_of_frame_and_box_tiles(length):
+    """Box tiles of 14 x 6 nodes around disks of fourteen sizes, so that the last tile
+    of either direction is of every size; frame tiles in turn."""
+    nx, ny = FRAMES[length % 3]
+    body = W.Body("disk", length=float(length), x_c=90.3, y_c=0.5 * ny + 0.2)
+    w = W.Workload(name="tiles", nx=nx, ny=ny, dtype="f32" if length % 2 else "f16sr", collision="trt",
+                   tau_plus=0.6, u_in=(0.04, 0.0), bc=("inlet", "outlet", "symmetry", "noslip"), body=body,
+                   steps=1, u_ref=(0.04, 0.0))
+    start = W.random_field(length, (9, ny, nx), lo=0.10, hi=0.12)
+    run_both(w, (1, 4, 3), start=start)
