@@ -944,6 +944,7 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   bs.estimator = b->estimator;
   body_sync_f32(bs);
   std::vector<SimPoint> pts;
+  Extent box;
   int n_sim = 0;
   if (b->kind != VPLBM_BODY_NONE) {
     if (b->kind != VPLBM_BODY_DISK && b->kind != VPLBM_BODY_NACA4)
@@ -965,34 +966,18 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
     if (n_sim > effective_max_sim(c->cfg))
       return fail(c, VPLBM_EINVAL, fmt("%d SIM points exceed the capacity %d", n_sim, effective_max_sim(c->cfg)));
     if (!build_polygon(*b, n_sim, pts)) return fail(c, VPLBM_EINVAL, "bad SIM point count for this body");
-    // the body (its polygon, with one node of margin) must lie inside the lattice
-    double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
-    for (const SimPoint &p : pts) {
-      x0 = std::min(x0, b->x_c + p.dx - 0.5 * p.s);
-      x1 = std::max(x1, b->x_c + p.dx + 0.5 * p.s);
-      y0 = std::min(y0, b->y_c + p.dy - 0.5 * p.s);
-      y1 = std::max(y1, b->y_c + p.dy + 0.5 * p.s);
-    }
-    if (!(x0 >= 0.0 && y0 >= 0.0 && x1 <= L.nx - 1.0 && y1 <= L.ny - 1.0))
+    // the body's polygon must lie inside the lattice
+    box = extent_of(*b, pts);
+    if (!(box.x0 >= 0.0 && box.y0 >= 0.0 && box.x1 <= L.nx - 1.0 && box.y1 <= L.ny - 1.0))
       return fail(c, VPLBM_EINVAL, "body does not fit in the lattice");
   }
-  // force region: tiles around the body (its farthest polygon point from the
-  // reference point sets the extent); tile (0, 0) alone for an empty lattice
-  double extent = 0.0, bx0 = 1e300, bx1 = -1e300, by0 = 1e300, by1 = -1e300;
-  for (const SimPoint &p : pts) {
-    extent = std::max(extent, sqrt(p.dx * p.dx + p.dy * p.dy) + 0.5 * p.s);
-    bx0 = std::min(bx0, b->x_c + p.dx - 0.5 * p.s);
-    bx1 = std::max(bx1, b->x_c + p.dx + 0.5 * p.s);
-    by0 = std::min(by0, b->y_c + p.dy - 0.5 * p.s);
-    by1 = std::max(by1, b->y_c + p.dy + 0.5 * p.s);
-  }
+  // force region: tiles around the body; tile (0, 0) alone for an empty lattice
   const int tw = kTileX;
   const int ntx = (L.nx + tw - 1) / tw, nty = (L.ny + kTileY - 1) / kTileY;
   ForceRegion reg{};
   if (b->kind != VPLBM_BODY_NONE) {
     reg = b->moving ? make_region(L, b->x_c, b->y_c, 0.5 * b->length, ntx, nty, tw)
-                    : make_region_box(L, bx0, bx1, by0, by1, ntx, nty, tw);
-    reg.error = 0;
+                    : make_region_box(L, box.x0, box.x1, box.y0, box.y1, ntx, nty, tw);
     if (reg.count > kRegionCapacity)
       return fail(c, VPLBM_EINVAL, fmt("body too large: %d force-region tiles (capacity %d)", reg.count, kRegionCapacity));
   } else {
@@ -1044,8 +1029,8 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
     // the predicate only where the body can be: its polygon's box with a
     // margin of three nodes (the surface bulges beyond the polygon's edges
     // by far less than a node); interface bits one node wider
-    int i0 = std::max(0, (int)floor(bx0) - 3), i1 = std::min(L.nx - 1, (int)ceil(bx1) + 3);
-    int j0 = std::max(0, (int)floor(by0) - 3), j1 = std::min(L.ny - 1, (int)ceil(by1) + 3);
+    int i0 = std::max(0, (int)floor(box.x0) - 3), i1 = std::min(L.nx - 1, (int)ceil(box.x1) + 3);
+    int j0 = std::max(0, (int)floor(box.y0) - 3), j1 = std::min(L.ny - 1, (int)ceil(box.y1) + 3);
     // a box reaching a periodic side: its neighbours across the side too
     if (L.bc[0] == VPLBM_PERIODIC && (i0 == 0 || i1 == L.nx - 1)) i0 = 0, i1 = L.nx - 1;
     if (L.bc[2] == VPLBM_PERIODIC && (j0 == 0 || j1 == L.ny - 1)) j0 = 0, j1 = L.ny - 1;

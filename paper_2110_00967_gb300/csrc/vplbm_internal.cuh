@@ -481,7 +481,7 @@ __device__ __forceinline__ bool neighbour(const Lattice &L, int a, int i, int j,
 struct ForceRegion {
   int32_t ti0, ti1, tj0, tj1;  // inclusive tile ranges
   int32_t count;               // number of region tiles (>= 1)
-  int32_t error;               // nonzero: the body left the lattice
+  int32_t reserved;            // zero (part of the snapshots' layout)
 };
 
 // nodes of margin around a body for its force region; a moving body travels
@@ -682,11 +682,6 @@ __host__ __device__ inline ForceRegion make_region_box(const Lattice &L, double 
   const double m = kRegionMargin;
   int i0 = (int)floor(x0 - m), i1 = (int)ceil(x1 + m);
   int j0 = (int)floor(y0 - m), j1 = (int)ceil(y1 + m);
-  g.error = (i0 < -kRegionMargin || j0 < -kRegionMargin || i1 > L.nx - 1 + kRegionMargin ||
-             j1 > L.ny - 1 + kRegionMargin || !(x0 == x0) || !(y0 == y0) || !(x1 == x1) ||
-             !(y1 == y1))
-                ? 1
-                : 0;
   i0 = i0 < 0 ? 0 : (i0 > L.nx - 1 ? L.nx - 1 : i0);
   i1 = i1 < 0 ? 0 : (i1 > L.nx - 1 ? L.nx - 1 : i1);
   j0 = j0 < 0 ? 0 : (j0 > L.ny - 1 ? L.ny - 1 : j0);
