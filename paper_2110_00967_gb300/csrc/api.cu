@@ -513,6 +513,7 @@ constexpr int64_t kPairTiny = 400000, kPairSmall = 700000;
 // 768 x 384 FP16 4.80 / 4.89 / 5.30; 1024 x 512 FP32 (5 / 6 / 8) 5.3 / 4.9 / 5.8 and
 // FP16 6.0 / 5.7 / 6.7; 2048 x 1024 FP32 (6 / 8 / 10) 15.6 / 15.2 / 15.6, 3614 x 1946
 // (6 / 8 / 16) 45.4 / 44.9 / 46.3; five 2048 x 1024 (16 / 20 / 24) 12.91 / 12.76 / 12.78.
+// (The small lattices are 0.15 us faster since, by the force sums: warp_add.)
 int pair_rows(const vplbm_ctx *c) {
   if (c->bulk_variant > 0) return c->bulk_variant == 1 ? 12 : 24;
   if (!is_alone(c->mode)) return 20;
@@ -614,8 +615,8 @@ PairPlan pair_plan(const vplbm_ctx *c, const vplbm_body &b, const std::vector<Si
 // each, one 512 x 256 lattice 7.3 -> 3.9).  16-bit storage already reads half
 // as much and is bound by its arithmetic once the GPU is full, where the rim
 // that a pair recomputes costs what the traffic saves (the serving mix of
-// five sizes, FP16 stochastic: 6.5 us per lattice step singly, 6.6 in pairs with
-// long runs, 7.6 with short ones); alone and up to about 1.5 M nodes the GPU is
+// five sizes, FP16 stochastic: 6.0 us per lattice step singly, 6.1, 6.5 and 7.4 in
+// pairs with runs of 20, 28 and 40 rows); alone and up to about 1.5 M nodes the GPU is
 // not full, and half as many launches win (512 x 256: 9.7 -> 4.2 us, 1024 x 512:
 // 10.2 -> 5.7, 1536 x 768: 12.2 -> 9.8, 2048 x 1024: 16.5 -> 16.6).  Every lattice
 // adds its frame and box on top of its nodes, counted as 100,000 nodes: FP16

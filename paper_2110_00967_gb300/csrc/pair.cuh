@@ -31,10 +31,10 @@
 // it is bound by the FMA pipe (62 % busy) and one row prefetched in registers is
 // enough.  Measured, us per step and lattice, five 2048 x 1024 lattices in FP32:
 // 22.9 in single steps (0.97 of the copy rate), 14.0 with the next row held in
-// registers, 12.8 with the ring, 11.3 being the traffic of a pair at the copy
-// rate; rings of three and four rows 13.15 and 13.8 (shared memory taken from
-// L1), five blocks per SM instead of four (96 registers, spilled in the special
-// blocks) 13.15 against 13.06.
+// registers, 13.15 with a ring of three rows and 13.8 with one of four (shared
+// memory taken from L1), 13.06 with four blocks per SM (96 registers, which five
+// need, spill in the special blocks: 13.15), 12.8 with the warps numbered over the
+// whole grid (kPairWarps); 11.3 is the traffic of a pair at the copy rate.
 // ---------------------------------------------------------------------------
 template <typename S>
 struct Cell;  // a lane's two nodes of one plane in storage form

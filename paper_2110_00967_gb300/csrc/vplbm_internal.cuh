@@ -435,8 +435,9 @@ __device__ __forceinline__ bool body_contains(const BodyState &b, int i, int j) 
 // squared distance, with coordinates taken relative to the node below the
 // centre, has a relative error below 1e-6, and only nodes closer to the circle
 // than 1e-5 of r^2 need the FP64 form (none in most warps).  GB300 has two FP64
-// lanes per SM: evaluated everywhere in FP64, the mask of a moving disk took
-// 1.8 us of a step (12 us then, 9.2 now).
+// lanes per SM: with the mask in FP64 everywhere and the rigid update on one lane
+// a moving disk's step (400 x 1600, a pair of lattices) took 12.8 us, with this form
+// and the update on three lanes 10.4.
 struct NearTest {
   const BodyState &body;
   int i0, j0;
@@ -542,7 +543,7 @@ struct StepArgs {
   int32_t sim_order;     // 0: stress copied from the sampled node; 1: extrapolated linearly
   int32_t sim_blocks;    // leading blocks that evaluate SIM (0: SIM not due)
   int32_t sim_per_block; // SIM points per block (a multiple of 32)
-  double *hist;          // [hist_len][6]
+  double *hist;          // [hist_len][kHistCols]
   int32_t hist_len;
   double *sums;          // [6]
   long long *counts;     // [2]
