@@ -125,9 +125,9 @@ __global__ void __launch_bounds__(kAuxThreads)
                       double *ux_o, double *uy_o, int j0, int rows, long long ox, long long oy,
                       bool fixed) {
   using T = typename Store<S>::T;
-  const int i = blockIdx.x * kAuxThreads + threadIdx.x;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= L.nx) return;
-  for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+  for (int r = blockIdx.y * blockDim.y + threadIdx.y; r < rows; r += gridDim.y * blockDim.y) {
     const int j = j0 + r;
     const int64_t node = (int64_t)j * L.pitch + i, k = (int64_t)r * L.nx + i;
     T h[9];
@@ -238,16 +238,21 @@ cudaError_t get_fields_t(bool gather, const Lattice &L, const void *buf, const v
                          double *ux, double *uy, int j0, int rows, cudaStream_t s) {
   using T = typename Store<S>::T;
   const T *prev = static_cast<const T *>(prev_v);
-  const dim3 g((L.nx + kAuxThreads - 1) / kAuxThreads, rows < 65535 ? rows : 65535);
+  // 256 nodes of a row per block, or as many whole rows of a narrow lattice (one
+  // row each left most threads idle: 3 x 100000 in FP64 296 us, 17 x 40000 in FP32 134)
+  const int w = L.nx < kAuxThreads ? L.nx : kAuxThreads;
+  const dim3 b(w, kAuxThreads / w);
+  const int high = (rows + (int)b.y - 1) / (int)b.y;
+  const dim3 g((L.nx + w - 1) / w, high < 65535 ? high : 65535);
   const double unit = (double)(1ll << kFixBits);
   const double mx = L.ur[0] + 0.5 * L.bf[0], my = L.ur[1] + 0.5 * L.bf[1];
   const bool fixed = fabs(mx) < 4.0 && fabs(my) < 4.0;  // a body force may be larger
   const long long ox = fixed ? llrint(mx * unit) : 0, oy = fixed ? llrint(my * unit) : 0;
   if (gather)
-    get_fields_kernel<S, true><<<g, kAuxThreads, 0, s>>>(L, (const S *)buf, prev, chi, body,
+    get_fields_kernel<S, true><<<g, b, 0, s>>>(L, (const S *)buf, prev, chi, body,
                                                          half_pen, rho, ux, uy, j0, rows, ox, oy, fixed);
   else
-    get_fields_kernel<S, false><<<g, kAuxThreads, 0, s>>>(L, (const S *)buf, prev, chi, body,
+    get_fields_kernel<S, false><<<g, b, 0, s>>>(L, (const S *)buf, prev, chi, body,
                                                           half_pen, rho, ux, uy, j0, rows, ox, oy, fixed);
   return cudaGetLastError();
 }
