@@ -1050,8 +1050,10 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
   // histories, sums, counters, status
   VPLBM_CUDA(c, cudaMemsetAsync(c->ws + c->lay.hist, 0, c->lay.body[0] - c->lay.hist, s));
   VPLBM_CUDA(c, cudaMemsetAsync(c->ws + c->lay.sums, 0, c->lay.total - c->lay.sums, s));
-  c->rigid_host = moves(*b) ? rigid_const(c->body_host) : RigidConst{};
-  VPLBM_CUDA(c, cudaMemcpyAsync(c->rigid, &c->rigid_host, sizeof(RigidConst), cudaMemcpyHostToDevice, s));
+  if (moves(*b)) {  // (cleared with the counters above otherwise)
+    c->rigid_host = rigid_const(c->body_host);
+    VPLBM_CUDA(c, cudaMemcpyAsync(c->rigid, &c->rigid_host, sizeof(RigidConst), cudaMemcpyHostToDevice, s));
+  }
   VPLBM_CUDA(c, cudaMemsetAsync(c->prev[0], 0, 3 * (size_t)L.ny * sizeof(double), s));
   VPLBM_CUDA(c, cudaMemsetAsync(c->prev[1], 0, 3 * (size_t)L.ny * sizeof(double), s));
   VPLBM_CUDA(c, cudaGetLastError());
@@ -1108,8 +1110,8 @@ vplbm_status vplbm_prepare(vplbm_ctx *c, int32_t nsteps) {
   return sync(c);
 }
 
-// The forces of one estimator at `step` (column col of its history row) and the
-// latched status, with two copies into page-locked memory and one wait: copies
+// The forces of one estimator at `step` (column col of its history row) and (status
+// not NULL) the latched status, with two copies into page-locked memory and one wait: copies
 // into pageable memory wait for themselves, and a caller that reads both
 // estimates after every step spent 45 of 60 us in four copies and four waits.
 static vplbm_status read_forces(vplbm_ctx *c, long long step, int col, double F[2], double *T,
@@ -1118,13 +1120,14 @@ static vplbm_status read_forces(vplbm_ctx *c, long long step, int col, double F[
   const int len = effective_hist(c->cfg);
   VPLBM_CUDA(c, cudaMemcpyAsync(c->staging->row, c->hist + kHistCols * (step % len) + col,
                                 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  VPLBM_CUDA(c, cudaMemcpyAsync(&c->staging->status, c->status, sizeof(int32_t),
-                                cudaMemcpyDeviceToHost, c->stream));
+  if (status)
+    VPLBM_CUDA(c, cudaMemcpyAsync(&c->staging->status, c->status, sizeof(int32_t),
+                                  cudaMemcpyDeviceToHost, c->stream));
   if (vplbm_status st = sync(c)) return st;
   F[0] = c->staging->row[0];
   F[1] = c->staging->row[1];
   *T = c->staging->row[2];
-  *status = c->staging->status;
+  if (status) *status = c->staging->status;
   return VPLBM_OK;
 }
 
@@ -1158,8 +1161,7 @@ vplbm_status vplbm_force_angot(vplbm_ctx *c, double F[2], double *T) {
   if (!c) return fail(nullptr, VPLBM_EINVAL, "ctx is NULL");
   if (!F || !T) return fail(c, VPLBM_EINVAL, "NULL output");
   if (c->steps == 0) return fail(c, VPLBM_ESTATE, "no step taken");
-  int32_t status = 0;
-  return read_forces(c, c->steps - 1, 6, F, T, &status);
+  return read_forces(c, c->steps - 1, 6, F, T, nullptr);
 }
 
 vplbm_status vplbm_forces_async(vplbm_ctx *c, double *out) {
