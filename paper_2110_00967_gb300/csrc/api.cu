@@ -234,6 +234,11 @@ bool finite_place(const vplbm_body &b) {
          (b.kind != VPLBM_BODY_NACA4 || std::isfinite(b.angle));
 }
 
+// The polygon lies inside the lattice.
+bool fits(const Extent &e, const Lattice &L) {
+  return e.x0 >= 0.0 && e.y0 >= 0.0 && e.x1 <= L.nx - 1.0 && e.y1 <= L.ny - 1.0;
+}
+
 // an empty lattice has nothing to move, whatever the flag says
 bool moves(const vplbm_body &b) { return b.kind != VPLBM_BODY_NONE && b.moving != 0; }
 
@@ -612,7 +617,7 @@ PairPlan pair_plan(const vplbm_ctx *c, const vplbm_body &b, const std::vector<Si
 // Chooses how the lattices of a call step, from the nodes that the call steps
 // side by side.  FP32 steps in pairs wherever it can: it is bound by HBM, and a
 // pair halves the traffic (five 2048 x 1024 lattices 22.9 -> 12.8 us per step
-// each, one 512 x 256 lattice 7.3 -> 3.9).  16-bit storage already reads half
+// each, one 512 x 256 lattice 7.3 -> 3.7).  16-bit storage already reads half
 // as much and is bound by its arithmetic once the GPU is full, where the rim
 // that a pair recomputes costs what the traffic saves (the serving mix of
 // five sizes, FP16 stochastic: 6.0 us per lattice step singly, 6.1, 6.5 and 7.4 in
@@ -967,9 +972,8 @@ vplbm_status vplbm_set_body(vplbm_ctx *c, const vplbm_body *b) {
     if (n_sim > effective_max_sim(c->cfg))
       return fail(c, VPLBM_EINVAL, fmt("%d SIM points exceed the capacity %d", n_sim, effective_max_sim(c->cfg)));
     if (!build_polygon(*b, n_sim, pts)) return fail(c, VPLBM_EINVAL, "bad SIM point count for this body");
-    // the body's polygon must lie inside the lattice
     box = extent_of(*b, pts);
-    if (!(box.x0 >= 0.0 && box.y0 >= 0.0 && box.x1 <= L.nx - 1.0 && box.y1 <= L.ny - 1.0))
+    if (!fits(box, L))
       return fail(c, VPLBM_EINVAL, "body does not fit in the lattice");
   }
   // force region: tiles around the body; tile (0, 0) alone for an empty lattice
@@ -1111,9 +1115,9 @@ vplbm_status vplbm_prepare(vplbm_ctx *c, int32_t nsteps) {
 }
 
 // The forces of one estimator at `step` (column col of its history row) and (status
-// not NULL) the latched status, with two copies into page-locked memory and one wait: copies
-// into pageable memory wait for themselves, and a caller that reads both
-// estimates after every step spent 45 of 60 us in four copies and four waits.
+// not NULL) the latched status, with two copies into page-locked memory and one
+// wait: copies into pageable memory wait for themselves, and a caller that reads
+// both estimates after every step spent 45 of 60 us in four copies and four waits.
 static vplbm_status read_forces(vplbm_ctx *c, long long step, int col, double F[2], double *T,
                                 int32_t *status) {
   const std::lock_guard<std::mutex> hold(c->staging_lock);
@@ -1486,7 +1490,8 @@ vplbm_status vplbm_load_state(vplbm_ctx *c, const void *host, size_t bytes) {
   // everything that can be refused is looked at before the lattice is touched
   std::vector<SimPoint> pts;
   if (h.body_cfg.kind != VPLBM_BODY_NONE &&
-      (!finite_place(h.body_cfg) || !build_polygon(h.body_cfg, h.n_sim, pts)))
+      (!finite_place(h.body_cfg) || !build_polygon(h.body_cfg, h.n_sim, pts) ||
+       !fits(extent_of(h.body_cfg, pts), c->L)))
     return fail(c, VPLBM_EINVAL, "corrupt snapshot body");
   const PairPlan plan = pair_plan(c, h.body_cfg, pts);
   const char *in = static_cast<const char *>(host);

@@ -41,6 +41,23 @@ def test_a_body_at_no_finite_place_is_refused(field, value):
     np.testing.assert_array_equal(lat.history(V.MEM, 7), twin.history(V.MEM, 7))
 
 
+@pytest.mark.parametrize("field,value", [("x_c", 5.0), ("y_c", 1e9), ("length", 1e9), ("length", 600.0)])
+def test_a_snapshot_of_a_body_beyond_the_lattice_is_refused(field, value):
+    """No such body can have been placed: EINVAL, and the lattice goes on as it was."""
+    w = W.naca(5.0, dtype="f32", nx=512, ny=256)
+    lat, twin = lattice(w), lattice(w)
+    lat.step(3)
+    snap = lat.save_state()
+    at = 16 + ctypes.sizeof(V.vplbm_config) + getattr(V.vplbm_body, field).offset
+    snap[at:at + 8].view(np.float64)[0] = value
+    with pytest.raises(V.VplbmError) as e:
+        lat.load_state(snap)
+    assert e.value.status == V.EINVAL
+    lat.step(4)
+    twin.step(7)
+    np.testing.assert_array_equal(lat.get_f(), twin.get_f())
+
+
 @pytest.mark.parametrize("dtype", ["f64", "f32", "f16"])
 @pytest.mark.parametrize("length", [0.0, 20.0])
 def test_an_empty_lattice_has_nothing_to_move(dtype, length):
