@@ -74,7 +74,7 @@ def config_block(dtype: str = "f32", extra=None):
          "storage": "f32" if dtype == "f32" else f"{dtype} offsets from feq(1, u_in)",
          "forces_per_step": ["mem", "sim-849"],
          "l2": f"inputs larger than L2: 5 lattices x {mb} MB ping-pong, stepped side by side"
-               + (" (ncu range replay: DRAM traffic 80.2 MB per lattice step, 75.5 algorithmic at two steps per pass)"
+               + (" (ncu range replay: DRAM traffic 78.6 MB per lattice step, 75.5 algorithmic at two steps per pass)"
                   if dtype == "f32" else "")}
     if extra:
         c.update(extra)
